@@ -233,6 +233,46 @@ __global__ void k_scan_sums(int* sums, int nblocks, int* total)
     if (threadIdx.x == 0) *total = carry;
 }
 
+// the whole scan by one block, for up to kScanOne entries: one launch instead of three (a small
+// catalog's call is a chain of launches)
+constexpr int kScanOne = 16384;
+
+__global__ void __launch_bounds__(1024) k_scan_one(const int* __restrict__ in, int* __restrict__ out, int K)
+{
+    __shared__ int wsum[32];
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    const int per = (K + 1023) / 1024, i0 = min(t * per, K), i1 = min(i0 + per, K);
+    int v[kScanOne / 1024], run = 0;
+#pragma unroll
+    for (int q = 0; q < kScanOne / 1024; ++q) {
+        v[q] = i0 + q < i1 ? in[i0 + q] : 0;
+        run += v[q];
+    }
+    int x = run;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[wid] = x;
+    __syncthreads();
+    if (wid == 0) {
+        int s = wsum[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, s, o);
+            if (lane >= o) s += y;
+        }
+        wsum[lane] = s;
+    }
+    __syncthreads();
+    int excl = x - run + (wid > 0 ? wsum[wid - 1] : 0);
+#pragma unroll
+    for (int q = 0; q < kScanOne / 1024; ++q) {
+        if (i0 + q < i1) out[i0 + q] = excl;
+        excl += v[q];
+    }
+    if (t == 1023) out[K] = excl;
+}
+
 __global__ void k_scan_add(int* __restrict__ out, int64_t K, const int* __restrict__ sums)
 {
     const int64_t base = (int64_t)blockIdx.x * kScanBlock;
@@ -278,7 +318,8 @@ __global__ void k_gather(int64_t n, const int* __restrict__ perm, const int32_t*
                          const float* __restrict__ g2, const float* __restrict__ w,
                          const uint8_t* __restrict__ zb, const uint8_t* __restrict__ mask,
                          int2* __restrict__ pos, Pay<T>* __restrict__ pay,
-                         uint8_t* __restrict__ zs, int* __restrict__ cflag, int nz)
+                         uint8_t* __restrict__ zs, int* __restrict__ cflag, int nz, int* __restrict__ centre_idx,
+                         int* __restrict__ crow)
 {
     for (int64_t d = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; d < n;
          d += (int64_t)gridDim.x * blockDim.x) {
@@ -287,7 +328,12 @@ __global__ void k_gather(int64_t n, const int* __restrict__ perm, const int32_t*
         const T wi = (T)w[i];
         pay[d] = Pay<T>{wi * (T)g1[i], wi * (T)g2[i], wi, T(0)};
         zs[d] = zb ? (uint8_t)min((int)zb[i], nz - 1) : 0;  // clamped like the cell key (k_keys)
-        cflag[d] = mask ? (mask[i] != 0) : 1;
+        if (mask) {
+            cflag[d] = mask[i] != 0;
+        } else {  // every galaxy is a centre
+            centre_idx[d] = (int)d;
+            crow[d] = i;
+        }
     }
 }
 
@@ -303,7 +349,10 @@ __global__ void k_mask_flags(int64_t n, const uint8_t* __restrict__ mask, int* _
 __global__ void k_zrange(int nz, int64_t ncells, const int* __restrict__ cell_start, const int* __restrict__ crank,
                          int* __restrict__ zrange)
 {
-    for (int z = threadIdx.x; z <= nz; z += blockDim.x) zrange[z] = crank[cell_start[(int64_t)z * ncells]];
+    for (int z = threadIdx.x; z <= nz; z += blockDim.x) {
+        const int d = cell_start[(int64_t)z * ncells];
+        zrange[z] = crank ? crank[d] : d;
+    }
 }
 
 // centre list in sorted order and, for each centre, its row in galaxy-index order
@@ -590,6 +639,12 @@ const char* mp3pcf_last_error(const mp3pcf_ctx* ctx)
 // exclusive scan of K ints from `in` to `out` (out has K+1 entries; out[K] = total)
 static mp3pcf_status scan_exclusive(mp3pcf_ctx* ctx, const int* in, int* out, int64_t K)
 {
+    if (K <= kScanOne) {
+        ctx->launches[ST_SORT] += 1;
+        k_scan_one<<<1, 1024, 0, ctx->st>>>(in, out, (int)K);
+        MP3_CK(cudaGetLastError());
+        return MP3PCF_OK;
+    }
     const int64_t nblk = (K + kScanBlock - 1) / kScanBlock;
     ctx->launches[ST_SORT] += nblk > 0 ? 3 : 1;
     MP3_CK(ctx->scan_sums.ensure(sizeof(int) * (nblk + 1)));
@@ -689,14 +744,16 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
     MP3_CK(ctx->pos.ensure(sizeof(int2) * n));
     MP3_CK(ctx->pay.ensure(sizeof(Pay<T>) * n));
     MP3_CK(ctx->zs.ensure(n));
-    MP3_CK(ctx->cflag.ensure(sizeof(int) * (n + 1)));
-    MP3_CK(ctx->crank.ensure(sizeof(int) * (n + 1)));
-    MP3_CK(ctx->oflag.ensure(sizeof(int) * (n + 1)));
-    MP3_CK(ctx->orank.ensure(sizeof(int) * (n + 1)));
+    if (mask) {
+        MP3_CK(ctx->cflag.ensure(sizeof(int) * (n + 1)));
+        MP3_CK(ctx->crank.ensure(sizeof(int) * (n + 1)));
+        MP3_CK(ctx->oflag.ensure(sizeof(int) * (n + 1)));
+        MP3_CK(ctx->orank.ensure(sizeof(int) * (n + 1)));
+    }
     MP3_CK(ctx->centre_idx.ensure(sizeof(int) * n));
     MP3_CK(ctx->crow.ensure(sizeof(int) * n));
     MP3_CK(cudaMemsetAsync(ctx->fill.p, 0, sizeof(int) * (K + 1), st));
-    ctx->launches[ST_SORT] += 6;
+    ctx->launches[ST_SORT] += 4;
     k_keys<<<grid1d(n, ctx->n_sm), 256, 0, st>>>(n, xq, yq, zb, nz, g, ctx->key.as<int>(), ctx->fill.as<int>());
     MP3_CK(cudaGetLastError());
     if (mp3pcf_status s = scan_exclusive(ctx, ctx->fill.as<int>(), ctx->count.as<int>(), K)) return s;
@@ -706,20 +763,25 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
     k_cell_order<<<grid1d(K, ctx->n_sm), 256, 0, st>>>(K, ctx->count.as<int>(), ctx->perm.as<int>());
     k_gather<T><<<grid1d(n, ctx->n_sm), 256, 0, st>>>(
         n, ctx->perm.as<int>(), xq, yq, g1, g2, w, zb, mask, ctx->pos.as<int2>(), ctx->pay.as<Pay<T>>(),
-        ctx->zs.as<uint8_t>(), ctx->cflag.as<int>(), nz);
+        ctx->zs.as<uint8_t>(), ctx->cflag.as<int>(), nz, ctx->centre_idx.as<int>(), ctx->crow.as<int>());
     MP3_CK(cudaGetLastError());
 
-    // ---- centre list (sorted order) and each centre's row in galaxy-index order
-    if (mp3pcf_status s = scan_exclusive(ctx, ctx->cflag.as<int>(), ctx->crank.as<int>(), n)) return s;
-    k_mask_flags<<<grid1d(n, ctx->n_sm), 256, 0, st>>>(n, mask, ctx->oflag.as<int>());
-    if (mp3pcf_status s = scan_exclusive(ctx, ctx->oflag.as<int>(), ctx->orank.as<int>(), n)) return s;
-    k_centres<<<grid1d(n, ctx->n_sm), 256, 0, st>>>(n, ctx->perm.as<int>(), ctx->cflag.as<int>(),
-                                                    ctx->crank.as<int>(), ctx->orank.as<int>(),
-                                                    ctx->centre_idx.as<int>(), ctx->crow.as<int>());
-    MP3_CK(cudaGetLastError());
+    // ---- centre list (sorted order) and each centre's row in galaxy-index order; without a mask
+    // k_gather has written them (every galaxy in sorted order)
+    if (mask) {
+        if (mp3pcf_status s = scan_exclusive(ctx, ctx->cflag.as<int>(), ctx->crank.as<int>(), n)) return s;
+        k_mask_flags<<<grid1d(n, ctx->n_sm), 256, 0, st>>>(n, mask, ctx->oflag.as<int>());
+        if (mp3pcf_status s = scan_exclusive(ctx, ctx->oflag.as<int>(), ctx->orank.as<int>(), n)) return s;
+        k_centres<<<grid1d(n, ctx->n_sm), 256, 0, st>>>(n, ctx->perm.as<int>(), ctx->cflag.as<int>(),
+                                                        ctx->crank.as<int>(), ctx->orank.as<int>(),
+                                                        ctx->centre_idx.as<int>(), ctx->crow.as<int>());
+        MP3_CK(cudaGetLastError());
+        ctx->launches[ST_SORT] += 2;
+    }
     if (nz > 1) {
         MP3_CK(ctx->zrange.ensure(sizeof(int) * (nz + 1)));
-        k_zrange<<<1, 32, 0, st>>>(nz, g.ncells, ctx->count.as<int>(), ctx->crank.as<int>(), ctx->zrange.as<int>());
+        k_zrange<<<1, 32, 0, st>>>(nz, g.ncells, ctx->count.as<int>(), mask ? ctx->crank.as<int>() : nullptr,
+                                    ctx->zrange.as<int>());
         MP3_CK(cudaGetLastError());
         ctx->launches[ST_SORT] += 1;
     }
