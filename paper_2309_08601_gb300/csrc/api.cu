@@ -16,6 +16,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "common.cuh"
+#include "moments_far.cuh"
 
 namespace mp3 {
 
@@ -96,41 +97,54 @@ __global__ void k_or_word(const unsigned long long* __restrict__ src, unsigned l
     if (threadIdx.x == 0 && blockIdx.x == 0) *dst |= *src;
 }
 
+// extent of the catalog (bb[0..3]: min x, min y, max x, max y), bad z-bins (bb[4]), and with a mask
+// the extent and number of the centres (bb[5..8], bb[9])
 __global__ void k_bbox_init(int* bb)
 {
-    bb[0] = INT_MAX;
-    bb[1] = INT_MAX;
-    bb[2] = INT_MIN;
-    bb[3] = INT_MIN;
-    bb[4] = 0;  // error flags
+    const int v[10] = {INT_MAX, INT_MAX, INT_MIN, INT_MIN, 0, INT_MAX, INT_MAX, INT_MIN, INT_MIN, 0};
+    if (threadIdx.x < 10) bb[threadIdx.x] = v[threadIdx.x];
 }
 
 __global__ void k_bbox(int64_t n, const int32_t* __restrict__ xq, const int32_t* __restrict__ yq,
-                       const uint8_t* __restrict__ zb, int nz, int* bb)
+                       const uint8_t* __restrict__ zb, const uint8_t* __restrict__ mask, int nz, int* bb)
 {
-    int mnx = INT_MAX, mny = INT_MAX, mxx = INT_MIN, mxy = INT_MIN, bad = 0;
+    int v[10] = {INT_MAX, INT_MAX, INT_MIN, INT_MIN, 0, INT_MAX, INT_MAX, INT_MIN, INT_MIN, 0};
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int x = xq[i], y = yq[i];
-        mnx = min(mnx, x);
-        mny = min(mny, y);
-        mxx = max(mxx, x);
-        mxy = max(mxy, y);
-        if (zb && zb[i] >= nz) bad = 1;
+        v[0] = min(v[0], x);
+        v[1] = min(v[1], y);
+        v[2] = max(v[2], x);
+        v[3] = max(v[3], y);
+        if (zb && zb[i] >= nz) v[4] = 1;
+        if (mask && mask[i]) {
+            v[5] = min(v[5], x);
+            v[6] = min(v[6], y);
+            v[7] = max(v[7], x);
+            v[8] = max(v[8], y);
+            v[9] += 1;
+        }
     }
     for (int o = 16; o > 0; o >>= 1) {
-        mnx = min(mnx, __shfl_xor_sync(0xffffffffu, mnx, o));
-        mny = min(mny, __shfl_xor_sync(0xffffffffu, mny, o));
-        mxx = max(mxx, __shfl_xor_sync(0xffffffffu, mxx, o));
-        mxy = max(mxy, __shfl_xor_sync(0xffffffffu, mxy, o));
-        bad |= __shfl_xor_sync(0xffffffffu, bad, o);
+#pragma unroll
+        for (int q = 0; q < 10; q += 5) {
+            v[q] = min(v[q], __shfl_xor_sync(0xffffffffu, v[q], o));
+            v[q + 1] = min(v[q + 1], __shfl_xor_sync(0xffffffffu, v[q + 1], o));
+            v[q + 2] = max(v[q + 2], __shfl_xor_sync(0xffffffffu, v[q + 2], o));
+            v[q + 3] = max(v[q + 3], __shfl_xor_sync(0xffffffffu, v[q + 3], o));
+        }
+        v[4] |= __shfl_xor_sync(0xffffffffu, v[4], o);
+        v[9] += __shfl_xor_sync(0xffffffffu, v[9], o);
     }
     if ((threadIdx.x & 31) == 0) {
-        atomicMin(&bb[0], mnx);
-        atomicMin(&bb[1], mny);
-        atomicMax(&bb[2], mxx);
-        atomicMax(&bb[3], mxy);
-        if (bad) atomicOr(&bb[4], 1);
+        for (int q = 0; q < (mask ? 10 : 5); q += 5) {
+            atomicMin(&bb[q], v[q]);
+            atomicMin(&bb[q + 1], v[q + 1]);
+            atomicMax(&bb[q + 2], v[q + 2]);
+            atomicMax(&bb[q + 3], v[q + 3]);
+        }
+        if (v[4]) atomicOr(&bb[4], 1);
+        if (v[9]) atomicAdd(&bb[9], v[9]);
     }
 }
 
@@ -318,13 +332,15 @@ __global__ void k_gather(int64_t n, const int* __restrict__ perm, const int32_t*
                          const float* __restrict__ g2, const float* __restrict__ w,
                          const uint8_t* __restrict__ zb, const uint8_t* __restrict__ mask,
                          int2* __restrict__ pos, Pay<T>* __restrict__ pay,
-                         uint8_t* __restrict__ zs, int* __restrict__ cflag, int nz, int* __restrict__ centre_idx,
-                         int* __restrict__ crow)
+                         uint8_t* __restrict__ zs, int* __restrict__ cflag, int nz, float2* __restrict__ posf,
+                         long long x0, long long y0, int* __restrict__ centre_idx, int* __restrict__ crow)
 {
     for (int64_t d = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; d < n;
          d += (int64_t)gridDim.x * blockDim.x) {
         const int i = perm[d];
         pos[d] = make_int2(xq[i], yq[i]);
+        // positions from the grid's origin are below 2^24 and so exact in FP32
+        posf[d] = make_float2((float)((long long)xq[i] - x0), (float)((long long)yq[i] - y0));
         const T wi = (T)w[i];
         pay[d] = Pay<T>{wi * (T)g1[i], wi * (T)g2[i], wi, T(0)};
         zs[d] = zb ? (uint8_t)min((int)zb[i], nz - 1) : 0;  // clamped like the cell key (k_keys)
@@ -367,6 +383,20 @@ __global__ void k_centres(int64_t n, const int* __restrict__ perm, const int* __
             centre_idx[r] = (int)d;
             crow[r] = orank[perm[d]];
         }
+    }
+}
+
+// strip-order bucket of every centre: strips of strip_rows cell rows, columns within a strip
+__global__ void k_strip_keys(int nc, const int* __restrict__ centre_idx, const int2* __restrict__ pos, GridDesc g,
+                             int strip_rows, int* __restrict__ key, int* __restrict__ count)
+{
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += gridDim.x * blockDim.x) {
+        const int2 p = pos[centre_idx[c]];
+        const int cx_ = (int)min(max(0LL, (long long)p.x - g.x0) / g.side, (long long)g.ncx - 1);
+        const int cy_ = (int)min(max(0LL, (long long)p.y - g.y0) / g.side, (long long)g.ncy - 1);
+        const int k = cy_ / strip_rows * g.ncx + cx_;
+        key[c] = k;
+        atomicAdd(&count[k], 1);
     }
 }
 
@@ -425,6 +455,9 @@ struct mp3pcf_ctx {
     DevBuf degen;                       // exclude_degenerate sums per (centre, z, bin)
     DevBuf degen_grad;                  // their gradient sums per (Z1, z, bin) in the adjoint
     DevBuf zrange;                      // [nz + 1] centre range of each z-bin
+    // wide bins by angular sectors (moments_far.cu): tables, FP32 positions, centres in strip order
+    FarTables far[kFarPlans];
+    DevBuf bingeom, ftable, posf, fkey, fstart, ffill, forder;
     DevBuf fftwork;                     // FFT grid moments: padded fields, kernels, products
     FftPlanCache* fft = nullptr;        // cuFFT plans of the FFT grid moments
     DevBuf gridsum;                     // per-pixel FP64 sums of the grid-based approximation
@@ -591,13 +624,22 @@ mp3pcf_status mp3pcf_create(const mp3pcf_config* cfg, void* stream, mp3pcf_ctx**
     if (ctx->d_e2q.ensure(sizeof(long long) * (nb + 1)) != cudaSuccess ||
         ctx->d_edges.ensure(sizeof(double) * (nb + 1)) != cudaSuccess ||
         ctx->d_nodes.ensure(sizeof(double) * nb) != cudaSuccess ||
-        ctx->bb.ensure(sizeof(int) * 8) != cudaSuccess || ctx->pairs.ensure(24) != cudaSuccess ||
+        ctx->bingeom.ensure(sizeof(BinGeom) * nb) != cudaSuccess ||
+        ctx->bb.ensure(sizeof(int) * 10) != cudaSuccess || ctx->pairs.ensure(8 * (4 + kFarPlans)) != cudaSuccess ||
         ctx->singular.ensure(8) != cudaSuccess)
         return cleanup(MP3PCF_ENOMEM);
     if (cudaMemcpy(ctx->d_e2q.p, ctx->e2q.data(), sizeof(long long) * (nb + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(ctx->d_edges.p, ctx->edges.data(), sizeof(double) * (nb + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(ctx->bingeom.p, bin_geometry(ctx->e2q).data(), sizeof(BinGeom) * nb, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(ctx->d_nodes.p, ctx->nodes.data(), sizeof(double) * nb, cudaMemcpyHostToDevice) != cudaSuccess)
         return cleanup(MP3PCF_ECUDA);
+    if (!ctx->fp64) {
+        std::vector<float> v;
+        far_tables(cfg->n_max, ctx->far, &v);
+        if (ctx->ftable.ensure(sizeof(float) * v.size()) != cudaSuccess) return cleanup(MP3PCF_ENOMEM);
+        if (cudaMemcpy(ctx->ftable.p, v.data(), sizeof(float) * v.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+            return cleanup(MP3PCF_ECUDA);
+    }
     *out = ctx;
     return MP3PCF_OK;
 }
@@ -612,7 +654,7 @@ mp3pcf_status mp3pcf_destroy(mp3pcf_ctx* ctx)
                       &ctx->crank, &ctx->oflag, &ctx->orank, &ctx->centre_idx, &ctx->crow,
                       &ctx->G, &ctx->W, &ctx->pairs, &ctx->partial, &ctx->singular,
                       &ctx->m3partial, &ctx->m3four, &ctx->fftwork, &ctx->ccoef, &ctx->gG, &ctx->gW, &ctx->gv, &ctx->gtab,
-                      &ctx->adjscratch, &ctx->degen, &ctx->degen_grad, &ctx->zrange, &ctx->gridsum, &ctx->gridflag, &ctx->bups, &ctx->bnorm,
+                      &ctx->adjscratch, &ctx->degen, &ctx->degen_grad, &ctx->zrange, &ctx->bingeom, &ctx->ftable, &ctx->posf, &ctx->fkey, &ctx->fstart, &ctx->ffill, &ctx->forder, &ctx->gridsum, &ctx->gridflag, &ctx->bups, &ctx->bnorm,
                       &ctx->bgam, &ctx->bgcen, &ctx->berr, &ctx->pix, &ctx->pixinv};
     for (DevBuf* b : bufs) b->release();
     if (ctx->fft) fft_cache_destroy(ctx->fft);
@@ -669,6 +711,112 @@ static unsigned grid1d(int64_t n, int n_sm)
     return (unsigned)(g < 1 ? 1 : g);
 }
 
+// The sector form of the moments (moments_far.cu) for the bins [b_far, b_hi): groups of kFarGroup
+// centres in strips of `rows` cell rows and at most `cols` columns, on cells of side `side`.
+struct FarPlan {
+    int b_far = 0, rows = 1, cols = 1;
+    int b[kFarPlans + 1] = {0};  // bins [b[v + 1], b[v]) take variant v (b[0] = b_hi)
+    double side = 1.0;
+};
+
+// Expected neighbours of a (centre, bin) below which the warp-per-centre form (moments_near.cu) is
+// faster than the block-per-centre form: about 300 + (5 + 6 SW + 4 SAB) N warp instructions a bin
+// against 300 n_max + n_max N / 2 (lines measured at n_max 10, 20 and 30 in FP32; in FP64, where a
+// warp-wide instruction takes 16 cycles, the line lies lower).
+static double near_line(int n_max, bool fp64) { return fp64 ? 100.0 : std::max(60.0, 24.0 * n_max); }
+
+// estimated warp instructions of a (centre, bin) with N neighbours, by the cheaper of those two forms
+static double small_cost(int n_max, double N)
+{
+    const int sw = std::max(2 * n_max, n_max + 3) / 32 + 1, sab = (n_max + 3) / 32 + 1;
+    return std::min(300.0 + (5 + 6 * sw + 4 * sab) * N, 300.0 * n_max + 0.5 * n_max * N);
+}
+
+static FarPlan plan_far(const mp3pcf_ctx* ctx, int64_t n, int64_t nc, double area, double carea, int b_lo, int b_hi)
+{
+    const mp3pcf_config& c = ctx->cfg;
+    FarPlan f;
+    f.b_far = b_hi;
+    if (nc < 1 || n >= (1 << 27)) return f;  // 32-bit byte offsets into the sorted catalog
+    const double rho = (double)n / c.n_z / area;  // galaxies per quantum^2 and z-bin
+    const double occ = c.cell_occupancy > 0 ? (double)c.cell_occupancy : 1.0;
+    f.side = std::max(1.0, std::max(sqrt(occ / rho), sqrt(area * c.n_z / (double)(1 << 26))));
+    const double per_cell = (double)nc / carea * f.side * f.side;  // centres
+    f.rows = (int)std::min(4.0, std::max(1.0, floor(sqrt(8.0 / per_cell) + 0.5)));
+    f.cols = (int)std::min(5.0, ceil(8.0 / (per_cell * f.rows)) + 1.0);
+    // sparse centres would leave most lanes of a group empty
+    if (per_cell * f.rows * f.cols < 4.0) return f;
+    // the direction from a centre to a galaxy differs from the sector's axis by at most half a
+    // sector plus the angle the cell's and the group's extents subtend
+    const double reach = f.side * (0.7072 + 0.5 * sqrt((double)f.rows * f.rows + (double)f.cols * f.cols)) + 8.0;
+    int b = b_hi;
+    f.b[0] = b_hi;
+    for (int v = 0; v < kFarPlans; ++v) {
+        const FarTables& t = ctx->far[v];
+        const double r_min = t.dmax > t.half_width ? reach / sin(t.dmax - t.half_width) : 1e300;
+        while (b > b_lo && (double)ctx->e2q[b - 1] >= r_min * r_min) {
+            // per centre: the sectors' enumeration and reduction, the FFT and orders, the pairs
+            const double N = M_PI * rho * (double)(ctx->e2q[b] - ctx->e2q[b - 1]);
+            const double cost = 75.0 * t.sectors + 0.35 * t.terms * t.sectors + N * (1.25 * t.terms + 30.0) / 24.0;
+            if (cost >= small_cost(c.n_max, N)) break;
+            --b;
+        }
+        f.b[v + 1] = b;
+    }
+    f.b_far = b;
+    return f;
+}
+
+static mp3pcf_status run_far(mp3pcf_ctx* ctx, const MomentArgs<float>& a, const FarPlan& fp, int b_lo, int b_hi)
+{
+    cudaStream_t st = ctx->st;
+    const int nc = a.n_centres;
+    const int64_t K = (int64_t)((a.g.ncy + fp.rows - 1) / fp.rows) * a.g.ncx;
+    MP3_CK(ctx->fkey.ensure(sizeof(int) * nc));
+    MP3_CK(ctx->fstart.ensure(sizeof(int) * (K + 1)));
+    MP3_CK(ctx->ffill.ensure(sizeof(int) * (K + 1)));
+    MP3_CK(ctx->forder.ensure(sizeof(int) * nc));
+    int* fill = ctx->ffill.as<int>();
+    MP3_CK(cudaMemsetAsync(fill, 0, sizeof(int) * (K + 1), st));
+    k_strip_keys<<<grid1d(nc, ctx->n_sm), 256, 0, st>>>(nc, a.centre_idx, a.pos, a.g, fp.rows, ctx->fkey.as<int>(), fill);
+    MP3_CK(cudaGetLastError());
+    if (mp3pcf_status s = scan_exclusive(ctx, fill, ctx->fstart.as<int>(), K)) return s;
+    MP3_CK(cudaMemsetAsync(fill, 0, sizeof(int) * (K + 1), st));
+    k_scatter<<<grid1d(nc, ctx->n_sm), 256, 0, st>>>(nc, ctx->fkey.as<int>(), ctx->fstart.as<int>(), fill,
+                                                     ctx->forder.as<int>());
+    k_cell_order<<<grid1d(K, ctx->n_sm), 256, 0, st>>>(K, ctx->fstart.as<int>(), ctx->forder.as<int>());
+    MP3_CK(cudaGetLastError());
+    ctx->launches[ST_MOMENTS] += 3;
+    const int groups = (nc + 7) / 8;
+    for (int v = 0; v < kFarPlans; ++v) {
+        const int b0 = fp.b[v + 1], nbv = fp.b[v] - b0;
+        if (nbv < 1) continue;
+        FarArgs f;
+        f.m = a;
+        f.m.nb = nbv;
+        f.m.e2q = a.e2q + (b0 - b_lo);
+        f.m.G = a.G + (b0 - b_lo);
+        f.m.W = a.W + (b0 - b_lo);
+        f.bins = ctx->bingeom.as<BinGeom>() + b0;
+        f.posf = ctx->posf.as<float2>();
+        f.order = ctx->forder.as<int>();
+        f.strip_rows = fp.rows;
+        f.max_cols = fp.cols;
+        // about six items per resident block, so that the last ones end together
+        f.parts = std::max(1, std::min(nbv * a.nz, (ctx->n_sm * 12 + groups - 1) / groups));
+        f.table = ctx->ftable.as<float>();
+        f.off_ray = ctx->far[v].off_ray;
+        f.off_sin = ctx->far[v].off_sin;
+        f.off_axis = ctx->far[v].off_axis;
+        f.off_rot = ctx->far[v].off_rot;
+        f.off_coef = ctx->far[v].off_coef;
+        f.queue = ctx->pairs.as<unsigned long long>() + 3 + v;
+        ctx->launches[ST_MOMENTS] += 1;
+        MP3_CK(launch_moments_far(f, v, ctx->n_sm, st));
+    }
+    return MP3PCF_OK;
+}
+
 template <typename T>
 static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq, const int32_t* yq,
                                   const float* g1, const float* g2, const float* w,
@@ -680,7 +828,7 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
     ctx->n = n;
     ctx->n_centres = 0;
     ctx->combined = false;
-    MP3_CK(cudaMemsetAsync(ctx->pairs.p, 0, 24, st));
+    MP3_CK(cudaMemsetAsync(ctx->pairs.p, 0, 8 * (4 + kFarPlans), st));
     if (n == 0) return MP3PCF_OK;
     if (ctx->inject_alloc_failure) return fail(ctx, MP3PCF_ENOMEM, "injected allocation failure");
 
@@ -689,6 +837,7 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
     NvtxRange nvtx_acc("mp3pcf accumulate_moments");
     cudaEvent_t t_sort = stage_begin(ctx);
     long long bb[5];
+    int hb[10] = {0};
     if (ctx->fixed_extent) {
         for (int i = 0; i < 4; ++i) bb[i] = ctx->ext[i];
         bb[4] = 0;
@@ -696,15 +845,16 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
         k_validate<<<grid1d(n, ctx->n_sm), 256, 0, st>>>(n, xq, yq, zb, nz, bb[0], bb[1], bb[2], bb[3],
                                                           ctx->pairs.as<unsigned long long>() + 1);
         MP3_CK(cudaGetLastError());
-    } else {
+    }
+    if (!ctx->fixed_extent || mask) {
         ctx->launches[ST_SORT] += 2;
-        k_bbox_init<<<1, 1, 0, st>>>(ctx->bb.as<int>());
-        k_bbox<<<grid1d(n, ctx->n_sm), 256, 0, st>>>(n, xq, yq, zb, nz, ctx->bb.as<int>());
+        k_bbox_init<<<1, 32, 0, st>>>(ctx->bb.as<int>());
+        k_bbox<<<grid1d(n, ctx->n_sm), 256, 0, st>>>(n, xq, yq, zb, mask, nz, ctx->bb.as<int>());
         MP3_CK(cudaGetLastError());
-        int hb[5];
         MP3_CK(cudaMemcpyAsync(hb, ctx->bb.p, sizeof(hb), cudaMemcpyDeviceToHost, st));
         MP3_CK(cudaStreamSynchronize(st));
-        for (int i = 0; i < 5; ++i) bb[i] = hb[i];
+        if (!ctx->fixed_extent)
+            for (int i = 0; i < 5; ++i) bb[i] = hb[i];
     }
     if (bb[4]) {
         stage_end(ctx, ST_SORT, t_sort);
@@ -718,11 +868,23 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
     }
 
     // ---- cell grid: ~4 galaxies per cell and bin, and at most kMaxRows rows per annulus of the
-    // computed bins
-    const double R = sqrt((double)ctx->e2q[b_hi]);
+    // bins of the direct form; the sector form takes bins [b_far, b_hi) (plan_far)
+    const int64_t nc64 = mask ? hb[9] : n;
     const double area = (double)(ex + 1) * (double)(ey + 1);
     const double occ = c.cell_occupancy > 0 ? (double)c.cell_occupancy : 4.0;
     double side = sqrt(area * occ / std::max(1.0, (double)n / nz));
+    FarPlan fp;
+    fp.b_far = b_hi;
+    if constexpr (sizeof(T) == 4) {
+        const double carea = mask ? (double)((long long)hb[7] - hb[5] + 1) * (double)((long long)hb[8] - hb[6] + 1) : area;
+        fp = plan_far(ctx, n, nc64, area, carea, b_lo, b_hi);
+        if (fp.b_far < b_hi) side = fp.side;
+    }
+    int b_near = b_lo;
+    while (b_near < fp.b_far &&
+           M_PI * (double)n / nz / area * (double)(ctx->e2q[b_near + 1] - ctx->e2q[b_near]) < near_line(c.n_max, ctx->fp64))
+        ++b_near;
+    const double R = sqrt((double)ctx->e2q[fp.b_far]);
     side = std::max(side, (2.0 * R + 16.0) / (kMaxRows - 4));
     side = std::max(side, sqrt(area * nz / (double)(1 << 26)));
     side = std::max(side, 1.0);
@@ -752,6 +914,7 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
     }
     MP3_CK(ctx->centre_idx.ensure(sizeof(int) * n));
     MP3_CK(ctx->crow.ensure(sizeof(int) * n));
+    MP3_CK(ctx->posf.ensure(sizeof(float2) * n));
     MP3_CK(cudaMemsetAsync(ctx->fill.p, 0, sizeof(int) * (K + 1), st));
     ctx->launches[ST_SORT] += 4;
     k_keys<<<grid1d(n, ctx->n_sm), 256, 0, st>>>(n, xq, yq, zb, nz, g, ctx->key.as<int>(), ctx->fill.as<int>());
@@ -763,7 +926,7 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
     k_cell_order<<<grid1d(K, ctx->n_sm), 256, 0, st>>>(K, ctx->count.as<int>(), ctx->perm.as<int>());
     k_gather<T><<<grid1d(n, ctx->n_sm), 256, 0, st>>>(
         n, ctx->perm.as<int>(), xq, yq, g1, g2, w, zb, mask, ctx->pos.as<int2>(), ctx->pay.as<Pay<T>>(),
-        ctx->zs.as<uint8_t>(), ctx->cflag.as<int>(), nz, ctx->centre_idx.as<int>(), ctx->crow.as<int>());
+        ctx->zs.as<uint8_t>(), ctx->cflag.as<int>(), nz, ctx->posf.as<float2>(), g.x0, g.y0, ctx->centre_idx.as<int>(), ctx->crow.as<int>());
     MP3_CK(cudaGetLastError());
 
     // ---- centre list (sorted order) and each centre's row in galaxy-index order; without a mask
@@ -785,11 +948,7 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
         MP3_CK(cudaGetLastError());
         ctx->launches[ST_SORT] += 1;
     }
-    int nc = (int)n;
-    if (mask) {
-        MP3_CK(cudaMemcpyAsync(&nc, ctx->crank.as<int>() + n, sizeof(int), cudaMemcpyDeviceToHost, st));
-        MP3_CK(cudaStreamSynchronize(st));
-    }
+    const int nc = (int)nc64;
     ctx->n_centres = nc;
     stage_end(ctx, ST_SORT, t_sort);
     if (nc == 0) return MP3PCF_OK;
@@ -805,7 +964,7 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
     a.cell_start = ctx->count.as<int>();
     a.g = g;
     a.nz = nz;
-    a.nb = b_hi - b_lo;
+    a.nb = fp.b_far - b_lo;
     a.nbp = nb_pad(nb);
     a.n_max = c.n_max;
     a.e2q = ctx->d_e2q.as<long long>() + b_lo;
@@ -814,16 +973,35 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
     a.pairs = ctx->pairs.as<unsigned long long>();
     a.queue = ctx->pairs.as<unsigned long long>() + 2;
     if (b_lo >= b_hi) return MP3PCF_OK;
-    cudaError_t e;
-    {
-        StageScope sc(ctx, ST_MOMENTS);
+    StageScope sc(ctx, ST_MOMENTS);
+    if (fp.b_far < b_hi) {
+        if constexpr (sizeof(T) == 4) {
+            if (mp3pcf_status s = run_far(ctx, a, fp, b_lo, b_hi)) return s;
+        }
+    }
+    if (b_near > b_lo) {
+        NearArgs<T> na;
+        na.m = a;
+        na.m.nb = b_near - b_lo;
+        na.bins = ctx->bingeom.as<BinGeom>() + b_lo;
+        na.posf = ctx->posf.as<float2>();
+        na.queue = ctx->pairs.as<unsigned long long>() + 3 + kFarPlans;
         ctx->launches[ST_MOMENTS] += 1;
+        MP3_CK(launch_moments_near(na, ctx->n_sm, st));
+        a.nb -= b_near - b_lo;
+        a.e2q += b_near - b_lo;
+        a.G += b_near - b_lo;
+        a.W += b_near - b_lo;
+    }
+    if (a.nb > 0) {
+        ctx->launches[ST_MOMENTS] += 1;
+        cudaError_t e;
         if constexpr (sizeof(T) == 8)
             e = launch_moments_f64(a, ctx->n_sm, st);
         else
             e = launch_moments_f32(a, ctx->n_sm, st);
+        MP3_CK(e);
     }
-    MP3_CK(e);
     return MP3PCF_OK;
 }
 

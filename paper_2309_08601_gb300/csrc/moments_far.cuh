@@ -1,0 +1,54 @@
+// The moments of wide radial bins by angular sectors (moments_far.cu) and of narrow ones by a warp per
+// centre (moments_near.cu).
+#pragma once
+
+#include <vector>
+
+#include "common.cuh"
+
+namespace mp3 {
+
+// A radial bin for the FP32 distance test: with r^2 = fma(dx, dx, dy dy) (off by at most 2^-23 r^2)
+// and d = |r^2 - mid|, d < d_in is inside, d >= d_out outside; in between the integers decide.
+struct BinGeom {
+    float Ri, Ro, mid, d_in, d_out, pad;
+    long long e0, e1;
+};
+std::vector<BinGeom> bin_geometry(const std::vector<long long>& e2q);
+
+// tables of a context (they depend on n_max only): offsets into one float array of all variants
+constexpr int kFarPlans = 3;  // variants, widest bins first
+struct FarTables {
+    int sectors = 0, terms = 0;
+    double dmax = 0.0, half_width = 0.0;  // largest angle from a sector's axis; half a sector
+    int off_ray = 0, off_sin = 0, off_axis = 0, off_rot = 0, off_coef = 0;
+};
+void far_tables(int n_max, FarTables (&t)[kFarPlans], std::vector<float>* v);
+
+struct FarArgs {
+    MomentArgs<float> m;   // bins, pointers and outputs as in the direct form
+    const BinGeom* bins;   // from bin b_lo of the range
+    const float2* posf;    // sorted positions from the grid's origin (exact: the extent is below 2^24)
+    const int32_t* order;  // rows of the centres in strip order: (strip, column, row)
+    int strip_rows;        // cell rows of a strip
+    int max_cols;          // columns a group may span
+    int parts;             // work items a group's (bin, z) pairs are split into
+    const float* table;
+    int off_ray, off_sin, off_axis, off_rot, off_coef;
+    unsigned long long* queue;  // items claimed beyond the first gridDim.x (zero at launch)
+};
+
+cudaError_t launch_moments_far(const FarArgs& a, int plan, int n_sm, cudaStream_t st);
+
+template <typename T>
+struct NearArgs {
+    MomentArgs<T> m;
+    const BinGeom* bins;        // as in FarArgs
+    const float2* posf;
+    unsigned long long* queue;  // items claimed beyond the first gridDim.x * warps (zero at launch)
+    int parts;                  // set by the launcher: work items the bins of a centre are split into
+};
+cudaError_t launch_moments_near(const NearArgs<float>& a, int n_sm, cudaStream_t st);
+cudaError_t launch_moments_near(const NearArgs<double>& a, int n_sm, cudaStream_t st);
+
+}  // namespace mp3

@@ -1,0 +1,239 @@
+// Stage (a) for the narrow radial bins, those with few neighbours: the same sums as moments.cuh.
+//
+// The block-per-centre form spends some 9000 warp instructions per (centre, bin) on barriers, range
+// set-up, half-empty batches and the reduction over lanes, whatever the bin holds. Here a warp works
+// on a centre by itself and its lanes are the orders: lane l keeps W_m, A_m and B_m of
+// m = l, l + 32, ... The warp tests 32 candidates at a time, one per lane, and the lanes of members
+// store the powers z^0..z^7, z^8, z^16, z^24, z^32 of their direction; then the members are added one
+// after the other, every lane forming its own z^m from two of the stored powers. About 27 warp
+// instructions a member at n_max = 30, no reduction, no barrier; the direct form's 14 a member plus its
+// overhead are less from a few hundred members on. The order of the sums is fixed.
+#include <algorithm>
+
+#include "moments_far.cuh"
+#include "sector.cuh"
+
+namespace mp3 {
+
+namespace near {
+
+constexpr int kQueue = 128;
+constexpr int kPow = 13;  // stored powers of a member: z^0..z^7, z^0, z^8, z^16, z^24, z^32
+
+// warps of a block (the stored powers take 3.3 KB a warp in FP32) and blocks per SM the registers are
+// sized for
+template <typename T>
+struct Block {
+    static constexpr int kWarps = sizeof(T) == 8 ? 4 : 8, kThreads = kWarps * 32, kMin = sizeof(T) == 8 ? 4 : 3;
+};
+
+template <typename T>
+struct alignas(16) Member {
+    T a, b, w, pad;
+};
+
+__device__ __forceinline__ cx<float> direction(float dx, float dy, float)
+{
+    const float r2 = fmaf(dx, dx, dy * dy);
+    float inv = rsqrtf(r2);
+    inv = inv * (1.5f - 0.5f * r2 * inv * inv);
+    return {dx * inv, dy * inv};
+}
+__device__ __forceinline__ cx<double> direction(float dx, float dy, double)
+{
+    const double x = dx, y = dy, inv = 1.0 / sqrt(x * x + y * y);
+    return {x * inv, y * inv};
+}
+
+template <typename T>
+__device__ __forceinline__ void cacc(cx<T>& s, T v, cx<T> c)
+{
+    s.x += v * c.x;
+    s.y += v * c.y;
+}
+
+template <typename T, int SW, int SAB>
+__global__ void __launch_bounds__(Block<T>::kThreads, Block<T>::kMin) near_moments_kernel(const NearArgs<T> A)
+{
+    constexpr int kWarps = Block<T>::kWarps, kThreads = Block<T>::kThreads;
+    constexpr unsigned FULL = 0xffffffffu;
+    const MomentArgs<T>& m = A.m;
+    __shared__ BinGeom bins[kMaxBins];
+    __shared__ int queue[kWarps][kQueue];
+    __shared__ cx<T> pw[kWarps][32 * kPow];
+    __shared__ Member<T> mem[kWarps][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt_mask = (1u << lane) - 1u;
+    const int nz = m.nz, n_max = m.n_max;
+    const size_t plane = (size_t)m.n_centres * nz * m.nbp;
+    for (int b = threadIdx.x; b < m.nb; b += kThreads) {
+        bins[b] = A.bins[b];
+    }
+    __syncthreads();
+    int* qu = queue[warp];
+    cx<T>* P = pw[warp];
+    Member<T>* V = mem[warp];
+    SectorGeom g;
+    g.hx = g.hy = 0.0f;
+    g.S = (float)m.g.side;
+    g.iS = 1.0f / g.S;
+    g.ncx = m.g.ncx;
+    g.ncy = m.g.ncy;
+    unsigned long long my_pairs = 0;
+
+    const long long nitems = (long long)m.n_centres * A.parts;
+    for (long long item = blockIdx.x * kWarps + warp; item < nitems;) {
+        const int c = (int)(item / A.parts), part = (int)(item - (long long)c * A.parts);
+        const float2 pc = A.posf[m.centre_idx[c]];
+        g.gx = pc.x;
+        g.gy = pc.y;
+        for (int z = 0; z < nz; ++z) {
+            const int* row_start = m.cell_start + (size_t)z * m.g.ncells;
+            for (int b = part; b < m.nb; b += A.parts) {
+                const BinGeom bg = bins[b];
+                g.Ri = bg.Ri;
+                g.Ro = bg.Ro;
+                cx<T> aw[SW], aa[SAB], ab[SAB];
+#pragma unroll
+                for (int s = 0; s < SW; ++s) aw[s] = cx<T>{T(0), T(0)};
+#pragma unroll
+                for (int s = 0; s < SAB; ++s) aa[s] = ab[s] = cx<T>{T(0), T(0)};
+                const float ro = g.Ro + 8.0f;
+                const float iy0 = fmaxf(floorf((g.gy - ro) * g.iS), 0.0f);
+                const float iy1 = fminf(floorf((g.gy + ro) * g.iS), (float)(g.ncy - 1));
+                for (float iy = iy0 + (float)lane; iy - (float)lane <= iy1; iy += 32.0f) {
+                    int st0 = 0, n0 = 0, st1 = 0, n1 = 0;
+                    if (iy <= iy1)
+                        annulus_runs(g, iy, (iy + 0.5f) * g.S - g.gy, 0, g.ncx - 1, row_start, st0, n0, st1, n1);
+                    while (true) {
+                        // list the rows' candidates in row order
+                        const int len = n0 + n1;
+                        int incl = len;
+#pragma unroll
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const int y = __shfl_up_sync(FULL, incl, o);
+                            if (lane >= o) incl += y;
+                        }
+                        const int total = __shfl_sync(FULL, incl, 31);
+                        if (total == 0) break;
+                        const int off = incl - len;
+                        const int put = max(0, min(len, kQueue - off));
+                        for (int j = 0; j < put; ++j) qu[off + j] = j < n0 ? st0 + j : st1 + (j - n0);
+                        const int t0 = min(put, n0);
+                        st0 += t0;
+                        n0 -= t0;
+                        st1 += put - t0;
+                        n1 -= put - t0;
+                        const int n = min(total, kQueue);
+                        __syncwarp();
+                        for (int t = lane; t < n + lane; t += 32) {
+                            const int i = qu[min(t, n - 1)];
+                            const float2 p = A.posf[i];
+                            const float dx = p.x - pc.x, dy = p.y - pc.y;  // exact
+                            const float d = fabsf(fmaf(dx, dx, dy * dy) - bg.mid);
+                            bool in = d < bg.d_in;
+                            if (!in && d < bg.d_out) {
+                                const long long q2 = (long long)(int)dx * (int)dx + (long long)(int)dy * (int)dy;
+                                in = q2 >= bg.e0 && q2 < bg.e1;
+                            }
+                            in = in && t < n;
+                            const unsigned mask = __ballot_sync(FULL, in);
+                            if (mask == 0) continue;
+                            if (in) {
+                                const int slot = __popc(mask & lt_mask);
+                                const Pay<T> v = m.pay[i];
+                                V[slot] = Member<T>{v.a, v.b, v.w, T(0)};
+                                const cx<T> z1 = direction(dx, dy, T(0));
+                                cx<T>* q = P + slot * kPow;
+                                const cx<T> z2 = cmul(z1, z1), z4 = cmul(z2, z2), z3 = cmul(z2, z1);
+                                const cx<T> z8 = cmul(z4, z4), z16 = cmul(z8, z8);
+                                q[0] = q[8] = cx<T>{T(1), T(0)};
+                                q[1] = z1;
+                                q[2] = z2;
+                                q[3] = z3;
+                                q[4] = z4;
+                                q[5] = cmul(z4, z1);
+                                q[6] = cmul(z4, z2);
+                                q[7] = cmul(z4, z3);
+                                q[9] = z8;
+                                q[10] = z16;
+                                q[11] = cmul(z16, z8);
+                                if (SW > 1) q[12] = cmul(z16, z16);
+                            }
+                            __syncwarp();
+                            const int cnt = __popc(mask);
+                            my_pairs += cnt;
+#pragma unroll 2
+                            for (int j = 0; j < cnt; ++j) {
+                                const cx<T>* q = P + j * kPow;
+                                const Member<T> v = V[j];
+                                cx<T> zc = cmul(q[lane & 7], q[8 + (lane >> 3)]);
+#pragma unroll
+                                for (int s = 0; s < SW; ++s) {
+                                    cacc(aw[s], v.w, zc);
+                                    if (s < SAB) {
+                                        cacc(aa[s], v.a, zc);
+                                        cacc(ab[s], v.b, zc);
+                                    }
+                                    if (s + 1 < SW) zc = cmul(zc, q[12]);
+                                }
+                            }
+                            __syncwarp();
+                        }
+                        if (total <= kQueue) break;
+                    }
+                }
+                const size_t row = ((size_t)c * nz + z) * m.nbp + b;
+#pragma unroll
+                for (int s = 0; s < SW; ++s) {
+                    const int mm = lane + 32 * s;
+                    if (mm <= 2 * n_max) m.W[(size_t)mm * plane + row] = aw[s];
+                    if (s < SAB) {
+                        const cx<T> a = aa[s < SAB ? s : 0], bb = ab[s < SAB ? s : 0];
+                        if (mm <= n_max - 1) m.G[(size_t)(mm + n_max + 3) * plane + row] = cx<T>{a.x - bb.y, a.y + bb.x};
+                        if (mm >= 1 && mm <= n_max + 3)
+                            m.G[(size_t)(n_max + 3 - mm) * plane + row] = cx<T>{a.x + bb.y, bb.x - a.y};
+                    }
+                }
+            }
+        }
+        long long nx = 0;
+        if (lane == 0) nx = (long long)atomicAdd(A.queue, 1ull) + (long long)gridDim.x * kWarps;
+        item = __shfl_sync(FULL, nx, 0);
+    }
+    if (lane == 0 && my_pairs) atomicAdd(m.pairs, my_pairs);
+}
+
+template <typename T, int SW, int SAB>
+static cudaError_t launch(NearArgs<T> a, int n_sm, cudaStream_t st)
+{
+    constexpr int kWarps = Block<T>::kWarps, kThreads = Block<T>::kThreads;
+    int per_sm = 0;
+    const cudaError_t e = occupancy(&per_sm, near_moments_kernel<T, SW, SAB>, kThreads, 0);
+    if (e != cudaSuccess) return e;
+    const int64_t slots = (int64_t)n_sm * std::max(per_sm, 1) * kWarps;
+    if (a.m.n_centres < 1) return cudaSuccess;
+    // few centres: the bins of a centre go to several warps (a chain of small bins is all latency)
+    a.parts = (int)std::min<int64_t>(a.m.nb, std::max<int64_t>(1, 4 * slots / a.m.n_centres));
+    const int64_t grid = (std::min<int64_t>((int64_t)a.m.n_centres * a.parts, slots) + kWarps - 1) / kWarps;
+    near_moments_kernel<T, SW, SAB><<<(unsigned)grid, kThreads, 0, st>>>(a);
+    return cudaGetLastError();
+}
+
+template <typename T>
+static cudaError_t dispatch(const NearArgs<T>& a, int n_sm, cudaStream_t st)
+{
+    const int sw = std::max(2 * a.m.n_max, a.m.n_max + 3) / 32 + 1, sab = (a.m.n_max + 3) / 32 + 1;
+    if (sw == 1) return launch<T, 1, 1>(a, n_sm, st);
+    if (sw == 2 && sab == 1) return launch<T, 2, 1>(a, n_sm, st);
+    if (sw == 2) return launch<T, 2, 2>(a, n_sm, st);
+    if (sw == 3) return launch<T, 3, 2>(a, n_sm, st);
+    return launch<T, 4, 2>(a, n_sm, st);
+}
+
+}  // namespace near
+
+cudaError_t launch_moments_near(const NearArgs<float>& a, int n_sm, cudaStream_t st) { return near::dispatch(a, n_sm, st); }
+cudaError_t launch_moments_near(const NearArgs<double>& a, int n_sm, cudaStream_t st) { return near::dispatch(a, n_sm, st); }
+
+}  // namespace mp3
