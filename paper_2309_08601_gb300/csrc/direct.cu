@@ -89,6 +89,164 @@ __global__ void __launch_bounds__(kDirThreads) map3_direct_kernel(int64_t n, con
     }
 }
 
+// The same sums from a cell-sorted copy of the catalog: a block per (aperture, radii triple) reads only
+// the cells its cut-off circle meets, warps over the cell rows (each a contiguous run), lanes over the
+// galaxies. Bound by FP64 arithmetic on the galaxies inside (two FP64 lanes per SM and cycle), so a
+// radius that occurs twice in a triple is evaluated once, and equal radii need three powers of one
+// factor. 200 000 galaxies, 900 apertures x 3 triples: 67.5 ms by scanning the catalog, 2.7 ms by cells.
+template <int R>  // distinct radii of the triple: 1 (all equal), 2 (the first two equal) or 3
+__device__ __forceinline__ void direct_sums(double (&s)[14], const double (&b)[3], double gt)
+{
+    double c[3];
+#pragma unroll
+    for (int l = 0; l < R; ++l) c[l] = b[l] * gt;
+    const int i1 = R == 3 ? 1 : 0, i2 = R - 1;
+    s[0] += c[0];
+    s[7] += b[0];
+    const double c01 = c[0] * c[i1], b01 = b[0] * b[i1];
+    s[3] += c01;
+    s[10] += b01;
+    s[6] += c01 * c[i2];
+    s[13] += b01 * b[i2];
+    if (R > 1) {
+        s[2] += c[i2];
+        s[4] += c[0] * c[i2];
+        s[9] += b[i2];
+        s[11] += b[0] * b[i2];
+    }
+    if (R > 2) {
+        s[1] += c[1];
+        s[5] += c[1] * c[2];
+        s[8] += b[1];
+        s[12] += b[1] * b[2];
+    }
+}
+
+template <int R>
+__device__ __forceinline__ void direct_cells(double (&s)[14], const int2* __restrict__ pos,
+                                             const float4* __restrict__ gw, const int* __restrict__ start,
+                                             const GridDesc& g, double quantum, double cx, double cy, double rcut,
+                                             double r2max, const double (&inv2)[3], const double (&nrm)[3])
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // in cells, two quanta wider than the circle; fmin and fmax drop NaNs (the whole grid)
+    const double is = 1.0 / (double)g.side, xc = (cx / quantum - (double)g.x0) * is, yc = (cy / quantum - (double)g.y0) * is;
+    const double rc = (rcut / quantum + 2.0) * is * (1.0 + 1e-9);
+    const int iy0 = (int)fmin(fmax(floor(yc - rc), 0.0), (double)g.ncy), iy1 = (int)fmax(fmin(floor(yc + rc), (double)g.ncy - 1.0), -1.0);
+    for (int iy = iy0 + warp; iy <= iy1; iy += kDirThreads / 32) {
+        const double dy = fmax(fmax((double)iy - yc, yc - (double)iy - 1.0), 0.0);
+        const double hx = sqrt(fmax(rc * rc - dy * dy, 0.0)) + 1e-6 * rc;
+        const int ix0 = (int)fmin(fmax(floor(xc - hx), 0.0), (double)g.ncx), ix1 = (int)fmax(fmin(floor(xc + hx), (double)g.ncx - 1.0), -1.0);
+        if (ix0 > ix1) continue;
+        const int k1 = start[iy * g.ncx + ix1 + 1];
+        for (int k = start[iy * g.ncx + ix0] + lane; k < k1; k += 32) {
+            const int2 p = pos[k];
+            const double dx = (double)p.x * quantum - cx, dyk = (double)p.y * quantum - cy;
+            const double r2 = dx * dx + dyk * dyk;
+            if (r2 == 0.0 || r2 > r2max) continue;
+            const float4 v = gw[k];
+            const double gt = -((double)v.x * (dx * dx - dyk * dyk) + 2.0 * (double)v.y * dx * dyk) / r2;
+            const double wr = (double)v.z * r2;
+            double b[3];
+#pragma unroll
+            for (int l = 0; l < R; ++l) {
+                const int i = R == 2 && l == 1 ? 2 : l;
+                b[l] = wr * nrm[i] * exp(-r2 * inv2[i]);
+            }
+            direct_sums<R>(s, b, gt);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kDirThreads) map3_direct_cells_kernel(const int2* __restrict__ pos,
+                                                                        const float4* __restrict__ gw,
+                                                                        const int* __restrict__ start,
+                                                                        const GridDesc* __restrict__ grid, double quantum,
+                                                                        int n_ap, const double* __restrict__ centres,
+                                                                        const double* __restrict__ theta,
+                                                                        double rcut_factor, double* __restrict__ out)
+{
+    __shared__ double red[14][kDirThreads / 32];
+    const int64_t job = blockIdx.x;
+    const int64_t t = job / n_ap;
+    const int a = (int)(job % n_ap);
+    double th[3], inv2[3], nrm[3];
+    for (int l = 0; l < 3; ++l) th[l] = theta[3 * a + l];
+    // equal radii first: the sums over distinct triplets are symmetric in the slots
+    if (th[0] != th[1]) {
+        if (th[0] == th[2]) {
+            const double x = th[1];
+            th[1] = th[2];
+            th[2] = x;
+        } else if (th[1] == th[2]) {
+            const double x = th[0];
+            th[0] = th[2];
+            th[2] = x;
+        }
+    }
+    for (int l = 0; l < 3; ++l) {
+        inv2[l] = 1.0 / (2.0 * th[l] * th[l]);
+        nrm[l] = 1.0 / (4.0 * M_PI * th[l] * th[l] * th[l] * th[l]);
+    }
+    const double rcut = rcut_factor * fmax(th[0], fmax(th[1], th[2]));
+    // the largest r^2 whose square root is not above rcut: the same galaxies as sqrt(r2) > rcut leaves
+    double r2max = rcut * rcut;
+    for (int i = 0; i < 4 && sqrt(r2max) > rcut; ++i) r2max = __longlong_as_double(__double_as_longlong(r2max) - 1);
+    for (int i = 0; i < 4 && r2max > 0.0; ++i) {
+        const double up = __longlong_as_double(__double_as_longlong(r2max) + 1);
+        if (!(sqrt(up) <= rcut)) break;
+        r2max = up;
+    }
+    if (!(rcut >= 0.0)) r2max = rcut;  // NaN: no galaxy is left out; negative: all are
+    double s[14];
+#pragma unroll
+    for (int v = 0; v < 14; ++v) s[v] = 0.0;
+    const GridDesc g = *grid;
+    const double cx = centres[2 * t], cy = centres[2 * t + 1];
+    const bool e01 = th[0] == th[1], e12 = th[1] == th[2];
+    if (e01 && e12) {
+        direct_cells<1>(s, pos, gw, start, g, quantum, cx, cy, rcut, r2max, inv2, nrm);
+        s[1] = s[2] = s[0];
+        s[4] = s[5] = s[3];
+        s[8] = s[9] = s[7];
+        s[11] = s[12] = s[10];
+    } else if (e01) {
+        direct_cells<2>(s, pos, gw, start, g, quantum, cx, cy, rcut, r2max, inv2, nrm);
+        s[1] = s[0];
+        s[5] = s[4];
+        s[8] = s[7];
+        s[12] = s[11];
+    } else {
+        direct_cells<3>(s, pos, gw, start, g, quantum, cx, cy, rcut, r2max, inv2, nrm);
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int v = 0; v < 14; ++v) {
+        double x = s[v];
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (lane == 0) red[v][warp] = x;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double q[14];
+        for (int v = 0; v < 14; ++v) {
+            q[v] = 0.0;
+            for (int k = 0; k < kDirThreads / 32; ++k) q[v] += red[v][k];
+        }
+        out[2 * job] = q[0] * q[1] * q[2] - q[3] * q[2] - q[4] * q[1] - q[5] * q[0] + 2.0 * q[6];
+        out[2 * job + 1] = q[7] * q[8] * q[9] - q[10] * q[9] - q[11] * q[8] - q[12] * q[7] + 2.0 * q[13];
+    }
+}
+
+cudaError_t launch_map3_direct_cells(const int2* pos, const float4* gw, const int* start, const GridDesc* grid,
+                                     double quantum, int64_t n_cen, const double* centres, int n_ap, const double* theta,
+                                     double rcut_factor, double* out, cudaStream_t st)
+{
+    map3_direct_cells_kernel<<<(unsigned)(n_cen * n_ap), kDirThreads, 0, st>>>(pos, gw, start, grid, quantum, n_ap, centres,
+                                                                               theta, rcut_factor, out);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_map3_direct(int64_t n, const int32_t* xq, const int32_t* yq, const float* g1, const float* g2,
                                const float* w, double quantum, int64_t n_cen, const double* centres, int n_ap,
                                const double* theta, double rcut_factor, double* out, cudaStream_t st)
