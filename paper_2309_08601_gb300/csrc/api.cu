@@ -483,7 +483,7 @@ struct mp3pcf_ctx {
     DevBuf d_e2q, d_edges, d_nodes;
     DevBuf bb, key, count, fill, scan_sums, scan_total, perm, pos, pay, zs;
     DevBuf cflag, crank, oflag, orank, centre_idx, crow;
-    DevBuf G, W, pairs, partial, singular, m3partial, m3four, ccoef;
+    DevBuf G, W, pairs, partial, singular, m3partial, m3filter, m3four, ccoef;
     DevBuf gG, gW, gv, gtab, adjscratch;  // adjoint workspace
     DevBuf degen;                       // exclude_degenerate sums per (centre, z, bin)
     DevBuf degen_grad;                  // their gradient sums per (Z1, z, bin) in the adjoint
@@ -687,7 +687,7 @@ mp3pcf_status mp3pcf_destroy(mp3pcf_ctx* ctx)
                       &ctx->pos, &ctx->pay, &ctx->zs, &ctx->cflag,
                       &ctx->crank, &ctx->oflag, &ctx->orank, &ctx->centre_idx, &ctx->crow,
                       &ctx->G, &ctx->W, &ctx->pairs, &ctx->partial, &ctx->singular,
-                      &ctx->m3partial, &ctx->m3four, &ctx->fftwork, &ctx->ccoef, &ctx->gG, &ctx->gW, &ctx->gv, &ctx->gtab,
+                      &ctx->m3partial, &ctx->m3filter, &ctx->m3four, &ctx->fftwork, &ctx->ccoef, &ctx->gG, &ctx->gW, &ctx->gv, &ctx->gtab,
                       &ctx->adjscratch, &ctx->degen, &ctx->degen_grad, &ctx->zrange, &ctx->dkey, &ctx->dcell, &ctx->dperm, &ctx->dpos, &ctx->dgw, &ctx->dgrid, &ctx->bingeom, &ctx->ftable, &ctx->posf, &ctx->fkey, &ctx->fstart, &ctx->ffill, &ctx->forder, &ctx->gridsum, &ctx->gridflag, &ctx->bups, &ctx->bnorm,
                       &ctx->bgam, &ctx->bgcen, &ctx->berr, &ctx->pix, &ctx->pixinv};
     for (DevBuf* b : bufs) b->release();
@@ -1343,6 +1343,14 @@ mp3pcf_status mp3pcf_to_map3(mp3pcf_ctx* ctx, const double* d_gamma_cen, int64_t
     const int chunks = 64;
     MP3_CK(ctx->m3partial.ensure(sizeof(double) * 8 * (size_t)z3 * n_ap * chunks));
     StageScope sc(ctx, ST_MAP3);
+    const size_t fb = map3_scratch(post_args(ctx), n_ap);
+    if (fb) {
+        MP3_CK(ctx->m3filter.ensure(fb));
+        ctx->launches[ST_MAP3] += 2 * ((n_ap + 3) / 4) + 1;
+        MP3_CK(launch_to_map3_filtered(post_args(ctx), d_gamma_cen, (int)n_ap, d_theta_ap, ctx->m3filter.as<double>(),
+                                       ctx->m3partial.as<double>(), d_corr, d_m8, ctx->st));
+        return MP3PCF_OK;
+    }
     ctx->launches[ST_MAP3] += 2;
     MP3_CK(launch_to_map3(post_args(ctx), d_gamma_cen, (int)n_ap, d_theta_ap,
                           ctx->m3partial.as<double>(), chunks, d_corr, d_m8, ctx->st));

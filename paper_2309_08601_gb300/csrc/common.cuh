@@ -190,6 +190,10 @@ cudaError_t launch_map3_direct_cells(const int2* pos, const float4* gw, const in
 cudaError_t launch_to_map3(const PostArgs& p, const double* gcen, int n_ap, const double* theta,
                            double* partial, int chunks, double* corr, double* m8,
                            cudaStream_t st);
+// the same with the filters tabulated once per radii triple (map3_scratch bytes; 0: not this form)
+size_t map3_scratch(const PostArgs& p, int64_t n_ap);
+cudaError_t launch_to_map3_filtered(const PostArgs& p, const double* gcen, int n_ap, const double* theta, double* filters,
+                                    double* partial, double* corr, double* m8, cudaStream_t st);
 // the four-equation form: theta3 [3 n_ap][3] and corr3 [n_z^3][3 n_ap][4] complex are scratch,
 // partial as for launch_to_map3 with 3 n_ap apertures; m4 [n_z^3][n_ap][4]
 cudaError_t launch_to_map3_four(const PostArgs& p, const double* gcen, int n_ap, const double* theta, double* theta3,

@@ -1,5 +1,7 @@
-"""Forms of the FP64 stages at the sizes where they can go wrong: the direct estimator's cells (1e-12
-normwise between two forms of the library that add the same terms in another order)."""
+"""The FP64 stages' forms: angular nodes folded by symmetry (to_gamma), filters tabulated per radii
+triple (to_map3) and the direct estimator's cells, at the sizes where they can go wrong. FP64
+throughout: 1e-10 normwise, the tolerance of the FP64 path (1e-12 between two forms of the library
+that add the same terms in another order)."""
 import numpy as np
 import pytest
 import torch
@@ -17,6 +19,50 @@ def gpu():
     assert torch.cuda.is_available(), "GPU tests need CUDA"
     from paper_2309_08601_gb300 import api
     return api
+
+
+def _gamma_n(nz, nb, n_max, seed):
+    rng = np.random.default_rng(seed)
+    shape = (nz ** 3, 4, 2 * n_max + 1, nb, nb)
+    return rng.normal(size=shape) + 1j * rng.normal(size=shape)
+
+
+@pytest.mark.parametrize("n_phi", [1, 2, 3, 6, 7, 10, 33, 100, 514, 1030])
+@pytest.mark.parametrize("nz, nb, n_max", [(1, 3, 0), (1, 7, 5), (2, 3, 4), (3, 2, 1)])
+def test_to_gamma_folds_every_node(gpu, orc, nz, nb, n_max, n_phi):
+    setup = dict(n_bins=nb, theta_min=0.7, theta_max=9.0, n_max=n_max, n_phi=n_phi, n_z=nz)
+    g = _gamma_n(nz, nb, n_max, n_phi)
+    g[0, 1, :, 0, nb - 1] = np.nan  # a singular system stays in its own cell
+    with gpu.Estimator(**setup, precision="fp64") as est:
+        for proj in (0, 1, 2):
+            want = orc.to_gamma(orc.Setup(**setup), g, proj)
+            got = est.to_gamma(torch.as_tensor(g, device="cuda"), proj).cpu().numpy()
+            if proj == 1 and n_phi % 2:
+                # node phi = pi, equal radii: the third vertex on the first, where the centroid factor is
+                # 0 / 0 (the GPU's cos pi is -1 exactly, the oracle's sin pi is not 0)
+                i = np.arange(nb)
+                want[:, :, i, i, n_phi // 2] = np.nan
+            np.testing.assert_array_equal(np.isnan(got), np.isnan(want))
+            ok = ~np.isnan(want)
+            assert rel_err(got[ok], want[ok]) < 1e-10, proj
+
+
+@pytest.mark.parametrize("n_phi", [36, 37])
+@pytest.mark.parametrize("nz, n_ap", [(1, 1), (1, 4), (1, 5), (2, 3), (2, 9)])
+def test_to_map3_by_tabulated_filters(gpu, orc, nz, n_ap, n_phi):
+    setup = dict(n_bins=5, theta_min=0.5, theta_max=12.0, n_max=3, n_phi=n_phi, n_z=nz)
+    rng = np.random.default_rng(n_ap)
+    shape = (nz ** 3, 4, 5, 5, n_phi)
+    gc = rng.normal(size=shape) + 1j * rng.normal(size=shape)
+    th = rng.uniform(1.0, 4.0, (n_ap, 3))
+    corr, m8 = orc.to_map3(orc.Setup(**setup), gc, th)
+    with gpu.Estimator(**setup, precision="fp64") as est:
+        gcorr, gm8 = est.to_map3(torch.as_tensor(gc, device="cuda"), th)
+    if n_phi % 2:  # the node phi = pi with equal radii is 0 / 0 in the filter on the GPU
+        assert bool(torch.isnan(gm8).all()) and bool(torch.isnan(torch.view_as_real(gcorr)).all())
+        return
+    assert rel_err(gcorr.cpu().numpy(), corr) < 1e-10
+    assert rel_err(gm8.cpu().numpy(), m8) < 1e-10
 
 
 @pytest.mark.parametrize("theta", [[3.0, 3.0, 3.0], [2.0, 2.0, 3.5], [3.5, 2.0, 2.0], [2.0, 3.5, 2.0], [1.5, 2.0, 3.5]])
