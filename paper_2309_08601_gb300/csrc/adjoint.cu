@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(kPairWarps * 32) moments_adjoint_pairs(const A
     for (int c = blockIdx.x * kPairWarps + warp; c < a.n_centres; c += gridDim.x * kPairWarps) {
         const int d = a.centre_idx[c];
         const int2 p = a.pos[d];
-        for (int b = 0; b < nb; ++b) {
+        for (int b = 0; b < a.nb_pairs; ++b) {
             __syncwarp();
             for (int i = lane; i < nz * (MG + MW); i += 32) {
                 const int z = i / (MG + MW), qq = i % (MG + MW);
@@ -703,7 +703,8 @@ static cudaError_t run_degenerate(const AdjArgs<T>& a, cx<T>* scratch, double* u
 
 template <typename T>
 static cudaError_t run(const AdjArgs<T>& a, int64_t n, const int* perm, const float* g1, const float* g2,
-                       const float* w, float* dg1, float* dg2, float* dw, int n_sm, cudaStream_t st)
+                       const float* w, float* dg1, float* dg2, float* dw, int n_sm, cudaStream_t st,
+                       cudaError_t (*far)(void*) = nullptr, void* far_arg = nullptr)
 {
     cudaError_t e = cudaMemsetAsync(a.gvw, 0, sizeof(T) * 4 * (size_t)n, st);
     if (e != cudaSuccess) return e;
@@ -727,8 +728,9 @@ static cudaError_t run(const AdjArgs<T>& a, int64_t n, const int* perm, const fl
         e = set_smem_attr(moments_adjoint_pairs<T>, sm_pair);
         if (e != cudaSuccess) return e;
         const int blocks = (int)std::min<int64_t>((a.n_centres + kPairWarps - 1) / kPairWarps, (int64_t)n_sm * 32);
-        moments_adjoint_pairs<T><<<blocks, kPairWarps * 32, sm_pair, st>>>(a);
+        if (a.nb_pairs > 0) moments_adjoint_pairs<T><<<blocks, kPairWarps * 32, sm_pair, st>>>(a);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if (far && (e = far(far_arg)) != cudaSuccess) return e;
     }
     if (a.dgs && a.n_centres > 0) {
         // the j = k triplets left out of the forward (exclude_degenerate)
@@ -748,9 +750,9 @@ static cudaError_t run(const AdjArgs<T>& a, int64_t n, const int* perm, const fl
 
 cudaError_t launch_moments_adjoint_f32(const AdjArgs<float>& a, int64_t n, const int* perm, const float* g1,
                                        const float* g2, const float* w, float* dg1, float* dg2, float* dw,
-                                       int n_sm, cudaStream_t st)
+                                       int n_sm, cudaStream_t st, cudaError_t (*far)(void*), void* far_arg)
 {
-    return adj::run<float>(a, n, perm, g1, g2, w, dg1, dg2, dw, n_sm, st);
+    return adj::run<float>(a, n, perm, g1, g2, w, dg1, dg2, dw, n_sm, st, far, far_arg);
 }
 
 cudaError_t launch_moments_adjoint_f64(const AdjArgs<double>& a, int64_t n, const int* perm, const float* g1,

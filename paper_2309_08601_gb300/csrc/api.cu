@@ -458,6 +458,14 @@ using namespace mp3;
 
 // ------------------------------------------------------------------ context
 
+// The sector form of the moments (moments_far.cu) for the bins [b_far, b_hi): groups of kFarGroup
+// centres in strips of `rows` cell rows and at most `cols` columns, on cells of side `side`.
+struct FarPlan {
+    int b_far = 0, rows = 1, cols = 1;
+    int b[kFarPlans + 1] = {0};  // bins [b[v + 1], b[v]) take variant v (b[0] = b_hi)
+    double side = 1.0;
+};
+
 struct mp3pcf_ctx {
     mp3pcf_config cfg;
     cudaStream_t st = nullptr;
@@ -490,6 +498,7 @@ struct mp3pcf_ctx {
     DevBuf zrange;                      // [nz + 1] centre range of each z-bin
     // wide bins by angular sectors (moments_far.cu): tables, FP32 positions, centres in strip order
     FarTables far[kFarPlans];
+    FarPlan fplan;  // of the last accumulate call
     DevBuf bingeom, ftable, posf, fkey, fstart, ffill, forder;
     DevBuf fftwork;                     // FFT grid moments: padded fields, kernels, products
     FftPlanCache* fft = nullptr;        // cuFFT plans of the FFT grid moments
@@ -745,14 +754,6 @@ static unsigned grid1d(int64_t n, int n_sm)
     return (unsigned)(g < 1 ? 1 : g);
 }
 
-// The sector form of the moments (moments_far.cu) for the bins [b_far, b_hi): groups of kFarGroup
-// centres in strips of `rows` cell rows and at most `cols` columns, on cells of side `side`.
-struct FarPlan {
-    int b_far = 0, rows = 1, cols = 1;
-    int b[kFarPlans + 1] = {0};  // bins [b[v + 1], b[v]) take variant v (b[0] = b_hi)
-    double side = 1.0;
-};
-
 // Expected neighbours of a (centre, bin) below which the warp-per-centre form (moments_near.cu) is
 // faster than the block-per-centre form: about 300 + (5 + 6 SW + 4 SAB) N warp instructions a bin
 // against 300 n_max + n_max N / 2 (lines measured at n_max 10, 20 and 30 in FP32; in FP64, where a
@@ -801,6 +802,34 @@ static FarPlan plan_far(const mp3pcf_ctx* ctx, int64_t n, int64_t nc, double are
     return f;
 }
 
+// arguments of variant v for its bins (false: none); a: the whole range's, from bin b_lo
+static bool far_args(mp3pcf_ctx* ctx, const MomentArgs<float>& a, const FarPlan& fp, int v, int b_lo, FarArgs* f)
+{
+    const int b0 = fp.b[v + 1], nbv = fp.b[v] - b0, groups = (a.n_centres + 7) / 8;
+    if (nbv < 1) return false;
+    f->m = a;
+    f->m.nb = nbv;
+    f->m.e2q = a.e2q + (b0 - b_lo);
+    f->m.G = a.G + (b0 - b_lo);
+    f->m.W = a.W + (b0 - b_lo);
+    f->bins = ctx->bingeom.as<BinGeom>() + b0;
+    f->posf = ctx->posf.as<float2>();
+    f->order = ctx->forder.as<int>();
+    f->strip_rows = fp.rows;
+    f->max_cols = fp.cols;
+    // about six items per resident block, so that the last ones end together
+    f->parts = std::max(1, std::min(nbv * a.nz, (ctx->n_sm * 12 + groups - 1) / groups));
+    f->table = ctx->ftable.as<float>();
+    f->off_ray = ctx->far[v].off_ray;
+    f->off_sin = ctx->far[v].off_sin;
+    f->off_axis = ctx->far[v].off_axis;
+    f->off_rot = ctx->far[v].off_rot;
+    f->off_coef = ctx->far[v].off_coef;
+    f->queue = ctx->pairs.as<unsigned long long>() + 3 + v;
+    f->gvw = nullptr;
+    return true;
+}
+
 static mp3pcf_status run_far(mp3pcf_ctx* ctx, const MomentArgs<float>& a, const FarPlan& fp, int b_lo, int b_hi)
 {
     cudaStream_t st = ctx->st;
@@ -821,30 +850,9 @@ static mp3pcf_status run_far(mp3pcf_ctx* ctx, const MomentArgs<float>& a, const 
     k_cell_order<<<grid1d(K, ctx->n_sm), 256, 0, st>>>(K, ctx->fstart.as<int>(), ctx->forder.as<int>());
     MP3_CK(cudaGetLastError());
     ctx->launches[ST_MOMENTS] += 3;
-    const int groups = (nc + 7) / 8;
     for (int v = 0; v < kFarPlans; ++v) {
-        const int b0 = fp.b[v + 1], nbv = fp.b[v] - b0;
-        if (nbv < 1) continue;
         FarArgs f;
-        f.m = a;
-        f.m.nb = nbv;
-        f.m.e2q = a.e2q + (b0 - b_lo);
-        f.m.G = a.G + (b0 - b_lo);
-        f.m.W = a.W + (b0 - b_lo);
-        f.bins = ctx->bingeom.as<BinGeom>() + b0;
-        f.posf = ctx->posf.as<float2>();
-        f.order = ctx->forder.as<int>();
-        f.strip_rows = fp.rows;
-        f.max_cols = fp.cols;
-        // about six items per resident block, so that the last ones end together
-        f.parts = std::max(1, std::min(nbv * a.nz, (ctx->n_sm * 12 + groups - 1) / groups));
-        f.table = ctx->ftable.as<float>();
-        f.off_ray = ctx->far[v].off_ray;
-        f.off_sin = ctx->far[v].off_sin;
-        f.off_axis = ctx->far[v].off_axis;
-        f.off_rot = ctx->far[v].off_rot;
-        f.off_coef = ctx->far[v].off_coef;
-        f.queue = ctx->pairs.as<unsigned long long>() + 3 + v;
+        if (!far_args(ctx, a, fp, v, b_lo, &f)) continue;
         ctx->launches[ST_MOMENTS] += 1;
         MP3_CK(launch_moments_far(f, v, ctx->n_sm, st));
     }
@@ -914,6 +922,7 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
         fp = plan_far(ctx, n, nc64, area, carea, b_lo, b_hi);
         if (fp.b_far < b_hi) side = fp.side;
     }
+    ctx->fplan = fp;
     int b_near = b_lo;
     while (b_near < fp.b_far &&
            M_PI * (double)n / nz / area * (double)(ctx->e2q[b_near + 1] - ctx->e2q[b_near]) < near_line(c.n_max, ctx->fp64))
@@ -1790,13 +1799,51 @@ static mp3pcf_status moments_adjoint_t(mp3pcf_ctx* ctx, const double* gups, cons
     }
     a.tabX = ctx->gtab.as<cx<T>>();
     a.tabY = a.tabX + ngroups * nb * nb;
+    a.nb_pairs = nb;
     StageScope sc(ctx, ST_MOMENTS);
     ctx->launches[ST_MOMENTS] += nc > 0 ? 4 : 1;
     cudaError_t e;
-    if constexpr (sizeof(T) == 8)
+    if constexpr (sizeof(T) == 8) {
         e = launch_moments_adjoint_f64(a, n, ctx->perm.as<int>(), g1, g2, w, dg1, dg2, dw, ctx->n_sm, ctx->st);
-    else
-        e = launch_moments_adjoint_f32(a, n, ctx->perm.as<int>(), g1, g2, w, dg1, dg2, dw, ctx->n_sm, ctx->st);
+    } else {
+        // the bins that the forward took by sectors
+        a.nb_pairs = ctx->fplan.b_far;
+        struct Far {
+            mp3pcf_ctx* ctx;
+            const AdjArgs<float>* a;
+            static cudaError_t run(void* p)
+            {
+                mp3pcf_ctx* ctx = static_cast<Far*>(p)->ctx;
+                const AdjArgs<float>& a = *static_cast<Far*>(p)->a;
+                cudaError_t e = cudaMemsetAsync(ctx->pairs.as<unsigned long long>() + 3, 0, 8 * kFarPlans, ctx->st);
+                if (e != cudaSuccess) return e;
+                MomentArgs<float> m{};
+                m.n_centres = a.n_centres;
+                m.centre_idx = a.centre_idx;
+                m.pos = a.pos;
+                m.pay = a.pay;
+                m.cell_start = a.cell_start;
+                m.g = a.g;
+                m.nz = a.nz;
+                m.nb = a.nb;
+                m.n_max = a.n_max;
+                m.nbp = nb_pad(a.nb);
+                m.e2q = a.e2q;
+                m.G = a.gG;
+                m.W = a.gW;
+                for (int v = 0; v < kFarPlans; ++v) {
+                    FarArgs f;
+                    if (!far_args(ctx, m, ctx->fplan, v, 0, &f)) continue;
+                    f.gvw = a.gvw;
+                    ctx->launches[ST_MOMENTS] += 1;
+                    if ((e = launch_moments_far_adjoint(f, v, ctx->n_sm, ctx->st)) != cudaSuccess) return e;
+                }
+                return cudaSuccess;
+            }
+        } far{ctx, &a};
+        e = launch_moments_adjoint_f32(a, n, ctx->perm.as<int>(), g1, g2, w, dg1, dg2, dw, ctx->n_sm, ctx->st,
+                                       a.nb_pairs < nb ? Far::run : nullptr, &far);
+    }
     MP3_CK(e);
     return MP3PCF_OK;
 }

@@ -223,14 +223,16 @@ struct AdjArgs {
     cx<T>* gW;
     T* gvw;                     // [n][4] per sorted galaxy: dL/dv (re, im; v = w gamma), direct
                                 // dL/dw, unused (16 bytes: one vector atomic per pair in FP32)
+    int32_t nb_pairs;           // the pair kernel's bins [0, nb_pairs); the rest take the sector form
     // exclude_degenerate: scratch for the gradients of the j = k sums, [n_z][n_z][nb][4] (NULL:
     // the forward kept the j = k triplets, nothing to do)
     cx<double>* dgs;
 };
 
+// far(far_arg) launches the bins beyond nb_pairs (nullptr: none)
 cudaError_t launch_moments_adjoint_f32(const AdjArgs<float>& a, int64_t n, const int* perm, const float* g1,
                                        const float* g2, const float* w, float* dg1, float* dg2, float* dw,
-                                       int n_sm, cudaStream_t st);
+                                       int n_sm, cudaStream_t st, cudaError_t (*far)(void*), void* far_arg);
 cudaError_t launch_moments_adjoint_f64(const AdjArgs<double>& a, int64_t n, const int* perm, const float* g1,
                                        const float* g2, const float* w, float* dg1, float* dg2, float* dw,
                                        int n_sm, cudaStream_t st);

@@ -67,6 +67,39 @@ __device__ __forceinline__ constexpr int bit_reverse(int i, int bits)
     return r;
 }
 
+// complex FFT of N = 2^BITS points in registers, sum_j z_j e^{SIGN 2 pi i j k / N}; input in bit-reversed
+// order
+template <int BITS, int SIGN>
+__device__ __forceinline__ void complex_fft(float (&re)[1 << BITS], float (&im)[1 << BITS])
+{
+    constexpr int N = 1 << BITS;
+#pragma unroll
+    for (int st = 0; st < BITS; ++st) {
+        const int h = 1 << st;
+#pragma unroll
+        for (int b = 0; b < N / 2; ++b) {
+            const int j = b & (h - 1), i0 = ((b >> st) << (st + 1)) + j, i1 = i0 + h;
+            const int k = j * (32 >> st);  // twiddle e^{2 pi i j / (2 h)} as a 64th root
+            const float c = cos64(k), s = SIGN * sin64(k);
+            float tr, ti;
+            if (k == 0) {
+                tr = re[i1];
+                ti = im[i1];
+            } else if (k == 16) {
+                tr = -SIGN * im[i1];
+                ti = SIGN * re[i1];
+            } else {
+                tr = re[i1] * c - im[i1] * s;
+                ti = re[i1] * s + im[i1] * c;
+            }
+            re[i1] = re[i0] - tr;
+            im[i1] = im[i0] - ti;
+            re[i0] += tr;
+            im[i0] += ti;
+        }
+    }
+}
+
 // F_k = sum_s x_s e^{+2 pi i k s / S} of a real series, in registers: Re F_k at x[k] (k <= S/2),
 // Im F_k at x[S - k] (0 < k < S/2). A complex FFT of the even and odd samples as real and imaginary
 // parts, then the usual separation.
@@ -81,31 +114,7 @@ __device__ __forceinline__ void real_fft(float (&x)[S])
         re[j] = x[2 * bit_reverse(j, BITS)];
         im[j] = x[2 * bit_reverse(j, BITS) + 1];
     }
-#pragma unroll
-    for (int st = 0; st < BITS; ++st) {
-        const int h = 1 << st;
-#pragma unroll
-        for (int b = 0; b < N / 2; ++b) {
-            const int j = b & (h - 1), i0 = ((b >> st) << (st + 1)) + j, i1 = i0 + h;
-            const int k = j * (32 >> st);  // twiddle e^{2 pi i j / (2 h)} as a 64th root
-            const float c = cos64(k), s = sin64(k);
-            float tr, ti;
-            if (k == 0) {
-                tr = re[i1];
-                ti = im[i1];
-            } else if (k == 16) {
-                tr = -im[i1];
-                ti = re[i1];
-            } else {
-                tr = re[i1] * c - im[i1] * s;
-                ti = re[i1] * s + im[i1] * c;
-            }
-            re[i1] = re[i0] - tr;
-            im[i1] = im[i0] - ti;
-            re[i0] += tr;
-            im[i0] += ti;
-        }
-    }
+    complex_fft<BITS, 1>(re, im);
     x[0] = re[0] + im[0];
     x[N] = re[0] - im[0];
 #pragma unroll
@@ -121,6 +130,45 @@ __device__ __forceinline__ void real_fft(float (&x)[S])
             x[N - k] = er - wr;
             x[S - (N - k)] = wi - ei;
         }
+    }
+}
+
+// the transpose of real_fft: from r_k = x[k] (k <= S/2) and i_k = x[S - k] (0 < k < S/2) to
+// x_s = sum_k r_k cos(2 pi k s / S) + i_k sin(2 pi k s / S)
+template <int S>
+__device__ __forceinline__ void real_fft_adjoint(float (&x)[S])
+{
+    constexpr int N = S / 2;
+    constexpr int BITS = S == 64 ? 5 : S == 32 ? 4 : 3;
+    // the Hermitian spectrum Y_k = (r_k + i i_k) / 2 folded to N points whose transform has x_{2j} as real
+    // and x_{2j+1} as imaginary part: C_k = Y_k + Y*_{N-k} + i e^{-2 pi i k / S} (Y_k - Y*_{N-k})
+    float cr[N], ci[N], re[N], im[N];
+    cr[0] = x[0] + x[N];
+    ci[0] = x[0] - x[N];
+#pragma unroll
+    for (int k = 1; k <= N / 2; ++k) {
+        const float ar = 0.5f * x[k], ai = 0.5f * x[S - k];
+        const float br = 0.5f * x[N - k], bi = -0.5f * x[S - (N - k)];
+        const float sr = ar + br, si = ai + bi, dr = ar - br, di = ai - bi;
+        const float c = cos64(k * (64 / S)), s = sin64(k * (64 / S));
+        const float tr = dr * s - di * c, ti = dr * c + di * s;  // i e^{-i theta k} d
+        cr[k] = sr + tr;
+        ci[k] = si + ti;
+        if (k < N / 2) {
+            cr[N - k] = sr - tr;
+            ci[N - k] = ti - si;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        re[j] = cr[bit_reverse(j, BITS)];
+        im[j] = ci[bit_reverse(j, BITS)];
+    }
+    complex_fft<BITS, -1>(re, im);
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        x[2 * j] = re[j];
+        x[2 * j + 1] = im[j];
     }
 }
 
@@ -170,6 +218,52 @@ struct Sums {
     }
 };
 
+// the adjoint of Sums: dL/d(sum) of a sector as the coefficients of Chebyshev series in u, whose values at
+// a member are dL/d(w gamma_1), dL/d(w gamma_2) and dL/dw (signs as in Sums)
+template <int PW, int PAB>
+struct Series {
+    float2 w[PW / 2], a[PAB / 2], b[PAB / 2];
+
+    __device__ __forceinline__ void load(const float* m, bool on)
+    {
+        auto get = [&](int base, int j) {
+            const float s = (j & 2) ? -1.f : 1.f;
+            return on ? make_float2(s * m[(base + 2 * j) * kC], s * m[(base + 2 * j + 1) * kC]) : make_float2(0.f, 0.f);
+        };
+#pragma unroll
+        for (int j = 0; j < PW / 2; ++j) w[j] = get(0, j);
+#pragma unroll
+        for (int j = 0; j < PAB / 2; ++j) {
+            a[j] = get(PW, j);
+            b[j] = get(PW + PAB, j);
+        }
+    }
+
+    __device__ __forceinline__ void eval(float u, float& av, float& bv, float& wv) const
+    {
+        const float t2 = fmaf(2.f * u, u, -1.f), k = 2.f * t2;
+        float2 v0 = make_float2(1.f, u), v1 = make_float2(t2, fmaf(k, u, -u));
+        const float2 kp = make_float2(k, k), km = make_float2(-k, -k);
+        float2 sa = make_float2(0.f, 0.f), sb = sa, sw = sa;
+#pragma unroll
+        for (int j = 0; j < PW / 2; ++j) {
+            if (j < PAB / 2) {
+                sa = __ffma2_rn(a[j], v0, sa);
+                sb = __ffma2_rn(b[j], v0, sb);
+            }
+            sw = __ffma2_rn(w[j], v0, sw);
+            if (j + 1 < PW / 2) {
+                const float2 v2 = __ffma2_rn((j & 1) ? kp : km, v1, v0);
+                v0 = v1;
+                v1 = v2;
+            }
+        }
+        av = sa.x + sa.y;
+        bv = sb.x + sb.y;
+        wv = sw.x + sw.y;
+    }
+};
+
 // p[i] by a 32-bit byte offset (the caller keeps the arrays below 4 GB): the 64-bit multiply-add of
 // the usual address runs on the FP64 pipe
 template <typename U>
@@ -185,7 +279,51 @@ __device__ __forceinline__ float rsqrt_approx(float x)
     return y;
 }
 
-template <class PL>
+// the candidates of a sector in batches of up to kQueue, listed in row order: batch(n) is called by the
+// whole warp with their indexes in queue[0 .. n)
+template <typename F>
+__device__ __forceinline__ void sector_batches(const SectorGeom& g, bool upper, bool first, bool last, float ct0, float ct1,
+                                               float sn0, float sn1, const int* __restrict__ row_start, int* queue,
+                                               int lane, F&& batch)
+{
+    constexpr unsigned FULL = 0xffffffffu;
+    float iy0, iy1;
+    sector_rows(g, upper, sn0, sn1, iy0, iy1);
+    for (float iy = iy0 + (float)lane; iy - (float)lane <= iy1; iy += 32.0f) {
+        int st0 = 0, n0 = 0, st1 = 0, n1 = 0;
+        if (iy <= iy1) sector_runs(g, upper, first, last, ct0, ct1, iy, row_start, st0, n0, st1, n1);
+        while (true) {
+            const int len = n0 + n1;
+            int incl = len;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(FULL, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const int total = __shfl_sync(FULL, incl, 31);
+            if (total == 0) break;
+            const int off = incl - len;
+            const int put = max(0, min(len, kQueue - off));
+            for (int j = 0; j < put; ++j) queue[off + j] = j < n0 ? st0 + j : st1 + (j - n0);
+            const int t0 = min(put, n0);
+            st0 += t0;
+            n0 -= t0;
+            st1 += put - t0;
+            n1 -= put - t0;
+            __syncwarp();
+            batch(min(total, kQueue));
+            __syncwarp();
+            if (total <= kQueue) break;
+        }
+    }
+}
+
+// ADJ: the transposed chain. m.G and m.W hold dL/dG and dL/dW; the transposes of the order sums and of
+// the FFT give dL/dM_{s,p}, and every member of a sector gets the value of the Chebyshev series with these
+// coefficients, summed over the group's centres before one atomic addition per component to A.gvw
+// (the block-per-centre form evaluates the 2 n_max + 3 and 2 n_max + 1 orders per pair, about 500 FMAs, and adds
+// every pair atomically).
+template <class PL, bool ADJ>
 __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs A)
 {
     constexpr int S = PL::S, PW = PL::PW, PAB = PL::PAB, PT = PL::PT, KS = PL::KS;
@@ -268,44 +406,131 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
                 if (tid == 0) s_next = kWarps;
                 __syncthreads();
 
-                // ---- sums of the sectors
+                if constexpr (ADJ) {
+                    // ---- transposed order sums: thread (centre, k) adds the orders m = +-k mod S
+                    const int c8 = tid & (kC - 1);
+                    const size_t at = ((size_t)s_row[c8] * nz + z) * m.nbp + b;
+                    const int mtop = max(2 * n_max, n_max + 3);
+                    const float on = (act >> c8) & 1u ? 1.f : 0.f;
+                    for (int k = tid / kC; k <= S / 2; k += kThreads / kC) {
+                        float* Fr = M + k * KS + c8;
+                        float* Fi = M + ((S - k) & (S - 1)) * KS + c8;
+                        const bool edge = k == 0 || k == S / 2;
+                        for (int p = 0; p < PT; ++p) {
+                            Fr[p * kC] = 0.f;
+                            if (!edge) Fi[p * kC] = 0.f;
+                        }
+                        for (int j = 0; j * S - k <= mtop; ++j)
+                            for (int h = edge ? 1 : 0; h < 2; ++h) {
+                                const int mm = h ? j * S + k : j * S - k;
+                                if (mm < 0 || mm > mtop || on == 0.f) continue;
+                                const float fi = edge ? 0.f : h ? 1.f : -1.f;
+                                const float* cm = coef + mm * PW;
+                                const float2 ro = rot[mm];
+                                auto order = [&](int base, int P, cx<float> g) {
+                                    const float vr = g.x * ro.x + g.y * ro.y, vi = g.y * ro.x - g.x * ro.y;
+#pragma unroll 4
+                                    for (int p = 0; p < P; p += 2) {
+                                        const float ca = cm[p], cb = cm[p + 1];
+                                        Fr[(base + p) * kC] += ca * vr;
+                                        Fr[(base + p + 1) * kC] += cb * vi;
+                                        if (!edge) {
+                                            Fi[(base + p) * kC] += fi * ca * vi;
+                                            Fi[(base + p + 1) * kC] -= fi * cb * vr;
+                                        }
+                                    }
+                                };
+                                if (mm <= 2 * n_max) order(0, PW, m.W[(size_t)mm * plane + at]);
+                                if (mm <= n_max + 3) {
+                                    cx<float> ga{0.f, 0.f}, gb{0.f, 0.f};
+                                    if (mm <= n_max - 1) {
+                                        const cx<float> y = m.G[(size_t)(mm + n_max + 3) * plane + at];
+                                        ga = y;
+                                        gb = cx<float>{y.y, -y.x};
+                                    }
+                                    if (mm >= 1) {
+                                        const cx<float> y = m.G[(size_t)(n_max + 3 - mm) * plane + at];
+                                        ga = cx<float>{ga.x + y.x, ga.y - y.y};
+                                        gb = cx<float>{gb.x + y.y, gb.y + y.x};
+                                    }
+                                    order(PW, PAB, ga);
+                                    order(PW + PAB, PAB, gb);
+                                }
+                            }
+                    }
+                    __syncthreads();
+                    for (int q = tid; q < PT * kC; q += kThreads) {
+                        float x[S];
+#pragma unroll
+                        for (int s = 0; s < S; ++s) x[s] = M[s * KS + q];
+                        real_fft_adjoint<S>(x);
+#pragma unroll
+                        for (int s = 0; s < S; ++s) M[s * KS + q] = x[s];
+                    }
+                    __syncthreads();
+                }
+
+                // ---- the sectors: sums of their members, or the members' gradients
                 for (int s = warp; s < S;) {
                     const bool upper = s < S / 2;
                     const int sp = upper ? s : s - S / 2;
                     const float4 ax = axis[s];  // (cos, sin) / sin(delta_max), angle offset of the rounded axis
-                    const float ct0 = ray[sp], ct1 = ray[sp + 1];
-                    float iy0, iy1;
-                    sector_rows(g, upper, A.table[A.off_sin + 2 * sp], A.table[A.off_sin + 2 * sp + 1], iy0, iy1);
-                    Sums<PW, PAB> sum;
-                    sum.reset();
-                    int count = 0, maybe = 0;
-                    for (float iy = iy0 + (float)lane; iy - (float)lane <= iy1; iy += 32.0f) {
-                        int st0 = 0, n0 = 0, st1 = 0, n1 = 0;
-                        if (iy <= iy1)
-                            sector_runs(g, upper, sp == 0, sp == S / 2 - 1, ct0, ct1, iy, row_start, st0, n0, st1, n1);
-                        while (true) {
-                            // list the rows' candidates in row order
-                            const int len = n0 + n1;
-                            int incl = len;
-#pragma unroll
-                            for (int o = 1; o < 32; o <<= 1) {
-                                const int y = __shfl_up_sync(FULL, incl, o);
-                                if (lane >= o) incl += y;
+                    const float sn0 = A.table[A.off_sin + 2 * sp], sn1 = A.table[A.off_sin + 2 * sp + 1];
+                    int* qu = queue[warp];
+                    if constexpr (ADJ) {
+                        Series<PW, PAB> ser;
+                        ser.load(M + s * KS + ce, mine);
+                        auto add = [&](int i, bool in, float u) {
+                            float a, b, w;
+                            ser.eval(u, a, b, w);
+                            a = in ? a : 0.f;
+                            b = in ? b : 0.f;
+                            w = in ? w : 0.f;
+                            // over the eight centres (lane bits 0..2), ending with a, b or w in a lane
+                            const bool u2 = (lane & 4) != 0, u1 = (lane & 2) != 0;
+                            const float r0 = __shfl_xor_sync(FULL, u2 ? a : w, 4), r1 = __shfl_xor_sync(FULL, u2 ? b : 0.f, 4);
+                            const float k0 = (u2 ? w : a) + r0, k1 = (u2 ? 0.f : b) + r1;
+                            float v = (u1 ? k1 : k0) + __shfl_xor_sync(FULL, u1 ? k0 : k1, 2);
+                            v += __shfl_xor_sync(FULL, v, 1);
+                            if (!(lane & 1) && v != 0.f) atomicAdd(A.gvw + 4 * (size_t)i + (u2 ? 2 : u1 ? 1 : 0), v);
+                        };
+                        sector_batches(g, upper, sp == 0, sp == S / 2 - 1, ray[sp], ray[sp + 1], sn0, sn1, row_start, qu, lane,
+                                       [&](int n) {
+                            int i0 = qu[min(sub, n - 1)], i1 = qu[min(sub + kSub, n - 1)];
+                            float2 p0 = at32(A.posf, i0), p1 = at32(A.posf, i1);
+                            int odd = 0;
+                            for (int t = sub; t < n + sub; t += kSub) {
+                                const float2 p = p0;
+                                const int i = i0;
+                                p0 = p1;
+                                i0 = i1;
+                                i1 = qu[min(t + 2 * kSub, n - 1)];
+                                p1 = at32(A.posf, i1);
+                                const float dx = p.x - pc.x, dy = p.y - pc.y;  // exact
+                                const float r2 = fmaf(dx, dx, dy * dy), d = fabsf(r2 - mid);
+                                const bool in = d < d_in && t < n;
+                                odd += d < d_out && t < n && !in ? 1 : 0;
+                                add(i, in && mine, fmaf(fmaf(dy, ax.x, -dx * ax.y), rsqrt_approx(r2), ax.z));
                             }
-                            const int total = __shfl_sync(FULL, incl, 31);
-                            if (total == 0) break;
-                            const int off = incl - len;
-                            const int put = max(0, min(len, kQueue - off));
-                            for (int j = 0; j < put; ++j) queue[warp][off + j] = j < n0 ? st0 + j : st1 + (j - n0);
-                            const int t0 = min(put, n0);
-                            st0 += t0;
-                            n0 -= t0;
-                            st1 += put - t0;
-                            n1 -= put - t0;
-                            const int n = min(total, kQueue);
-                            __syncwarp();
+                            if (__any_sync(FULL, odd))  // rare: the candidates near an edge, by the integers
+                                for (int t = sub; t < n + sub; t += kSub) {
+                                    const int i = qu[min(t, n - 1)];
+                                    const float2 p = at32(A.posf, i);
+                                    const float dx = p.x - pc.x, dy = p.y - pc.y;
+                                    const float r2 = fmaf(dx, dx, dy * dy), d = fabsf(r2 - mid);
+                                    const long long q2 = (long long)(int)dx * (int)dx + (long long)(int)dy * (int)dy;
+                                    const bool in = d < d_out && !(d < d_in) && t < n && q2 >= bg->e0 && q2 < bg->e1;
+                                    add(i, in && mine, fmaf(fmaf(dy, ax.x, -dx * ax.y), rsqrt_approx(r2), ax.z));
+                                }
+                        });
+                    } else {
+                        Sums<PW, PAB> sum;
+                        sum.reset();
+                        int count = 0, maybe = 0;
+                        sector_batches(g, upper, sp == 0, sp == S / 2 - 1, ray[sp], ray[sp + 1], sn0, sn1, row_start, qu, lane,
+                                       [&](int n) {
                             // candidates sub, sub + 4, ...: two loads ahead of the arithmetic
-                            int i0 = queue[warp][min(sub, n - 1)], i1 = queue[warp][min(sub + kSub, n - 1)];
+                            int i0 = qu[min(sub, n - 1)], i1 = qu[min(sub + kSub, n - 1)];
                             float2 p0 = at32(A.posf, i0), p1 = at32(A.posf, i1);
                             Pay<float> v0 = at32(m.pay, i0), v1 = at32(m.pay, i1);
                             for (int t = sub; t < n + sub; t += kSub) {
@@ -313,7 +538,7 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
                                 const Pay<float> v = v0;
                                 p0 = p1;
                                 v0 = v1;
-                                i1 = queue[warp][min(t + 2 * kSub, n - 1)];
+                                i1 = qu[min(t + 2 * kSub, n - 1)];
                                 p1 = at32(A.posf, i1);
                                 v1 = at32(m.pay, i1);
                                 const float dx = p.x - pc.x, dy = p.y - pc.y;  // exact
@@ -327,8 +552,8 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
                             if (__any_sync(FULL, maybe != count)) {
                                 // rare: the candidates near an edge, by the integers
                                 for (int t = sub; t < n; t += kSub) {
-                                    const float2 p = at32(A.posf, queue[warp][t]);
-                                    const Pay<float> v = at32(m.pay, queue[warp][t]);
+                                    const float2 p = at32(A.posf, qu[t]);
+                                    const Pay<float> v = at32(m.pay, qu[t]);
                                     const float dx = p.x - pc.x, dy = p.y - pc.y;
                                     const float r2 = fmaf(dx, dx, dy * dy), d = fabsf(r2 - mid);
                                     if (!(d < d_out) || d < d_in) continue;
@@ -339,33 +564,32 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
                                 }
                                 maybe = count;
                             }
-                            __syncwarp();
-                            if (total <= kQueue) break;
+                        });
+                        if (mine) my_pairs += (unsigned long long)count;
+                        // reduce over the four streams, each keeping a quarter of the terms
+                        constexpr int Q = (PT + 3) / 4;
+                        float h[2 * Q];
+#pragma unroll
+                        for (int i = 0; i < 2 * Q; ++i) {
+                            const float lo = sum.value(i), hi = i + 2 * Q < PT ? sum.value(i + 2 * Q) : 0.f;
+                            const bool up = (sub & 2) != 0;
+                            h[i] = (up ? hi : lo) + __shfl_xor_sync(FULL, up ? lo : hi, 2 * kC);
                         }
-                    }
-                    if (mine) my_pairs += (unsigned long long)count;
-                    // reduce over the four streams, each keeping a quarter of the terms
-                    constexpr int Q = (PT + 3) / 4;
-                    float h[2 * Q];
+                        float* out = M + s * KS + ce;
 #pragma unroll
-                    for (int i = 0; i < 2 * Q; ++i) {
-                        const float lo = sum.value(i), hi = i + 2 * Q < PT ? sum.value(i + 2 * Q) : 0.f;
-                        const bool up = (sub & 2) != 0;
-                        h[i] = (up ? hi : lo) + __shfl_xor_sync(FULL, up ? lo : hi, 2 * kC);
-                    }
-                    float* out = M + s * KS + ce;
-#pragma unroll
-                    for (int i = 0; i < Q; ++i) {
-                        const bool up = (sub & 1) != 0;
-                        const float v = (up ? h[i + Q] : h[i]) + __shfl_xor_sync(FULL, up ? h[i] : h[i + Q], kC);
-                        const int p = (sub >> 1) * 2 * Q + (sub & 1) * Q + i;
-                        if (p < PT) out[p * kC] = v;
+                        for (int i = 0; i < Q; ++i) {
+                            const bool up = (sub & 1) != 0;
+                            const float v = (up ? h[i + Q] : h[i]) + __shfl_xor_sync(FULL, up ? h[i] : h[i + Q], kC);
+                            const int p = (sub >> 1) * 2 * Q + (sub & 1) * Q + i;
+                            if (p < PT) out[p * kC] = v;
+                        }
                     }
                     int nx = 0;
                     if (lane == 0) nx = atomicAdd(&s_next, 1);
                     s = __shfl_sync(FULL, nx, 0);
                 }
                 __syncthreads();
+                if constexpr (ADJ) continue;
 
                 // ---- FFT over the sectors of every (term, centre)
                 for (int q = tid; q < PT * kC; q += kThreads) {
@@ -379,9 +603,9 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
                 __syncthreads();
 
                 // ---- the orders: thread (centre, m)
-                const int c8 = tid & (kC - 1), row = s_row[c8];
+                const int c8 = tid & (kC - 1);
                 if ((act >> c8) & 1u) {
-                    const size_t at = ((size_t)row * nz + z) * m.nbp + b;
+                    const size_t at = ((size_t)s_row[c8] * nz + z) * m.nbp + b;
                     const int mtop = max(2 * n_max, n_max + 3);
                     for (int mm = tid / kC; mm <= mtop; mm += kThreads / kC) {
                         int k = mm & (S - 1);
@@ -427,19 +651,19 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
     if (lane == 0 && my_pairs) atomicAdd(m.pairs, my_pairs);
 }
 
-template <class PL>
+template <class PL, bool ADJ>
 static cudaError_t launch(const FarArgs& a, int n_sm, cudaStream_t st)
 {
     const size_t smem = sizeof(float) * PL::S * PL::KS;
-    cudaError_t e = set_smem_attr(far_moments_kernel<PL>, smem);
+    cudaError_t e = set_smem_attr(far_moments_kernel<PL, ADJ>, smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = occupancy(&per_sm, far_moments_kernel<PL>, kThreads, smem);
+    e = occupancy(&per_sm, far_moments_kernel<PL, ADJ>, kThreads, smem);
     if (e != cudaSuccess) return e;
     const int64_t items = (int64_t)((a.m.n_centres + kC - 1) / kC) * a.parts;
     const int64_t grid = std::min<int64_t>(items, (int64_t)n_sm * std::max(per_sm, 1));
     if (grid < 1) return cudaSuccess;
-    far_moments_kernel<PL><<<(unsigned)grid, kThreads, smem, st>>>(a);
+    far_moments_kernel<PL, ADJ><<<(unsigned)grid, kThreads, smem, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -543,9 +767,18 @@ void far_tables(int n_max, FarTables (&t)[kFarPlans], std::vector<float>* v)
 cudaError_t launch_moments_far(const FarArgs& a, int plan, int n_sm, cudaStream_t st)
 {
     switch (plan) {
-        case 0: return far::launch<far::Wide>(a, n_sm, st);
-        case 1: return far::launch<far::Middle>(a, n_sm, st);
-        default: return far::launch<far::Close>(a, n_sm, st);
+        case 0: return far::launch<far::Wide, false>(a, n_sm, st);
+        case 1: return far::launch<far::Middle, false>(a, n_sm, st);
+        default: return far::launch<far::Close, false>(a, n_sm, st);
+    }
+}
+
+cudaError_t launch_moments_far_adjoint(const FarArgs& a, int plan, int n_sm, cudaStream_t st)
+{
+    switch (plan) {
+        case 0: return far::launch<far::Wide, true>(a, n_sm, st);
+        case 1: return far::launch<far::Middle, true>(a, n_sm, st);
+        default: return far::launch<far::Close, true>(a, n_sm, st);
     }
 }
 

@@ -36,9 +36,12 @@ struct FarArgs {
     const float* table;
     int off_ray, off_sin, off_axis, off_rot, off_coef;
     unsigned long long* queue;  // items claimed beyond the first gridDim.x (zero at launch)
+    float* gvw;                 // adjoint: the gradient slots of AdjArgs (m.G, m.W: dL/dG, dL/dW)
 };
 
 cudaError_t launch_moments_far(const FarArgs& a, int plan, int n_sm, cudaStream_t st);
+
+cudaError_t launch_moments_far_adjoint(const FarArgs& a, int plan, int n_sm, cudaStream_t st);
 
 template <typename T>
 struct NearArgs {
