@@ -28,7 +28,8 @@
 
 #include <algorithm>
 
-#include "common.cuh"
+#include "moments_far.cuh"
+#include "sector.cuh"
 
 namespace mp3 {
 
@@ -278,21 +279,6 @@ __global__ void __launch_bounds__(kCoefWarps * 32) contract_adjoint_coef(const A
 
 // ------------------------------------------------------------------ stage (a): pair loop
 
-__device__ __forceinline__ long long isqrt_floor(long long v)
-{
-    if (v <= 0) return 0;
-    long long r = (long long)sqrt((double)v);
-    while (r * r > v) --r;
-    while ((r + 1) * (r + 1) <= v) ++r;
-    return r;
-}
-
-__device__ __forceinline__ long long fdiv(long long a, long long b)
-{
-    const long long q = a / b;
-    return (a % b != 0 && ((a < 0) != (b < 0))) ? q - 1 : q;
-}
-
 // adds (re grad v, im grad v, grad w) to a galaxy's 16-byte (FP32) or 32-byte (FP64) slot
 __device__ __forceinline__ void atomic_add_vw(float* p, float vr, float vi, float w)
 {
@@ -306,16 +292,15 @@ __device__ __forceinline__ void atomic_add_vw(double* p, double vr, double vi, d
 }
 
 template <typename T>
-__device__ __forceinline__ cx<T> unit_dir(long long dx, long long dy);
+__device__ __forceinline__ cx<T> unit_dir(float dx, float dy);
 template <>
-__device__ __forceinline__ cx<float> unit_dir<float>(long long dx, long long dy)
+__device__ __forceinline__ cx<float> unit_dir<float>(float dx, float dy)
 {
-    const float fx = (float)dx, fy = (float)dy;
-    const float ir = rsqrtf(fx * fx + fy * fy);
-    return {fx * ir, fy * ir};
+    const float ir = rsqrtf(dx * dx + dy * dy);
+    return {dx * ir, dy * ir};
 }
 template <>
-__device__ __forceinline__ cx<double> unit_dir<double>(long long dx, long long dy)
+__device__ __forceinline__ cx<double> unit_dir<double>(float dx, float dy)
 {
     const double fx = (double)dx, fy = (double)dy;
     const double ir = 1.0 / sqrt(fx * fx + fy * fy);
@@ -331,62 +316,69 @@ __device__ __forceinline__ cx<T> horner_step(cx<T> p, cx<T> x, cx<T> c)
     return {fma(p.x, x.x, fma(-p.y, x.y, c.x)), fma(p.x, x.y, fma(p.y, x.x, c.y))};
 }
 
-// Walks the candidates of redshift bin z around the centre (px, py): the warp goes row by row of
-// the cell grid over the one or two runs of cells that meet the annulus (cells wholly inside the
-// inner radius are skipped), 32 candidates at a time, one per lane, and calls f(in, k, dx, dy) on
-// every lane of the warp at every step (warp-uniform), with in = whether galaxy k's squared
-// separation r2 lies in [r2lo, r2hi). Must be called by the whole warp.
-template <typename F>
-__device__ __forceinline__ void for_each_in_annulus(const GridDesc& g, const int32_t* __restrict__ cell_start,
-                                                    const int2* __restrict__ pos, long long px, long long py,
-                                                    long long r2lo, long long r2hi, int z, int lane, F&& f)
+constexpr int kList = 128;  // candidates listed at a time per warp
+
+// Walks the candidates of redshift bin z around the centre at pc (from the grid's origin): the lanes find
+// the one or two runs of cells of 32 cell rows at a time that meet bin b's annulus (annulus_runs), the
+// candidates are listed in row order in the warp's list, and f(in, k, dx, dy) is called on every lane for
+// 32 of them at a time (warp-uniform), with in = whether galaxy k is in the bin (decided on the integers
+// near an edge). Must be called by the whole warp. A walk over one row at a time with 64-bit
+// divisions took about 1500 instructions a row, most of the time of the narrow bins.
+template <typename T, typename F>
+__device__ __forceinline__ void for_each_in_annulus(const AdjArgs<T>& a, float2 pc, int b, int z, int lane, int* list, F&& f)
 {
-    const long long R = isqrt_floor(r2hi - 1);
-    const long long ya = max(0LL, fdiv(py - R - g.y0, g.side));
-    const long long yb = min((long long)g.ncy - 1, fdiv(py + R - g.y0, g.side));
-    for (long long yy = ya; yy <= yb; ++yy) {
-        const long long ylo = g.y0 + yy * g.side, yhi = ylo + g.side - 1;
-        const long long dymin = max(0LL, max(ylo - py, py - yhi));
-        const long long dymax = max(llabs(ylo - py), llabs(yhi - py));
-        if (dymin * dymin > r2hi - 1) continue;
-        const long long dxo = isqrt_floor(r2hi - 1 - dymin * dymin);
-        long long ca = fdiv(px - dxo - g.x0, g.side), cb = fdiv(px + dxo - g.x0, g.side);
-        if (cb < 0 || ca > g.ncx - 1) continue;
-        ca = max(ca, 0LL);
-        cb = min(cb, (long long)g.ncx - 1);
-        long long cl = cb + 1, cr = cb;
-        if (r2lo - 1 - dymax * dymax >= 0) {
-            const long long hx = isqrt_floor(r2lo - 1 - dymax * dymax);
-            cl = -fdiv(-(px - hx - g.x0), g.side);      // first cell starting at >= px - hx
-            cr = fdiv(px + hx - g.x0 + 1, g.side) - 1;  // last cell ending at <= px + hx
-        }
-        long long segs[2][2];
-        int nseg = 0;
-        if (cl <= cr && cl <= cb && cr >= ca) {
-            if (ca <= cl - 1) { segs[nseg][0] = ca; segs[nseg][1] = cl - 1; ++nseg; }
-            if (cr + 1 <= cb) { segs[nseg][0] = cr + 1; segs[nseg][1] = cb; ++nseg; }
-        } else {
-            segs[0][0] = ca;
-            segs[0][1] = cb;
-            nseg = 1;
-        }
-        const size_t key0 = (size_t)z * g.ncells + (size_t)yy * g.ncx;
-        for (int sgi = 0; sgi < nseg; ++sgi) {
-            const int k0 = cell_start[key0 + segs[sgi][0]];
-            const int k1 = cell_start[key0 + segs[sgi][1] + 1];
-            for (int kb = k0; kb < k1; kb += 32) {
-                const int k = kb + lane;
-                long long dx = 0, dy = 0;
-                bool in = false;
-                if (k < k1) {
-                    const int2 qk = pos[k];
-                    dx = (long long)qk.x - px;
-                    dy = (long long)qk.y - py;
-                    const long long r2 = dx * dx + dy * dy;
-                    in = r2 >= r2lo && r2 < r2hi;
-                }
-                f(in, k, dx, dy);
+    constexpr unsigned FULL = 0xffffffffu;
+    const BinGeom* bg = a.bins + b;
+    SectorGeom g;
+    g.gx = pc.x;
+    g.gy = pc.y;
+    g.hx = g.hy = 0.0f;
+    g.Ri = bg->Ri;
+    g.Ro = bg->Ro;
+    g.S = (float)a.g.side;
+    g.iS = 1.0f / g.S;
+    g.ncx = a.g.ncx;
+    g.ncy = a.g.ncy;
+    const float mid = bg->mid, d_in = bg->d_in, d_out = bg->d_out;
+    const int* row_start = a.cell_start + (size_t)z * a.g.ncells;
+    const float ro = g.Ro + 8.0f;
+    const float iy0 = fmaxf(floorf((g.gy - ro) * g.iS), 0.0f), iy1 = fminf(floorf((g.gy + ro) * g.iS), (float)(g.ncy - 1));
+    for (float iy = iy0 + (float)lane; iy - (float)lane <= iy1; iy += 32.0f) {
+        int st0 = 0, n0 = 0, st1 = 0, n1 = 0;
+        if (iy <= iy1) annulus_runs(g, iy, (iy + 0.5f) * g.S - g.gy, 0, g.ncx - 1, row_start, st0, n0, st1, n1);
+        while (true) {
+            const int len = n0 + n1;
+            int incl = len;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(FULL, incl, o);
+                if (lane >= o) incl += y;
             }
+            const int total = __shfl_sync(FULL, incl, 31);
+            if (total == 0) break;
+            const int off = incl - len, put = max(0, min(len, kList - off));
+            for (int j = 0; j < put; ++j) list[off + j] = j < n0 ? st0 + j : st1 + (j - n0);
+            const int t0 = min(put, n0);
+            st0 += t0;
+            n0 -= t0;
+            st1 += put - t0;
+            n1 -= put - t0;
+            const int n = min(total, kList);
+            __syncwarp();
+            for (int t = lane; t < n + lane; t += 32) {
+                const int k = list[min(t, n - 1)];
+                const float2 p = a.posf[k];
+                const float dx = p.x - pc.x, dy = p.y - pc.y;  // exact
+                const float d = fabsf(fmaf(dx, dx, dy * dy) - mid);
+                bool in = d < d_in;
+                if (!in && d < d_out) {
+                    const long long q2 = (long long)(int)dx * (int)dx + (long long)(int)dy * (int)dy;
+                    in = q2 >= bg->e0 && q2 < bg->e1;
+                }
+                f(in && t < n, k, dx, dy);
+            }
+            __syncwarp();
+            if (total <= kList) break;
         }
     }
 }
@@ -403,6 +395,7 @@ __global__ void __launch_bounds__(kPairWarps * 32) moments_adjoint_pairs(const A
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nb = a.nb, nz = a.nz, nmax = a.n_max, nbp = nb_pad(nb);
     const int MG = 2 * nmax + 3, MW = 2 * nmax + 1, o = nmax + 3;
+    __shared__ int list[kPairWarps][kList];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned lt_mask = (1u << lane) - 1u;
     cx<T>* co = reinterpret_cast<cx<T>*>(smem_raw) + (size_t)warp * nz * (MG + MW);  // [z][MG + MW]
@@ -412,7 +405,7 @@ __global__ void __launch_bounds__(kPairWarps * 32) moments_adjoint_pairs(const A
     const size_t plane = (size_t)a.n_centres * nz * nbp;
     for (int c = blockIdx.x * kPairWarps + warp; c < a.n_centres; c += gridDim.x * kPairWarps) {
         const int d = a.centre_idx[c];
-        const int2 p = a.pos[d];
+        const float2 p = a.posf[d];
         for (int b = 0; b < a.nb_pairs; ++b) {
             __syncwarp();
             for (int i = lane; i < nz * (MG + MW); i += 32) {
@@ -446,8 +439,8 @@ __global__ void __launch_bounds__(kPairWarps * 32) moments_adjoint_pairs(const A
                     atomic_add_vw(a.gvw + 4 * (size_t)k, P.x + Q.x, P.y + Q.y, Rw.x);
                 };
                 int qn = 0;  // queued members (warp-uniform), < 32 between steps
-                for_each_in_annulus(a.g, a.cell_start, a.pos, p.x, p.y, a.e2q[b], a.e2q[b + 1], z, lane,
-                                    [&](bool in, int k, long long dx, long long dy) {
+                for_each_in_annulus(a, p, b, z, lane, list[warp],
+                                    [&](bool in, int k, float dx, float dy) {
                     const unsigned m = __ballot_sync(0xffffffffu, in);
                     if (in) {
                         const int slot = qn + __popc(m & lt_mask);
@@ -509,14 +502,15 @@ template <typename T>
 __global__ void __launch_bounds__(kPairWarps * 32) degenerate_moments(const AdjArgs<T> a, cx<T>* __restrict__ out)
 {
     const int nb = a.nb, nz = a.nz;
+    __shared__ int list[kPairWarps][kList];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int c = blockIdx.x * kPairWarps + warp; c < a.n_centres; c += gridDim.x * kPairWarps) {
-        const int2 p = a.pos[a.centre_idx[c]];
+        const float2 p = a.posf[a.centre_idx[c]];
         for (int b = 0; b < nb; ++b)
             for (int z = 0; z < nz; ++z) {
                 T s[7] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
-                for_each_in_annulus(a.g, a.cell_start, a.pos, p.x, p.y, a.e2q[b], a.e2q[b + 1], z, lane,
-                                    [&](bool in, int k, long long dx, long long dy) {
+                for_each_in_annulus(a, p, b, z, lane, list[warp],
+                                    [&](bool in, int k, float dx, float dy) {
                     if (!in) return;
                     const cx<T> zz = unit_dir<T>(dx, dy);
                     const cx<T> u{zz.x, -zz.y};
@@ -635,10 +629,11 @@ template <typename T>
 __global__ void __launch_bounds__(kPairWarps * 32) degenerate_adjoint_pairs(const AdjArgs<T> a)
 {
     const int nb = a.nb, nz = a.nz;
+    __shared__ int list[kPairWarps][kList];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int c = blockIdx.x * kPairWarps + warp; c < a.n_centres; c += gridDim.x * kPairWarps) {
         const int d = a.centre_idx[c];
-        const int2 p = a.pos[d];
+        const float2 p = a.posf[d];
         const int z1 = a.zs ? (int)a.zs[d] : 0;
         const Pay<T> pv = a.pay[d];
         const cx<double> vi{(double)pv.a, (double)pv.b};
@@ -652,8 +647,8 @@ __global__ void __launch_bounds__(kPairWarps * 32) degenerate_adjoint_pairs(cons
                 const cx<double> gD6 = cmul(cconj(vi), gS0), gD2 = cmul(vi, gS1), gE2 = cmul(cconj(vi), gS2);
                 const double gF = wi * gSN;
                 double sd[7] = {0, 0, 0, 0, 0, 0, 0};  // this lane's share of D6, D2, E2, F
-                for_each_in_annulus(a.g, a.cell_start, a.pos, p.x, p.y, a.e2q[b], a.e2q[b + 1], z, lane,
-                                    [&](bool in, int k, long long dx, long long dy) {
+                for_each_in_annulus(a, p, b, z, lane, list[warp],
+                                    [&](bool in, int k, float dx, float dy) {
                     if (!in) return;
                     const cx<T> zz = unit_dir<T>(dx, dy);
                     const cx<double> u{(double)zz.x, -(double)zz.y};

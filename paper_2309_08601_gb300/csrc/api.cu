@@ -1734,7 +1734,8 @@ static AdjArgs<T> catalog_args(mp3pcf_ctx* ctx)
     a.nb = c.n_bins;
     a.n_max = c.n_max;
     a.centre_idx = ctx->centre_idx.as<int>();
-    a.pos = ctx->pos.as<int2>();
+    a.posf = ctx->posf.as<float2>();
+    a.bins = ctx->bingeom.as<BinGeom>();
     a.pay = ctx->pay.as<Pay<T>>();
     a.zs = c.n_z > 1 ? ctx->zs.as<uint8_t>() : nullptr;
     a.cell_start = ctx->count.as<int>();
@@ -1779,7 +1780,8 @@ static mp3pcf_status moments_adjoint_t(mp3pcf_ctx* ctx, const double* gups, cons
     a.nb = nb;
     a.n_max = c.n_max;
     a.centre_idx = ctx->centre_idx.as<int>();
-    a.pos = ctx->pos.as<int2>();
+    a.posf = ctx->posf.as<float2>();
+    a.bins = ctx->bingeom.as<BinGeom>();
     a.pay = ctx->pay.as<Pay<T>>();
     a.zs = nz > 1 ? ctx->zs.as<uint8_t>() : nullptr;
     a.cell_start = ctx->count.as<int>();
@@ -1820,7 +1822,7 @@ static mp3pcf_status moments_adjoint_t(mp3pcf_ctx* ctx, const double* gups, cons
                 MomentArgs<float> m{};
                 m.n_centres = a.n_centres;
                 m.centre_idx = a.centre_idx;
-                m.pos = a.pos;
+                m.pos = ctx->pos.as<int2>();
                 m.pay = a.pay;
                 m.cell_start = a.cell_start;
                 m.g = a.g;

@@ -201,11 +201,14 @@ cudaError_t launch_to_map3_four(const PostArgs& p, const double* gcen, int n_ap,
 
 // ------------------------------------------------------------------ adjoint of stages (b), (a)
 
+struct BinGeom;
+
 template <typename T>
 struct AdjArgs {
     int32_t n_centres, nz, nb, n_max;
     const int32_t* centre_idx;  // sorted position of each centre
-    const int2* pos;            // sorted fixed-point positions
+    const float2* posf;         // sorted positions from the grid's origin (exact in FP32)
+    const BinGeom* bins;        // the bins' FP32 distance tests
     const Pay<T>* pay;          // sorted (w gamma_1, w gamma_2, w)
     const uint8_t* zs;          // sorted zbin (NULL: one bin)
     const int32_t* cell_start;  // as in MomentArgs
