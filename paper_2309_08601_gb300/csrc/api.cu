@@ -491,7 +491,7 @@ struct mp3pcf_ctx {
     DevBuf d_e2q, d_edges, d_nodes;
     DevBuf bb, key, count, fill, scan_sums, scan_total, perm, pos, pay, zs;
     DevBuf cflag, crank, oflag, orank, centre_idx, crow;
-    DevBuf G, W, pairs, partial, singular, m3partial, m3filter, m3four, ccoef;
+    DevBuf G, W, pairs, partial, singular, edgelist, m3partial, m3filter, m3four, ccoef;
     DevBuf gG, gW, gv, gtab, adjscratch;  // adjoint workspace
     DevBuf degen;                       // exclude_degenerate sums per (centre, z, bin)
     DevBuf degen_grad;                  // their gradient sums per (Z1, z, bin) in the adjoint
@@ -668,6 +668,7 @@ mp3pcf_status mp3pcf_create(const mp3pcf_config* cfg, void* stream, mp3pcf_ctx**
         ctx->d_edges.ensure(sizeof(double) * (nb + 1)) != cudaSuccess ||
         ctx->d_nodes.ensure(sizeof(double) * nb) != cudaSuccess ||
         ctx->bingeom.ensure(sizeof(BinGeom) * nb) != cudaSuccess ||
+        ctx->edgelist.ensure(sizeof(int) * (1 + (size_t)cfg->n_z * cfg->n_z * cfg->n_z * nb * nb)) != cudaSuccess ||
         ctx->bb.ensure(sizeof(int) * 10) != cudaSuccess || ctx->pairs.ensure(8 * (4 + kFarPlans)) != cudaSuccess ||
         ctx->singular.ensure(8) != cudaSuccess)
         return cleanup(MP3PCF_ENOMEM);
@@ -696,7 +697,7 @@ mp3pcf_status mp3pcf_destroy(mp3pcf_ctx* ctx)
                       &ctx->pos, &ctx->pay, &ctx->zs, &ctx->cflag,
                       &ctx->crank, &ctx->oflag, &ctx->orank, &ctx->centre_idx, &ctx->crow,
                       &ctx->G, &ctx->W, &ctx->pairs, &ctx->partial, &ctx->singular,
-                      &ctx->m3partial, &ctx->m3filter, &ctx->m3four, &ctx->fftwork, &ctx->ccoef, &ctx->gG, &ctx->gW, &ctx->gv, &ctx->gtab,
+                      &ctx->edgelist, &ctx->m3partial, &ctx->m3filter, &ctx->m3four, &ctx->fftwork, &ctx->ccoef, &ctx->gG, &ctx->gW, &ctx->gv, &ctx->gtab,
                       &ctx->adjscratch, &ctx->degen, &ctx->degen_grad, &ctx->zrange, &ctx->dkey, &ctx->dcell, &ctx->dperm, &ctx->dpos, &ctx->dgw, &ctx->dgrid, &ctx->bingeom, &ctx->ftable, &ctx->posf, &ctx->fkey, &ctx->fstart, &ctx->ffill, &ctx->forder, &ctx->gridsum, &ctx->gridflag, &ctx->bups, &ctx->bnorm,
                       &ctx->bgam, &ctx->bgcen, &ctx->berr, &ctx->pix, &ctx->pixinv};
     for (DevBuf* b : bufs) b->release();
@@ -1314,9 +1315,10 @@ mp3pcf_status mp3pcf_edge_correct(mp3pcf_ctx* ctx, const double* d_upsilon, cons
     MP3_CK(cudaMemsetAsync(ctx->singular.p, 0, 8, ctx->st));
     {
         StageScope sc(ctx, ST_EDGE);
-        ctx->launches[ST_EDGE] += 1;
+        ctx->launches[ST_EDGE] += 2;
         MP3_CK(launch_edge_correct(post_args(ctx), d_upsilon, d_norm, d_gamma_n,
-                                   ctx->singular.as<unsigned long long>(), ctx->st));
+                                   ctx->edgelist.as<int>(), ctx->singular.as<unsigned long long>(), ctx->n_sm,
+                                   ctx->st));
     }
     if (h_n_singular) {
         unsigned long long ns = 0;

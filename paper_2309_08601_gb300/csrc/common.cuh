@@ -140,8 +140,9 @@ struct PostArgs {
     const double* nodes;  // device, nb radial nodes
 };
 
+// list: 1 + systems ints of scratch (the systems that need pivoting)
 cudaError_t launch_edge_correct(const PostArgs& p, const double* ups, const double* norm,
-                                double* gam, unsigned long long* n_singular, cudaStream_t st);
+                                double* gam, int* list, unsigned long long* n_singular, int n_sm, cudaStream_t st);
 cudaError_t launch_to_gamma(const PostArgs& p, const double* gam, int projection, double* out,
                             cudaStream_t st);
 // pixel catalog of the grid-based approximation (Sec. 3.2): per-pixel sums (scratch: 3 n_z npx npy

@@ -85,3 +85,34 @@ def test_direct_cells_equal_the_whole_scan(gpu, theta):
     for k in (0, 1):
         ok = ~np.isnan(one[..., k])
         assert rel_err(many[..., k][ok], one[..., k][ok]) < 1e-12
+
+
+@pytest.mark.parametrize("n_max", [0, 1, 7, 8, 15, 16, 23, 31, 32, 47, 48, 50])
+@pytest.mark.parametrize("nz, truncate", [(1, False), (2, False), (1, True)])
+def test_edge_correction_by_the_toeplitz_recursion(gpu, orc, nz, truncate, n_max):
+    """Diagonally dominant systems of no symmetry take the recursion; one whose leading entry is small,
+    one that is nearly singular (pivoted elimination) and a singular one are among them."""
+    nb, D = 3, 2 * n_max + 1
+    rng = np.random.default_rng(n_max + 100 * nz)
+    c = lambda *s: rng.normal(size=s) + 1j * rng.normal(size=s)  # noqa: E731
+    norm = c(nz ** 3, D, nb, nb)
+    norm[:, 0] = 4.0 * D + rng.normal(size=(nz ** 3, nb, nb))
+    norm[0, 0, 0, 1] = norm[0, 0, 1, 0] = 1e-3
+    if n_max > 0:
+        norm[0, :, 1, 1] = 1.0  # constant in the order: rank one, up to a small diagonal
+        norm[0, 0, 1, 1] = 1.0 + 1e-5
+    norm[0, :, 2, 2] = 0.0
+    ups = c(nz ** 3, 4, n_max + 1, nb, nb)
+    setup = dict(n_bins=nb, theta_min=0.7, theta_max=9.0, n_max=n_max, n_z=nz, norm_truncate=truncate)
+    want, ns = orc.edge_correct(orc.Setup(**setup), ups, norm)
+    with gpu.Estimator(**setup, precision="fp64") as est:
+        got, gs = est.edge_correct(torch.as_tensor(ups, device="cuda"), torch.as_tensor(norm, device="cuda"))
+    got = got.cpu().numpy()
+    assert gs == ns and ns >= 1
+    np.testing.assert_array_equal(np.isnan(got), np.isnan(want))
+    for b1 in range(nb):
+        for b2 in range(nb):
+            g, w = got[..., b1, b2], want[..., b1, b2]
+            ok = ~np.isnan(w)
+            # the nearly singular system: conditioned like D 1e5
+            assert rel_err(g[ok], w[ok]) < (1e-8 if b1 == b2 == 1 else 1e-10), (b1, b2)
