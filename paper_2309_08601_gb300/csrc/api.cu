@@ -420,13 +420,12 @@ __global__ void k_centres(int64_t n, const int* __restrict__ perm, const int* __
 }
 
 // strip-order bucket of every centre: strips of strip_rows cell rows, columns within a strip
-__global__ void k_strip_keys(int nc, const int* __restrict__ centre_idx, const int2* __restrict__ pos, GridDesc g,
+__global__ void k_strip_keys(int nc, const int* __restrict__ centre_idx, const float2* __restrict__ pos, GridDesc g,
                              int strip_rows, int* __restrict__ key, int* __restrict__ count)
 {
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += gridDim.x * blockDim.x) {
-        const int2 p = pos[centre_idx[c]];
-        const int cx_ = (int)min(max(0LL, (long long)p.x - g.x0) / g.side, (long long)g.ncx - 1);
-        const int cy_ = (int)min(max(0LL, (long long)p.y - g.y0) / g.side, (long long)g.ncy - 1);
+        const float2 p = pos[centre_idx[c]];
+        const int cx_ = min(max(0, (int)p.x) / g.side, g.ncx - 1), cy_ = min(max(0, (int)p.y) / g.side, g.ncy - 1);
         const int k = cy_ / strip_rows * g.ncx + cx_;
         key[c] = k;
         atomicAdd(&count[k], 1);
@@ -488,7 +487,7 @@ struct mp3pcf_ctx {
     // fault injection on the host side (tests of failure detection): see mp3pcf_inject
     bool inject_wait_timeout = false, inject_alloc_failure = false;
     cudaEvent_t batch_ev[2] = {nullptr, nullptr};
-    DevBuf d_e2q, d_edges, d_nodes;
+    DevBuf d_edges, d_nodes;
     DevBuf bb, key, count, fill, scan_sums, scan_total, perm, pos, pay, zs;
     DevBuf cflag, crank, oflag, orank, centre_idx, crow;
     DevBuf G, W, pairs, partial, singular, edgelist, m3partial, m3filter, m3four, ccoef;
@@ -664,16 +663,14 @@ mp3pcf_status mp3pcf_create(const mp3pcf_config* cfg, void* stream, mp3pcf_ctx**
     if (cudaDeviceGetAttribute(&ctx->n_sm, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess)
         return cleanup(MP3PCF_ECUDA);
     const int nb = cfg->n_bins;
-    if (ctx->d_e2q.ensure(sizeof(long long) * (nb + 1)) != cudaSuccess ||
-        ctx->d_edges.ensure(sizeof(double) * (nb + 1)) != cudaSuccess ||
+    if (ctx->d_edges.ensure(sizeof(double) * (nb + 1)) != cudaSuccess ||
         ctx->d_nodes.ensure(sizeof(double) * nb) != cudaSuccess ||
         ctx->bingeom.ensure(sizeof(BinGeom) * nb) != cudaSuccess ||
         ctx->edgelist.ensure(sizeof(int) * (1 + (size_t)cfg->n_z * cfg->n_z * cfg->n_z * nb * nb)) != cudaSuccess ||
         ctx->bb.ensure(sizeof(int) * 10) != cudaSuccess || ctx->pairs.ensure(8 * (4 + kFarPlans)) != cudaSuccess ||
         ctx->singular.ensure(8) != cudaSuccess)
         return cleanup(MP3PCF_ENOMEM);
-    if (cudaMemcpy(ctx->d_e2q.p, ctx->e2q.data(), sizeof(long long) * (nb + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(ctx->d_edges.p, ctx->edges.data(), sizeof(double) * (nb + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
+    if (cudaMemcpy(ctx->d_edges.p, ctx->edges.data(), sizeof(double) * (nb + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(ctx->bingeom.p, bin_geometry(ctx->e2q).data(), sizeof(BinGeom) * nb, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(ctx->d_nodes.p, ctx->nodes.data(), sizeof(double) * nb, cudaMemcpyHostToDevice) != cudaSuccess)
         return cleanup(MP3PCF_ECUDA);
@@ -692,7 +689,7 @@ mp3pcf_status mp3pcf_destroy(mp3pcf_ctx* ctx)
 {
     if (!ctx) return MP3PCF_OK;
     cudaStreamSynchronize(ctx->st);
-    DevBuf* bufs[] = {&ctx->d_e2q, &ctx->d_edges, &ctx->d_nodes, &ctx->bb, &ctx->key,
+    DevBuf* bufs[] = {&ctx->d_edges, &ctx->d_nodes, &ctx->bb, &ctx->key,
                       &ctx->count, &ctx->fill, &ctx->scan_sums, &ctx->scan_total, &ctx->perm,
                       &ctx->pos, &ctx->pay, &ctx->zs, &ctx->cflag,
                       &ctx->crank, &ctx->oflag, &ctx->orank, &ctx->centre_idx, &ctx->crow,
@@ -810,11 +807,9 @@ static bool far_args(mp3pcf_ctx* ctx, const MomentArgs<float>& a, const FarPlan&
     if (nbv < 1) return false;
     f->m = a;
     f->m.nb = nbv;
-    f->m.e2q = a.e2q + (b0 - b_lo);
+    f->m.bins = a.bins + (b0 - b_lo);
     f->m.G = a.G + (b0 - b_lo);
     f->m.W = a.W + (b0 - b_lo);
-    f->bins = ctx->bingeom.as<BinGeom>() + b0;
-    f->posf = ctx->posf.as<float2>();
     f->order = ctx->forder.as<int>();
     f->strip_rows = fp.rows;
     f->max_cols = fp.cols;
@@ -842,7 +837,7 @@ static mp3pcf_status run_far(mp3pcf_ctx* ctx, const MomentArgs<float>& a, const 
     MP3_CK(ctx->forder.ensure(sizeof(int) * nc));
     int* fill = ctx->ffill.as<int>();
     MP3_CK(cudaMemsetAsync(fill, 0, sizeof(int) * (K + 1), st));
-    k_strip_keys<<<grid1d(nc, ctx->n_sm), 256, 0, st>>>(nc, a.centre_idx, a.pos, a.g, fp.rows, ctx->fkey.as<int>(), fill);
+    k_strip_keys<<<grid1d(nc, ctx->n_sm), 256, 0, st>>>(nc, a.centre_idx, a.posf, a.g, fp.rows, ctx->fkey.as<int>(), fill);
     MP3_CK(cudaGetLastError());
     if (mp3pcf_status s = scan_exclusive(ctx, fill, ctx->fstart.as<int>(), K)) return s;
     MP3_CK(cudaMemsetAsync(fill, 0, sizeof(int) * (K + 1), st));
@@ -1003,7 +998,7 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
     MomentArgs<T> a;
     a.n_centres = nc;
     a.centre_idx = ctx->centre_idx.as<int>();
-    a.pos = ctx->pos.as<int2>();
+    a.posf = ctx->posf.as<float2>();
     a.pay = ctx->pay.as<Pay<T>>();
     a.cell_start = ctx->count.as<int>();
     a.g = g;
@@ -1011,7 +1006,7 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
     a.nb = fp.b_far - b_lo;
     a.nbp = nb_pad(nb);
     a.n_max = c.n_max;
-    a.e2q = ctx->d_e2q.as<long long>() + b_lo;
+    a.bins = ctx->bingeom.as<BinGeom>() + b_lo;
     a.G = ctx->G.as<cx<T>>() + b_lo;
     a.W = ctx->W.as<cx<T>>() + b_lo;
     a.pairs = ctx->pairs.as<unsigned long long>();
@@ -1027,13 +1022,11 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
         NearArgs<T> na;
         na.m = a;
         na.m.nb = b_near - b_lo;
-        na.bins = ctx->bingeom.as<BinGeom>() + b_lo;
-        na.posf = ctx->posf.as<float2>();
         na.queue = ctx->pairs.as<unsigned long long>() + 3 + kFarPlans;
         ctx->launches[ST_MOMENTS] += 1;
         MP3_CK(launch_moments_near(na, ctx->n_sm, st));
         a.nb -= b_near - b_lo;
-        a.e2q += b_near - b_lo;
+        a.bins += b_near - b_lo;
         a.G += b_near - b_lo;
         a.W += b_near - b_lo;
     }
@@ -1742,7 +1735,6 @@ static AdjArgs<T> catalog_args(mp3pcf_ctx* ctx)
     a.zs = c.n_z > 1 ? ctx->zs.as<uint8_t>() : nullptr;
     a.cell_start = ctx->count.as<int>();
     a.g = ctx->grid;
-    a.e2q = ctx->d_e2q.as<long long>();
     a.G = ctx->G.as<cx<T>>();
     a.W = ctx->W.as<cx<T>>();
     return a;
@@ -1788,7 +1780,6 @@ static mp3pcf_status moments_adjoint_t(mp3pcf_ctx* ctx, const double* gups, cons
     a.zs = nz > 1 ? ctx->zs.as<uint8_t>() : nullptr;
     a.cell_start = ctx->count.as<int>();
     a.g = ctx->grid;
-    a.e2q = ctx->d_e2q.as<long long>();
     a.G = ctx->G.as<cx<T>>();
     a.W = ctx->W.as<cx<T>>();
     a.gups = gups;
@@ -1824,7 +1815,7 @@ static mp3pcf_status moments_adjoint_t(mp3pcf_ctx* ctx, const double* gups, cons
                 MomentArgs<float> m{};
                 m.n_centres = a.n_centres;
                 m.centre_idx = a.centre_idx;
-                m.pos = ctx->pos.as<int2>();
+                m.posf = a.posf;
                 m.pay = a.pay;
                 m.cell_start = a.cell_start;
                 m.g = a.g;
@@ -1832,7 +1823,7 @@ static mp3pcf_status moments_adjoint_t(mp3pcf_ctx* ctx, const double* gups, cons
                 m.nb = a.nb;
                 m.n_max = a.n_max;
                 m.nbp = nb_pad(a.nb);
-                m.e2q = a.e2q;
+                m.bins = a.bins;
                 m.G = a.gG;
                 m.W = a.gW;
                 for (int v = 0; v < kFarPlans; ++v) {

@@ -79,17 +79,19 @@ struct GridDesc {
 
 // ------------------------------------------------------------------ stage (a) arguments
 
+struct BinGeom;
+
 template <typename T>
 struct MomentArgs {
     int32_t n_centres;
     const int32_t* centre_idx;  // sorted position of each centre
-    const int2* pos;            // sorted fixed-point positions
+    const float2* posf;         // sorted positions from the grid's origin (exact: the extent is below 2^24)
     const Pay<T>* pay;          // sorted (w gamma_1, w gamma_2, w)
     const int32_t* cell_start;  // [n_z * ncells + 1], key = zbin * ncells + cy * ncx + cx
     GridDesc g;
     int32_t nz, nb, n_max;      // nb: the radial bins computed, a range [b_lo, b_lo + nb) of the layout's
     int32_t nbp;                // bins per row of the layout (nb_pad of all its bins)
-    const long long* e2q;       // [nb + 1] exact squared edges in fixed-point units^2, from bin b_lo
+    const BinGeom* bins;        // [nb] the bins' distance tests (moments_far.cuh), from bin b_lo
     cx<T>* G;                   // [2 n_max + 3][n_centres][nz][nbp], offset to bin b_lo
     cx<T>* W;                   // [2 n_max + 1][n_centres][nz][nbp], offset to bin b_lo
     unsigned long long* pairs;  // [0] pair counter, [1] error flags (1: a bounded wait gave up)
@@ -202,8 +204,6 @@ cudaError_t launch_to_map3_four(const PostArgs& p, const double* gcen, int n_ap,
 
 // ------------------------------------------------------------------ adjoint of stages (b), (a)
 
-struct BinGeom;
-
 template <typename T>
 struct AdjArgs {
     int32_t n_centres, nz, nb, n_max;
@@ -214,7 +214,6 @@ struct AdjArgs {
     const uint8_t* zs;          // sorted zbin (NULL: one bin)
     const int32_t* cell_start;  // as in MomentArgs
     GridDesc g;
-    const long long* e2q;
     const cx<T>* G;             // forward moments (order-major)
     const cx<T>* W;
     const double* gups;         // dL/dUpsilon [z3][4][n_max+1][nb][nb] complex

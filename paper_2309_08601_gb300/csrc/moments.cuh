@@ -8,8 +8,8 @@
 //    cell row crossed by the annulus [e_b, e_{b+1}). The ranges are concatenated into one flat
 //    candidate stream (prefix sums of their lengths) and split evenly between the warps.
 //  * The bin is processed in rounds. Produce: each warp tests SCR candidates of its share,
-//    exactly on the integer squared separation, and compacts the members (ballot + popc) into
-//    its region of a shared-memory chunk, storing z = (dx + i dy)/r, its powers z^2..z^P, the
+//    in FP32 and near the bin's edges on the integer squared separation, and compacts the members
+//    (ballot + popc) into its region of a shared-memory chunk, storing z = (dx + i dy)/r, its powers z^2..z^P, the
 //    pair (w gamma_1, w gamma_2) as one 8-byte record (one shared load per member where two
 //    4-byte loads cost 2.6 % of the kernel's time) and w. The candidates' positions and
 //    payloads were copied into shared memory by cp.async one round earlier, so this phase does
@@ -27,7 +27,7 @@
 // and hence the result, reproducible run to run.
 #pragma once
 
-#include "common.cuh"
+#include "moments_far.cuh"
 
 // Tiling parameters (compile-time; the defaults are the tuned values).
 // At n_max <= 30 (four warps) the FP32 kernel then holds 4 CTAs per SM: 128 registers per
@@ -91,11 +91,11 @@ struct MomSmem {
     cx<T> zp[P][P * SCR];     // z^1 .. z^P of each member
     cx<T> ab[P * SCR];        // (w gamma_1, w gamma_2) of each member
     T w[P * SCR];
-    int2 spos[P][SCR];        // staged candidate positions (cp.async, one round ahead)
+    float2 spos[P][SCR];      // staged candidate positions (cp.async, one round ahead)
     Pay<T> spay[P][SCR];      // staged candidate payloads
     int2 seg[2 * kMaxRows];   // (first sorted index, count) of the current bin's ranges
     int pre[2 * kMaxRows + 1];  // exclusive prefix sums of the range lengths
-    long long e2q[kMaxBins + 1];
+    unsigned char found[P][SCR];  // staged candidates that are members
     int cnt[8];   // members in each warp's region this round
     int wtot[8];  // per-warp partial sums of the prefix scan
     int claim;    // the CTA's next centre from the work queue
@@ -167,25 +167,23 @@ __device__ __forceinline__ void stage_pay<double>(Pay<double>* dst, const Pay<do
 }
 
 template <typename T>
-__device__ __forceinline__ cx<T> unit_vector(int dx, int dy);
+__device__ __forceinline__ cx<T> unit_vector(float dx, float dy);
 
 template <>
-__device__ __forceinline__ cx<float> unit_vector<float>(int dx, int dy)
+__device__ __forceinline__ cx<float> unit_vector<float>(float dx, float dy)
 {
-    // |dx|, |dy| < 2^24 are exact in FP32; r^2 here only normalises z (the bin test uses the
-    // exact integer r^2)
-    const float fdx = (float)dx, fdy = (float)dy;
-    const float rf = fdx * fdx + fdy * fdy;
+    // |dx|, |dy| < 2^24 are exact in FP32; r^2 here only normalises z (see the bin test)
+    const float rf = dx * dx + dy * dy;
     float inv = rsqrtf(rf);
     inv = inv * (1.5f - 0.5f * rf * inv * inv);  // one Newton step
-    return {fdx * inv, fdy * inv};
+    return {dx * inv, dy * inv};
 }
 
 template <>
-__device__ __forceinline__ cx<double> unit_vector<double>(int dx, int dy)
+__device__ __forceinline__ cx<double> unit_vector<double>(float dx, float dy)
 {
-    const double inv = 1.0 / sqrt((double)dx * dx + (double)dy * dy);
-    return {(double)dx * inv, (double)dy * inv};
+    const double x = dx, y = dy, inv = rsqrt(x * x + y * y);
+    return {x * inv, y * inv};
 }
 
 // Reduce-scatter of N (multiple of 32) per-lane values over the warp: afterwards lane l holds
@@ -359,11 +357,11 @@ __global__ void __launch_bounds__(MomPlan<T, NMAX>::NT, MomPlan<T, NMAX>::MINB) 
     const uint32_t ab_base = smem_u32(&s.ab[0]), w_base = smem_u32(&s.w[0]);
     const uint32_t aP = zp_base + (uint32_t)((P - 1) * CH * sizeof(cx<T>));
     const uint32_t aq = zp_base + (uint32_t)(zsel * CH * sizeof(cx<T>));
-    int2* my_pos = s.spos[warp];
+    float2* my_pos = s.spos[warp];
+    unsigned char* my_found = s.found[warp];
     Pay<T>* my_pay = s.spay[warp];
     unsigned long long my_pairs = 0;
 
-    for (int i = tid; i <= nb; i += NT) s.e2q[i] = A.e2q[i];
     __syncthreads();
 
     MomAcc<T, NABM, NWM, PL::PACKED> macc;
@@ -372,15 +370,15 @@ __global__ void __launch_bounds__(MomPlan<T, NMAX>::NT, MomPlan<T, NMAX>::MINB) 
     // regions, patch edges, sparse z-bins) take more of them and all finish together. A centre's
     // result does not depend on the CTA that computes it.
     for (int c = blockIdx.x; c < A.n_centres;) {
-        const int2 pc = A.pos[A.centre_idx[c]];
-        const float fx = (float)((long long)pc.x - A.g.x0);
-        const float fy = (float)((long long)pc.y - A.g.y0);
+        const float2 pc = A.posf[A.centre_idx[c]];
+        const float fx = pc.x, fy = pc.y;
         for (int z = 0; z < nz; ++z) {
             for (int b = 0; b < nb; ++b) {
-                const long long lo = s.e2q[b], hi = s.e2q[b + 1];
+                const BinGeom* bg = A.bins + b;
+                const float mid = bg->mid, d_in = bg->d_in, d_out = bg->d_out;
                 // ---- index ranges of the cell rows the annulus crosses (conservative)
-                const float Ro = sqrtf((float)hi) * 1.000001f + 4.0f;
-                const float Ri = fmaxf(sqrtf((float)lo) * 0.999999f - 4.0f, 0.0f);
+                const float Ro = bg->Ro * 1.000001f + 4.0f;
+                const float Ri = fmaxf(bg->Ri * 0.999999f - 4.0f, 0.0f);
                 int iy0 = (int)floorf((fy - Ro) * iS - 0.001f);
                 int iy1 = (int)floorf((fy + Ro) * iS + 0.001f);
                 iy0 = max(iy0, 0);
@@ -471,7 +469,7 @@ __global__ void __launch_bounds__(MomPlan<T, NMAX>::NT, MomPlan<T, NMAX>::MINB) 
                         if (t < tq1) {
                             while (ks + 1 < n_seg && s.pre[ks + 1] <= t) ++ks;
                             const int j = s.seg[ks].x + (t - s.pre[ks]);
-                            cp_async8(&my_pos[u * 32 + lane], &A.pos[j]);
+                            cp_async8(&my_pos[u * 32 + lane], &A.posf[j]);
                             stage_pay<T>(&my_pay[u * 32 + lane], &A.pay[j]);
                         }
                     }
@@ -486,31 +484,42 @@ __global__ void __launch_bounds__(MomPlan<T, NMAX>::NT, MomPlan<T, NMAX>::MINB) 
                     cp_async_wait_all();
                     int mycnt = 0;
                     const int base = warp * SCR;
+                    // the members among the candidates: in FP32 away from the bin's edges, by the
+                    // integers near them (64-bit products run on the FP64 pipe)
 #pragma unroll
                     for (int u = 0; u < SCR / 32; ++u) {
                         const bool ok = tb + u * 32 + lane < tq1;
-                        const int2 pu = ok ? my_pos[u * 32 + lane] : pc;
-                        const int dx = pu.x - pc.x, dy = pu.y - pc.y;
-                        const long long r2 = (long long)dx * dx + (long long)dy * dy;
-                        const bool in = ok && (r2 >= lo) && (r2 < hi);
+                        const float2 pu = ok ? my_pos[u * 32 + lane] : pc;
+                        const float dx = pu.x - pc.x, dy = pu.y - pc.y;  // exact
+                        const float d = fabsf(fmaf(dx, dx, dy * dy) - mid);
+                        bool in = d < d_in;
+                        if (!in && d < d_out) {
+                            const long long r2 = (long long)(int)dx * (int)dx + (long long)(int)dy * (int)dy;
+                            in = r2 >= bg->e0 && r2 < bg->e1;
+                        }
+                        in = in && ok;
                         const unsigned m = __ballot_sync(FULL, in);
-                        const int slot = base + mycnt + __popc(m & lt_mask);
-                        // computed by every lane (no divergence), stored by members only
-                        const cx<T> zu = unit_vector<T>(dx, dy);
+                        if (in) my_found[mycnt + __popc(m & lt_mask)] = (unsigned char)(u * 32 + lane);
+                        mycnt += __popc(m);
+                    }
+                    __syncwarp();
+                    // their directions and powers, all lanes busy
+                    for (int i = lane; i < mycnt; i += 32) {
+                        const int at = my_found[i], slot = base + i;
+                        const float2 pu = my_pos[at];
+                        const Pay<T> py = my_pay[at];
+                        const cx<T> zu = unit_vector<T>(pu.x - pc.x, pu.y - pc.y);
                         cx<T> zz = zu;
-                        if (in) s.zp[0][slot] = zu;
+                        s.zp[0][slot] = zu;
 #pragma unroll
                         for (int k = 1; k < P; ++k) {
                             zz = cmul(zz, zu);
-                            if (in) s.zp[k][slot] = zz;
+                            s.zp[k][slot] = zz;
                         }
-                        if (in) {
-                            const Pay<T> py = my_pay[u * 32 + lane];
-                            s.ab[slot] = cx<T>{py.a, py.b};
-                            s.w[slot] = py.w;
-                        }
-                        mycnt += __popc(m);
+                        s.ab[slot] = cx<T>{py.a, py.b};
+                        s.w[slot] = py.w;
                     }
+                    __syncwarp();  // the staging area is free
                     if (lane == 0) s.cnt[warp] = mycnt;
                     tb += SCR;
                     const bool more = __syncthreads_or(tb < tq1) != 0;

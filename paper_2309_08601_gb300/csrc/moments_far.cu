@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
             float2 p = make_float2(0.f, 0.f);
             if (i < m.n_centres) {
                 row = A.order[i];
-                p = A.posf[m.centre_idx[row]];
+                p = A.m.posf[m.centre_idx[row]];
                 cell = (int)p.y / (m.g.side * A.strip_rows) * m.g.ncx + (int)p.x / m.g.side;
             }
             s_row[tid] = row;
@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
                 const int b = m.nb - 1 - zb / nz, z = zb % nz;
                 // from memory, not from the integer edges: 64-bit conversions run on the FP64 pipe, and
                 // the compiler would repeat them in the candidate loop
-                const BinGeom* bg = A.bins + b;
+                const BinGeom* bg = A.m.bins + b;
                 const float mid = bg->mid, d_in = bg->d_in, d_out = bg->d_out;
                 g.Ri = bg->Ri;
                 g.Ro = bg->Ro;
@@ -497,7 +497,7 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
                         sector_batches(g, upper, sp == 0, sp == S / 2 - 1, ray[sp], ray[sp + 1], sn0, sn1, row_start, qu, lane,
                                        [&](int n) {
                             int i0 = qu[min(sub, n - 1)], i1 = qu[min(sub + kSub, n - 1)];
-                            float2 p0 = at32(A.posf, i0), p1 = at32(A.posf, i1);
+                            float2 p0 = at32(A.m.posf, i0), p1 = at32(A.m.posf, i1);
                             int odd = 0;
                             for (int t = sub; t < n + sub; t += kSub) {
                                 const float2 p = p0;
@@ -505,7 +505,7 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
                                 p0 = p1;
                                 i0 = i1;
                                 i1 = qu[min(t + 2 * kSub, n - 1)];
-                                p1 = at32(A.posf, i1);
+                                p1 = at32(A.m.posf, i1);
                                 const float dx = p.x - pc.x, dy = p.y - pc.y;  // exact
                                 const float r2 = fmaf(dx, dx, dy * dy), d = fabsf(r2 - mid);
                                 const bool in = d < d_in && t < n;
@@ -515,7 +515,7 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
                             if (__any_sync(FULL, odd))  // rare: the candidates near an edge, by the integers
                                 for (int t = sub; t < n + sub; t += kSub) {
                                     const int i = qu[min(t, n - 1)];
-                                    const float2 p = at32(A.posf, i);
+                                    const float2 p = at32(A.m.posf, i);
                                     const float dx = p.x - pc.x, dy = p.y - pc.y;
                                     const float r2 = fmaf(dx, dx, dy * dy), d = fabsf(r2 - mid);
                                     const long long q2 = (long long)(int)dx * (int)dx + (long long)(int)dy * (int)dy;
@@ -531,7 +531,7 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
                                        [&](int n) {
                             // candidates sub, sub + 4, ...: two loads ahead of the arithmetic
                             int i0 = qu[min(sub, n - 1)], i1 = qu[min(sub + kSub, n - 1)];
-                            float2 p0 = at32(A.posf, i0), p1 = at32(A.posf, i1);
+                            float2 p0 = at32(A.m.posf, i0), p1 = at32(A.m.posf, i1);
                             Pay<float> v0 = at32(m.pay, i0), v1 = at32(m.pay, i1);
                             for (int t = sub; t < n + sub; t += kSub) {
                                 const float2 p = p0;
@@ -539,7 +539,7 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
                                 p0 = p1;
                                 v0 = v1;
                                 i1 = qu[min(t + 2 * kSub, n - 1)];
-                                p1 = at32(A.posf, i1);
+                                p1 = at32(A.m.posf, i1);
                                 v1 = at32(m.pay, i1);
                                 const float dx = p.x - pc.x, dy = p.y - pc.y;  // exact
                                 const float r2 = fmaf(dx, dx, dy * dy), d = fabsf(r2 - mid);
@@ -552,7 +552,7 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
                             if (__any_sync(FULL, maybe != count)) {
                                 // rare: the candidates near an edge, by the integers
                                 for (int t = sub; t < n; t += kSub) {
-                                    const float2 p = at32(A.posf, qu[t]);
+                                    const float2 p = at32(A.m.posf, qu[t]);
                                     const Pay<float> v = at32(m.pay, qu[t]);
                                     const float dx = p.x - pc.x, dy = p.y - pc.y;
                                     const float r2 = fmaf(dx, dx, dy * dy), d = fabsf(r2 - mid);

@@ -27,8 +27,6 @@ void far_tables(int n_max, FarTables (&t)[kFarPlans], std::vector<float>* v);
 
 struct FarArgs {
     MomentArgs<float> m;   // bins, pointers and outputs as in the direct form
-    const BinGeom* bins;   // from bin b_lo of the range
-    const float2* posf;    // sorted positions from the grid's origin (exact: the extent is below 2^24)
     const int32_t* order;  // rows of the centres in strip order: (strip, column, row)
     int strip_rows;        // cell rows of a strip
     int max_cols;          // columns a group may span
@@ -46,8 +44,6 @@ cudaError_t launch_moments_far_adjoint(const FarArgs& a, int plan, int n_sm, cud
 template <typename T>
 struct NearArgs {
     MomentArgs<T> m;
-    const BinGeom* bins;        // as in FarArgs
-    const float2* posf;
     unsigned long long* queue;  // items claimed beyond the first gridDim.x * warps (zero at launch)
     int parts;                  // set by the launcher: work items the bins of a centre are split into
 };

@@ -3,8 +3,8 @@
 // The block-per-centre form spends some 9000 warp instructions per (centre, bin) on barriers, range
 // set-up, half-empty batches and the reduction over lanes, whatever the bin holds. Here a warp works
 // on a centre by itself and its lanes are the orders: lane l keeps W_m, A_m and B_m of
-// m = l, l + 32, ... The warp tests 32 candidates at a time, one per lane, and the lanes of members
-// store the powers z^0..z^7, z^8, z^16, z^24, z^32 of their direction; then the members are added one
+// m = l, l + 32, ... The warp tests 32 candidates at a time, one per lane; once 32 members are found
+// (or the bin ends) the lanes store the powers of their directions, and the members are added one
 // after the other, every lane forming its own z^m from two of the stored powers. About 27 warp
 // instructions a member at n_max = 30, no reduction, no barrier; the direct form's 14 a member plus its
 // overhead are less from a few hundred members on. The order of the sums is fixed.
@@ -18,7 +18,6 @@ namespace mp3 {
 namespace near {
 
 constexpr int kQueue = 128;
-constexpr int kPow = 13;  // stored powers of a member: z^0..z^7, z^0, z^8, z^16, z^24, z^32
 
 // warps of a block (the stored powers take 3.3 KB a warp in FP32) and blocks per SM the registers are
 // sized for
@@ -41,7 +40,7 @@ __device__ __forceinline__ cx<float> direction(float dx, float dy, float)
 }
 __device__ __forceinline__ cx<double> direction(float dx, float dy, double)
 {
-    const double x = dx, y = dy, inv = 1.0 / sqrt(x * x + y * y);
+    const double x = dx, y = dy, inv = rsqrt(x * x + y * y);
     return {x * inv, y * inv};
 }
 
@@ -59,19 +58,26 @@ __global__ void __launch_bounds__(Block<T>::kThreads, Block<T>::kMin) near_momen
     constexpr unsigned FULL = 0xffffffffu;
     const MomentArgs<T>& m = A.m;
     __shared__ BinGeom bins[kMaxBins];
-    __shared__ int queue[kWarps][kQueue];
-    __shared__ cx<T> pw[kWarps][32 * kPow];
+    // stored powers of a member: z^0..z^7, z^0, z^8, z^16, z^24, z^32, of which a lane forms its own by a
+    // product; in FP64 with up to 31 orders all of them, as an FP64 instruction takes 16 cycles whatever the
+    // number of lanes that need it
+    constexpr bool kAll = sizeof(T) == 8 && SW == 1;
+    constexpr int kPow = kAll ? 33 : 13;
+    extern __shared__ __align__(16) unsigned char smem_raw[];  // powers [kWarps][32 kPow]
+    __shared__ int queue[kWarps][kQueue], founds[kWarps][64];
     __shared__ Member<T> mem[kWarps][32];
+    const int mtop = max(2 * A.m.n_max, A.m.n_max + 3);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt_mask = (1u << lane) - 1u;
     const int nz = m.nz, n_max = m.n_max;
     const size_t plane = (size_t)m.n_centres * nz * m.nbp;
     for (int b = threadIdx.x; b < m.nb; b += kThreads) {
-        bins[b] = A.bins[b];
+        bins[b] = A.m.bins[b];
     }
     __syncthreads();
     int* qu = queue[warp];
-    cx<T>* P = pw[warp];
+    int* found = founds[warp];
+    cx<T>* P = reinterpret_cast<cx<T>*>(smem_raw) + warp * 32 * kPow;
     Member<T>* V = mem[warp];
     SectorGeom g;
     g.hx = g.hy = 0.0f;
@@ -84,7 +90,7 @@ __global__ void __launch_bounds__(Block<T>::kThreads, Block<T>::kMin) near_momen
     const long long nitems = (long long)m.n_centres * A.parts;
     for (long long item = blockIdx.x * kWarps + warp; item < nitems;) {
         const int c = (int)(item / A.parts), part = (int)(item - (long long)c * A.parts);
-        const float2 pc = A.posf[m.centre_idx[c]];
+        const float2 pc = A.m.posf[m.centre_idx[c]];
         g.gx = pc.x;
         g.gy = pc.y;
         for (int z = 0; z < nz; ++z) {
@@ -98,6 +104,66 @@ __global__ void __launch_bounds__(Block<T>::kThreads, Block<T>::kMin) near_momen
                 for (int s = 0; s < SW; ++s) aw[s] = cx<T>{T(0), T(0)};
 #pragma unroll
                 for (int s = 0; s < SAB; ++s) aa[s] = ab[s] = cx<T>{T(0), T(0)};
+                // the first cnt members found: their powers by the lanes, then one member after the other
+                auto add_members = [&](int cnt) {
+                    if (lane < cnt) {
+                        const int i = found[lane];
+                        const float2 p = A.m.posf[i];
+                        const Pay<T> v = m.pay[i];
+                        V[lane] = Member<T>{v.a, v.b, v.w, T(0)};
+                        const cx<T> z1 = direction(p.x - pc.x, p.y - pc.y, T(0));
+                        cx<T>* q = P + lane * kPow;
+                        const cx<T> z2 = cmul(z1, z1), z4 = cmul(z2, z2), z3 = cmul(z2, z1);
+                        q[0] = cx<T>{T(1), T(0)};
+                        q[1] = z1;
+                        q[2] = z2;
+                        q[3] = z3;
+                        q[4] = z4;
+                        const cx<T> z5 = cmul(z4, z1), z6 = cmul(z4, z2), z7 = cmul(z4, z3), z8 = cmul(z4, z4);
+                        q[5] = z5;
+                        q[6] = z6;
+                        q[7] = z7;
+                        if constexpr (kAll) {  // every power up to the highest order
+                            cx<T> lo[8] = {q[0], z1, z2, z3, z4, z5, z6, z7}, hi = z8;
+#pragma unroll
+                            for (int k = 8; k < kPow; ++k) {
+                                if (k > mtop) break;
+                                if (k % 8 == 0 && k > 8) hi = cmul(hi, z8);
+                                q[k] = k % 8 == 0 ? hi : cmul(hi, lo[k % 8]);
+                            }
+                        } else {
+                            const cx<T> z16 = cmul(z8, z8);
+                            q[8] = cx<T>{T(1), T(0)};
+                            q[9] = z8;
+                            q[10] = z16;
+                            q[11] = cmul(z16, z8);
+                            if (SW > 1) q[12] = cmul(z16, z16);
+                        }
+                    }
+                    __syncwarp();
+                    my_pairs += cnt;
+#pragma unroll 2
+                    for (int j = 0; j < cnt; ++j) {
+                        const cx<T>* q = P + j * kPow;
+                        const Member<T> v = V[j];
+                        cx<T> zc;
+                        if constexpr (kAll)
+                            zc = q[min(lane, mtop)];
+                        else
+                            zc = cmul(q[lane & 7], q[8 + (lane >> 3)]);
+#pragma unroll
+                        for (int s = 0; s < SW; ++s) {
+                            cacc(aw[s], v.w, zc);
+                            if (s < SAB) {
+                                cacc(aa[s], v.a, zc);
+                                cacc(ab[s], v.b, zc);
+                            }
+                            if (s + 1 < SW) zc = cmul(zc, q[12]);
+                        }
+                    }
+                    __syncwarp();
+                };
+                int nm = 0;  // members found and not yet added
                 const float ro = g.Ro + 8.0f;
                 const float iy0 = fmaxf(floorf((g.gy - ro) * g.iS), 0.0f);
                 const float iy1 = fminf(floorf((g.gy + ro) * g.iS), (float)(g.ncy - 1));
@@ -128,7 +194,7 @@ __global__ void __launch_bounds__(Block<T>::kThreads, Block<T>::kMin) near_momen
                         __syncwarp();
                         for (int t = lane; t < n + lane; t += 32) {
                             const int i = qu[min(t, n - 1)];
-                            const float2 p = A.posf[i];
+                            const float2 p = A.m.posf[i];
                             const float dx = p.x - pc.x, dy = p.y - pc.y;  // exact
                             const float d = fabsf(fmaf(dx, dx, dy * dy) - bg.mid);
                             bool in = d < bg.d_in;
@@ -136,53 +202,21 @@ __global__ void __launch_bounds__(Block<T>::kThreads, Block<T>::kMin) near_momen
                                 const long long q2 = (long long)(int)dx * (int)dx + (long long)(int)dy * (int)dy;
                                 in = q2 >= bg.e0 && q2 < bg.e1;
                             }
-                            in = in && t < n;
-                            const unsigned mask = __ballot_sync(FULL, in);
-                            if (mask == 0) continue;
-                            if (in) {
-                                const int slot = __popc(mask & lt_mask);
-                                const Pay<T> v = m.pay[i];
-                                V[slot] = Member<T>{v.a, v.b, v.w, T(0)};
-                                const cx<T> z1 = direction(dx, dy, T(0));
-                                cx<T>* q = P + slot * kPow;
-                                const cx<T> z2 = cmul(z1, z1), z4 = cmul(z2, z2), z3 = cmul(z2, z1);
-                                const cx<T> z8 = cmul(z4, z4), z16 = cmul(z8, z8);
-                                q[0] = q[8] = cx<T>{T(1), T(0)};
-                                q[1] = z1;
-                                q[2] = z2;
-                                q[3] = z3;
-                                q[4] = z4;
-                                q[5] = cmul(z4, z1);
-                                q[6] = cmul(z4, z2);
-                                q[7] = cmul(z4, z3);
-                                q[9] = z8;
-                                q[10] = z16;
-                                q[11] = cmul(z16, z8);
-                                if (SW > 1) q[12] = cmul(z16, z16);
-                            }
+                            const unsigned mask = __ballot_sync(FULL, in && t < n);
+                            if (in && t < n) found[nm + __popc(mask & lt_mask)] = i;
+                            nm += __popc(mask);
                             __syncwarp();
-                            const int cnt = __popc(mask);
-                            my_pairs += cnt;
-#pragma unroll 2
-                            for (int j = 0; j < cnt; ++j) {
-                                const cx<T>* q = P + j * kPow;
-                                const Member<T> v = V[j];
-                                cx<T> zc = cmul(q[lane & 7], q[8 + (lane >> 3)]);
-#pragma unroll
-                                for (int s = 0; s < SW; ++s) {
-                                    cacc(aw[s], v.w, zc);
-                                    if (s < SAB) {
-                                        cacc(aa[s], v.a, zc);
-                                        cacc(ab[s], v.b, zc);
-                                    }
-                                    if (s + 1 < SW) zc = cmul(zc, q[12]);
-                                }
+                            if (nm >= 32) {
+                                add_members(32);
+                                if (lane < nm - 32) found[lane] = found[32 + lane];
+                                nm -= 32;
+                                __syncwarp();
                             }
-                            __syncwarp();
                         }
                         if (total <= kQueue) break;
                     }
                 }
+                if (nm > 0) add_members(nm);
                 const size_t row = ((size_t)c * nz + z) * m.nbp + b;
 #pragma unroll
                 for (int s = 0; s < SW; ++s) {
@@ -208,15 +242,18 @@ template <typename T, int SW, int SAB>
 static cudaError_t launch(NearArgs<T> a, int n_sm, cudaStream_t st)
 {
     constexpr int kWarps = Block<T>::kWarps, kThreads = Block<T>::kThreads;
+    const size_t smem = sizeof(cx<T>) * kWarps * 32 * (sizeof(T) == 8 && SW == 1 ? 33 : 13);
     int per_sm = 0;
-    const cudaError_t e = occupancy(&per_sm, near_moments_kernel<T, SW, SAB>, kThreads, 0);
+    cudaError_t e = set_smem_attr(near_moments_kernel<T, SW, SAB>, smem);
+    if (e != cudaSuccess) return e;
+    e = occupancy(&per_sm, near_moments_kernel<T, SW, SAB>, kThreads, smem);
     if (e != cudaSuccess) return e;
     const int64_t slots = (int64_t)n_sm * std::max(per_sm, 1) * kWarps;
     if (a.m.n_centres < 1) return cudaSuccess;
     // few centres: the bins of a centre go to several warps (a chain of small bins is all latency)
     a.parts = (int)std::min<int64_t>(a.m.nb, std::max<int64_t>(1, 4 * slots / a.m.n_centres));
     const int64_t grid = (std::min<int64_t>((int64_t)a.m.n_centres * a.parts, slots) + kWarps - 1) / kWarps;
-    near_moments_kernel<T, SW, SAB><<<(unsigned)grid, kThreads, 0, st>>>(a);
+    near_moments_kernel<T, SW, SAB><<<(unsigned)grid, kThreads, smem, st>>>(a);
     return cudaGetLastError();
 }
 
