@@ -432,23 +432,48 @@ __global__ void k_strip_keys(int nc, const int* __restrict__ centre_idx, const f
     }
 }
 
+// order-major src[q][c][z][nb_pad] (centres in sorted order) -> dst[crow[c]][z][b][q]. A block moves
+// `rows` neighbouring (c, z) rows through shared memory, so that both sides go in long runs (written
+// one element at a time, 8 bytes of each 32-byte sector, 398 MB took 1.48 ms; DRAM-bound now: 363 us).
 template <typename T>
-__global__ void k_copy_rows(int64_t nc, int nz, int nb, int len, const int* __restrict__ crow,
-                            const cx<T>* __restrict__ src, cx<T>* __restrict__ dst)
+__global__ void __launch_bounds__(256) k_copy_rows(int64_t nc, int nz, int nb, int len, int rows,
+                                                   const int* __restrict__ crow, const cx<T>* __restrict__ src,
+                                                   cx<T>* __restrict__ dst)
 {
-    // order-major src[q][c][z][nb_pad] (centres in sorted order) -> dst[crow[c]][z][b][q]
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    cx<T>* tile = reinterpret_cast<cx<T>*>(smem_raw);  // [len][rows * nb + 1]
     const int nbp = nb_pad(nb);
-    const int64_t total = (int64_t)len * nc * nz * nb;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int b = (int)(t % nb);
-        int64_t r = t / nb;
-        const int z = (int)(r % nz);
-        r /= nz;
-        const int64_t c = r % nc;
-        const int q = (int)(r / nc);
-        dst[(((int64_t)crow[c] * nz + z) * nb + b) * len + q] = src[(((int64_t)q * nc + c) * nz + z) * nbp + b];
+    const int64_t total = nc * nz;
+    for (int64_t r0 = (int64_t)blockIdx.x * rows; r0 < total; r0 += (int64_t)gridDim.x * rows) {
+        const int nr = (int)min((int64_t)rows, total - r0), w = nr * nb, pitch = rows * nb + 1;
+        for (int i = threadIdx.x; i < len * w; i += 256) {
+            const int q = i / w, j = i - q * w, r = j / nb, b = j - r * nb;
+            tile[q * pitch + j] = src[((size_t)q * total + r0 + r) * nbp + b];
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < len * w; i += 256) {
+            const int j = i / len, q = i - j * len, r = j / nb, b = j - r * nb;
+            const int64_t cz = r0 + r, c = cz / nz;
+            dst[(((int64_t)crow[c] * nz + (cz - c * nz)) * nb + b) * len + q] = tile[q * pitch + j];
+        }
+        __syncthreads();
     }
+}
+
+template <typename T>
+static cudaError_t copy_rows(int64_t nc, int nz, int nb, int len, const int* crow, const void* src, void* dst, int n_sm,
+                             cudaStream_t st)
+{
+    // up to 40 KB a block (at most 103 orders x 64 bins x 16 bytes for one row)
+    const size_t one = sizeof(cx<T>) * (size_t)len * nb;
+    const int rows = (int)std::max<size_t>(1, std::min<size_t>(16, 40 * 1024 / one));
+    const size_t smem = sizeof(cx<T>) * (size_t)len * ((size_t)rows * nb + 1);
+    cudaError_t e = set_smem_attr(k_copy_rows<T>, smem);
+    if (e != cudaSuccess) return e;
+    const int64_t groups = (nc * nz + rows - 1) / rows;
+    k_copy_rows<T><<<(unsigned)std::min<int64_t>(groups, (int64_t)n_sm * 32), 256, smem, st>>>(
+        nc, nz, nb, len, rows, crow, (const cx<T>*)src, (cx<T>*)dst);
+    return cudaGetLastError();
 }
 
 }  // namespace mp3
@@ -1212,15 +1237,10 @@ mp3pcf_status mp3pcf_copy_moments(mp3pcf_ctx* ctx, void* d_G, void* d_W)
     if (nc == 0) return MP3PCF_OK;
     const mp3pcf_config& c = ctx->cfg;
     const int nz = c.n_z, nb = c.n_bins, lg = 2 * c.n_max + 3, lw = 2 * c.n_max + 1;
-    const unsigned gr = grid1d(nc * nz * nb * lg, ctx->n_sm);
-    if (ctx->fp64) {
-        if (d_G) k_copy_rows<double><<<gr, 256, 0, ctx->st>>>(nc, nz, nb, lg, ctx->crow.as<int>(), ctx->G.as<cx<double>>(), (cx<double>*)d_G);
-        if (d_W) k_copy_rows<double><<<gr, 256, 0, ctx->st>>>(nc, nz, nb, lw, ctx->crow.as<int>(), ctx->W.as<cx<double>>(), (cx<double>*)d_W);
-    } else {
-        if (d_G) k_copy_rows<float><<<gr, 256, 0, ctx->st>>>(nc, nz, nb, lg, ctx->crow.as<int>(), ctx->G.as<cx<float>>(), (cx<float>*)d_G);
-        if (d_W) k_copy_rows<float><<<gr, 256, 0, ctx->st>>>(nc, nz, nb, lw, ctx->crow.as<int>(), ctx->W.as<cx<float>>(), (cx<float>*)d_W);
-    }
-    MP3_CK(cudaGetLastError());
+    const int* crow = ctx->crow.as<int>();
+    auto copy = ctx->fp64 ? copy_rows<double> : copy_rows<float>;
+    if (d_G) MP3_CK(copy(nc, nz, nb, lg, crow, ctx->G.p, d_G, ctx->n_sm, ctx->st));
+    if (d_W) MP3_CK(copy(nc, nz, nb, lw, crow, ctx->W.p, d_W, ctx->n_sm, ctx->st));
     return MP3PCF_OK;
 }
 
