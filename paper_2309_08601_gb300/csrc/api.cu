@@ -371,6 +371,10 @@ __global__ void k_gather(int64_t n, const int* __restrict__ perm, const int32_t*
     for (int64_t d = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; d < n;
          d += (int64_t)gridDim.x * blockDim.x) {
         const int i = perm[d];
+        if (d == 0) {  // the sector form's filler entry: twice the largest extent away
+            posf[n] = make_float2(67108864.0f, 67108864.0f);
+            pay[n] = Pay<T>{T(0), T(0), T(0), T(0)};
+        }
         pos[d] = make_int2(xq[i], yq[i]);
         // positions from the grid's origin are below 2^24 and so exact in FP32
         posf[d] = make_float2((float)((long long)xq[i] - x0), (float)((long long)yq[i] - y0));
@@ -836,6 +840,7 @@ static bool far_args(mp3pcf_ctx* ctx, const MomentArgs<float>& a, const FarPlan&
     f->m.G = a.G + (b0 - b_lo);
     f->m.W = a.W + (b0 - b_lo);
     f->order = ctx->forder.as<int>();
+    f->none = (int)ctx->n;
     f->strip_rows = fp.rows;
     f->max_cols = fp.cols;
     // about six items per resident block, so that the last ones end together
@@ -968,7 +973,7 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
     MP3_CK(ctx->fill.ensure(sizeof(int) * (K + 1)));
     MP3_CK(ctx->perm.ensure(sizeof(int) * n));
     MP3_CK(ctx->pos.ensure(sizeof(int2) * n));
-    MP3_CK(ctx->pay.ensure(sizeof(Pay<T>) * n));
+    MP3_CK(ctx->pay.ensure(sizeof(Pay<T>) * (n + 1)));
     MP3_CK(ctx->zs.ensure(n));
     if (mask) {
         MP3_CK(ctx->cflag.ensure(sizeof(int) * (n + 1)));
@@ -978,7 +983,7 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
     }
     MP3_CK(ctx->centre_idx.ensure(sizeof(int) * n));
     MP3_CK(ctx->crow.ensure(sizeof(int) * n));
-    MP3_CK(ctx->posf.ensure(sizeof(float2) * n));
+    MP3_CK(ctx->posf.ensure(sizeof(float2) * (n + 1)));
     MP3_CK(cudaMemsetAsync(ctx->fill.p, 0, sizeof(int) * (K + 1), st));
     ctx->launches[ST_SORT] += 4;
     k_keys<<<grid1d(n, ctx->n_sm), 256, 0, st>>>(n, xq, yq, zb, nz, g, ctx->key.as<int>(), ctx->fill.as<int>());

@@ -37,6 +37,7 @@ constexpr int kWarps = 8, kThreads = kWarps * 32;
 constexpr int kC = 8;       // centres of a group
 constexpr int kSub = 4;     // candidate streams of a warp (kC * kSub = 32 lanes)
 constexpr int kQueue = 128; // candidates listed at a time per warp
+constexpr int kAhead = 3;   // candidates of a lane in flight
 
 // S sectors, PW terms of W, PAB terms of A and B
 template <int S_, int PW_, int PAB_>
@@ -280,11 +281,12 @@ __device__ __forceinline__ float rsqrt_approx(float x)
 }
 
 // the candidates of a sector in batches of up to kQueue, listed in row order: batch(n) is called by the
-// whole warp with their indexes in queue[0 .. n)
+// whole warp with their indexes in queue[0 .. n), followed by kAhead kSub times `none`, a galaxy far from
+// everything (so the candidate loop needs no test for its end)
 template <typename F>
 __device__ __forceinline__ void sector_batches(const SectorGeom& g, bool upper, bool first, bool last, float ct0, float ct1,
-                                               float sn0, float sn1, const int* __restrict__ row_start, int* queue,
-                                               int lane, F&& batch)
+                                               float sn0, float sn1, const int* __restrict__ row_start, int none,
+                                               int* queue, int lane, F&& batch)
 {
     constexpr unsigned FULL = 0xffffffffu;
     float iy0, iy1;
@@ -310,8 +312,10 @@ __device__ __forceinline__ void sector_batches(const SectorGeom& g, bool upper, 
             n0 -= t0;
             st1 += put - t0;
             n1 -= put - t0;
+            const int n = min(total, kQueue);
+            if (lane < kAhead * kSub) queue[n + lane] = none;
             __syncwarp();
-            batch(min(total, kQueue));
+            batch(n);
             __syncwarp();
             if (total <= kQueue) break;
         }
@@ -329,7 +333,7 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
     constexpr int S = PL::S, PW = PL::PW, PAB = PL::PAB, PT = PL::PT, KS = PL::KS;
     constexpr unsigned FULL = 0xffffffffu;
     extern __shared__ __align__(16) float M[];  // [S][KS]: sums of (sector, term, centre), then their FFT
-    __shared__ int queue[kWarps][kQueue];
+    __shared__ int queue[kWarps][kQueue + kAhead * kSub];
     __shared__ float2 s_pos[kC];
     __shared__ int s_row[kC], s_cell[kC];
     __shared__ int s_next, s_item;
@@ -355,7 +359,7 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
             float2 p = make_float2(0.f, 0.f);
             if (i < m.n_centres) {
                 row = A.order[i];
-                p = A.m.posf[m.centre_idx[row]];
+                p = m.posf[m.centre_idx[row]];
                 cell = (int)p.y / (m.g.side * A.strip_rows) * m.g.ncx + (int)p.x / m.g.side;
             }
             s_row[tid] = row;
@@ -398,7 +402,7 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
                 const int b = m.nb - 1 - zb / nz, z = zb % nz;
                 // from memory, not from the integer edges: 64-bit conversions run on the FP64 pipe, and
                 // the compiler would repeat them in the candidate loop
-                const BinGeom* bg = A.m.bins + b;
+                const BinGeom* bg = m.bins + b;
                 const float mid = bg->mid, d_in = bg->d_in, d_out = bg->d_out;
                 g.Ri = bg->Ri;
                 g.Ro = bg->Ro;
@@ -494,28 +498,36 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
                             v += __shfl_xor_sync(FULL, v, 1);
                             if (!(lane & 1) && v != 0.f) atomicAdd(A.gvw + 4 * (size_t)i + (u2 ? 2 : u1 ? 1 : 0), v);
                         };
-                        sector_batches(g, upper, sp == 0, sp == S / 2 - 1, ray[sp], ray[sp + 1], sn0, sn1, row_start, qu, lane,
+                        sector_batches(g, upper, sp == 0, sp == S / 2 - 1, ray[sp], ray[sp + 1], sn0, sn1, row_start, A.none, qu, lane,
                                        [&](int n) {
-                            int i0 = qu[min(sub, n - 1)], i1 = qu[min(sub + kSub, n - 1)];
-                            float2 p0 = at32(A.m.posf, i0), p1 = at32(A.m.posf, i1);
                             int odd = 0;
-                            for (int t = sub; t < n + sub; t += kSub) {
-                                const float2 p = p0;
-                                const int i = i0;
-                                p0 = p1;
-                                i0 = i1;
-                                i1 = qu[min(t + 2 * kSub, n - 1)];
-                                p1 = at32(A.m.posf, i1);
+                            auto one = [&](int i, float2 p) {
                                 const float dx = p.x - pc.x, dy = p.y - pc.y;  // exact
                                 const float r2 = fmaf(dx, dx, dy * dy), d = fabsf(r2 - mid);
-                                const bool in = d < d_in && t < n;
-                                odd += d < d_out && t < n && !in ? 1 : 0;
+                                const bool in = d < d_in;
+                                odd += d < d_out && !in ? 1 : 0;
                                 add(i, in && mine, fmaf(fmaf(dy, ax.x, -dx * ax.y), rsqrt_approx(r2), ax.z));
+                            };
+                            const int its = (n + kSub - 1) / kSub;
+                            const int* q = qu + sub;
+                            int i0 = q[0], i1 = q[kSub], i2 = q[2 * kSub];
+                            float2 p0 = at32(m.posf, i0), p1 = at32(m.posf, i1), p2 = at32(m.posf, i2);
+                            for (int it = 0;;) {
+                                one(i0, p0);
+                                if (++it >= its) break;
+                                p0 = at32(m.posf, i0 = q[3 * kSub]);
+                                one(i1, p1);
+                                if (++it >= its) break;
+                                p1 = at32(m.posf, i1 = q[4 * kSub]);
+                                one(i2, p2);
+                                if (++it >= its) break;
+                                p2 = at32(m.posf, i2 = q[5 * kSub]);
+                                q += kAhead * kSub;
                             }
                             if (__any_sync(FULL, odd))  // rare: the candidates near an edge, by the integers
                                 for (int t = sub; t < n + sub; t += kSub) {
                                     const int i = qu[min(t, n - 1)];
-                                    const float2 p = at32(A.m.posf, i);
+                                    const float2 p = at32(m.posf, i);
                                     const float dx = p.x - pc.x, dy = p.y - pc.y;
                                     const float r2 = fmaf(dx, dx, dy * dy), d = fabsf(r2 - mid);
                                     const long long q2 = (long long)(int)dx * (int)dx + (long long)(int)dy * (int)dy;
@@ -527,32 +539,45 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
                         Sums<PW, PAB> sum;
                         sum.reset();
                         int count = 0, maybe = 0;
-                        sector_batches(g, upper, sp == 0, sp == S / 2 - 1, ray[sp], ray[sp + 1], sn0, sn1, row_start, qu, lane,
+                        sector_batches(g, upper, sp == 0, sp == S / 2 - 1, ray[sp], ray[sp + 1], sn0, sn1, row_start, A.none, qu, lane,
                                        [&](int n) {
-                            // candidates sub, sub + 4, ...: two loads ahead of the arithmetic
-                            int i0 = qu[min(sub, n - 1)], i1 = qu[min(sub + kSub, n - 1)];
-                            float2 p0 = at32(A.m.posf, i0), p1 = at32(A.m.posf, i1);
-                            Pay<float> v0 = at32(m.pay, i0), v1 = at32(m.pay, i1);
-                            for (int t = sub; t < n + sub; t += kSub) {
-                                const float2 p = p0;
-                                const Pay<float> v = v0;
-                                p0 = p1;
-                                v0 = v1;
-                                i1 = qu[min(t + 2 * kSub, n - 1)];
-                                p1 = at32(A.m.posf, i1);
-                                v1 = at32(m.pay, i1);
+                            // candidates sub, sub + 4, ...: three loads in flight
+                            auto one = [&](float2 p, const Pay<float>& v) {
                                 const float dx = p.x - pc.x, dy = p.y - pc.y;  // exact
                                 const float r2 = fmaf(dx, dx, dy * dy), d = fabsf(r2 - mid);
-                                const bool in = d < d_in && t < n;
+                                const bool in = d < d_in;
                                 count += in ? 1 : 0;
-                                maybe += d < d_out && t < n ? 1 : 0;
+                                maybe += d < d_out ? 1 : 0;
                                 const float u = fmaf(fmaf(dy, ax.x, -dx * ax.y), rsqrt_approx(r2), ax.z);
                                 sum.add(in ? v.a : 0.f, in ? v.b : 0.f, in ? v.w : 0.f, u);
+                            };
+                            const int its = (n + kSub - 1) / kSub;
+                            const int* q = qu + sub;
+                            int i0 = q[0], i1 = q[kSub], i2 = q[2 * kSub];
+                            float2 p0 = at32(m.posf, i0), p1 = at32(m.posf, i1), p2 = at32(m.posf, i2);
+                            Pay<float> v0 = at32(m.pay, i0), v1 = at32(m.pay, i1), v2 = at32(m.pay, i2);
+                            for (int it = 0;;) {
+                                one(p0, v0);
+                                if (++it >= its) break;
+                                i0 = q[3 * kSub];
+                                p0 = at32(m.posf, i0);
+                                v0 = at32(m.pay, i0);
+                                one(p1, v1);
+                                if (++it >= its) break;
+                                i1 = q[4 * kSub];
+                                p1 = at32(m.posf, i1);
+                                v1 = at32(m.pay, i1);
+                                one(p2, v2);
+                                if (++it >= its) break;
+                                i2 = q[5 * kSub];
+                                p2 = at32(m.posf, i2);
+                                v2 = at32(m.pay, i2);
+                                q += kAhead * kSub;
                             }
                             if (__any_sync(FULL, maybe != count)) {
                                 // rare: the candidates near an edge, by the integers
                                 for (int t = sub; t < n; t += kSub) {
-                                    const float2 p = at32(A.m.posf, qu[t]);
+                                    const float2 p = at32(m.posf, qu[t]);
                                     const Pay<float> v = at32(m.pay, qu[t]);
                                     const float dx = p.x - pc.x, dy = p.y - pc.y;
                                     const float r2 = fmaf(dx, dx, dy * dy), d = fabsf(r2 - mid);

@@ -28,6 +28,7 @@ void far_tables(int n_max, FarTables (&t)[kFarPlans], std::vector<float>* v);
 struct FarArgs {
     MomentArgs<float> m;   // bins, pointers and outputs as in the direct form
     const int32_t* order;  // rows of the centres in strip order: (strip, column, row)
+    int none;              // index of an entry of posf and pay far from every galaxy, with zero payload
     int strip_rows;        // cell rows of a strip
     int max_cols;          // columns a group may span
     int parts;             // work items a group's (bin, z) pairs are split into
