@@ -156,26 +156,31 @@ struct Tf32Split {
 // (1,1)(b1, b2) = conj(Upsilon_1,n(b2, b1)) of the triplet with Z2 and Z3 exchanged (Eqs.
 // Upsilon0_Derivation, Upsilon1-3): four components from four moment rows. N tiles hold two
 // orders n, n+1 (c = w, X_s = W_{n+s}, Y_s = W_{n+s}^*), blocks (0,0) and (1,1) only.
+// Quad tiles (8 n_bins <= 128) hold two such tiles, sides 0, 1 and 2, 3: with up to 16 bins a paired
+// tile fills half of the rows and gives half of the converter warps work, while the cost of a stage
+// is mostly its waits (five redshift bins, 15 bins, n_max 20, TF32: 13.5 ms with paired tiles, 9.5 ms).
 // Single tiles (n_bins > 32): one component per tile.
 struct TileSpec {
     int z1, z2, z3;
     int ns;              // sides with data
     int mapw;            // 0: G moments, 1: W moments
-    int ox[2], oy[2];    // order slots of X_s and Y_s
-    float xs[2], ys[2];  // +1, or -1 for the complex conjugate
+    int ox[4], oy[4];    // order slots of X_s and Y_s
+    float xs[4], ys[4];  // +1, or -1 for the complex conjugate
     float cb, cw;        // c = -w gamma_1 + i cb w gamma_2 (cw = 0), or c = w (cw = 1)
     int nblk;
-    int bl[4], br[4], bg[4], bt[4];  // block: left side, right side, group, 1 = transposed conjugate
+    int bl[8], br[8], bg[8], bt[8];  // block: left side, right side, group, 1 = transposed conjugate
 };
 
-__host__ __device__ inline int tiles_per_zt(int pair, int n_max)
+// sides: 4 (quad tiles), 2 (paired) or 1 (single)
+__host__ __device__ inline int ups_tiles(int sides, int n_max) { return sides == 4 ? (n_max + 2) / 2 : n_max + 1; }
+__host__ __device__ inline int tiles_per_zt(int sides, int n_max)
 {
-    return pair ? 2 * (n_max + 1) : 4 * (n_max + 1) + 2 * n_max + 1;
+    return sides > 1 ? ups_tiles(sides, n_max) + (2 * n_max + sides) / sides : 4 * (n_max + 1) + 2 * n_max + 1;
 }
 
-__device__ void make_tile(TileSpec& t, int tile, int pair, int nz, int n_max)
+__device__ void make_tile(TileSpec& t, int tile, int sides, int nz, int n_max)
 {
-    const int per = tiles_per_zt(pair, n_max);
+    const int per = tiles_per_zt(sides, n_max);
     const int zt = tile / per, r = tile % per;
     t.z1 = zt / (nz * nz);
     t.z2 = (zt / nz) % nz;
@@ -195,28 +200,33 @@ __device__ void make_tile(TileSpec& t, int tile, int pair, int nz, int n_max)
         t.bg[i] = g;
         t.bt[i] = tr;
     };
-    side(1, 0, 1.f, 0, 1.f);
-    if (pair && r <= n_max) {
-        const int n = r;
-        t.ns = 2;
+    for (int q = 1; q < 4; ++q) side(q, 0, 1.f, 0, 1.f);
+    const int nu = ups_tiles(sides, n_max);
+    if (sides > 1 && r < nu) {
+        t.ns = 0;
+        t.nblk = 0;
         t.mapw = 0;
-        side(0, n - 3 + offg, 1.f, -n - 3 + offg, 1.f);
-        side(1, -n - 1 + offg, -1.f, n - 1 + offg, -1.f);
         t.cb = -1.f, t.cw = 0.f;
-        t.nblk = 4;
-        block(0, 0, 0, gid(zt, 0, n), 0);
-        block(1, 0, 1, gid(zt, 3, n), 0);
-        block(2, 1, 0, gid(zt, 2, n), 0);
-        block(3, 1, 1, gid(zsw, 1, n), 1);
-    } else if (pair) {
-        const int n0 = 2 * (r - n_max - 1);
-        t.ns = min(2, 2 * n_max + 1 - n0);
+        for (int n = r * sides / 2; n < min((r + 1) * sides / 2, n_max + 1); ++n) {
+            const int s0 = t.ns, k = t.nblk;
+            side(s0, n - 3 + offg, 1.f, -n - 3 + offg, 1.f);
+            side(s0 + 1, -n - 1 + offg, -1.f, n - 1 + offg, -1.f);
+            block(k, s0, s0, gid(zt, 0, n), 0);
+            block(k + 1, s0, s0 + 1, gid(zt, 3, n), 0);
+            block(k + 2, s0 + 1, s0, gid(zt, 2, n), 0);
+            block(k + 3, s0 + 1, s0 + 1, gid(zsw, 1, n), 1);
+            t.ns += 2;
+            t.nblk += 4;
+        }
+    } else if (sides > 1) {
+        const int n0 = sides * (r - nu);
+        t.ns = min(sides, 2 * n_max + 1 - n0);
         t.mapw = 1;
         t.cb = 0.f, t.cw = 1.f;
         t.nblk = t.ns;
-        for (int s = 0; s < t.ns; ++s) {
-            side(s, n0 + s, 1.f, n0 + s, -1.f);
-            block(s, s, s, gid(zt, 4, n0 + s), 0);
+        for (int q = 0; q < t.ns; ++q) {
+            side(q, n0 + q, 1.f, n0 + q, -1.f);
+            block(q, q, q, gid(zt, 4, n0 + q), 0);
         }
     } else {
         t.ns = 1;
@@ -238,7 +248,7 @@ __device__ void make_tile(TileSpec& t, int tile, int pair, int nz, int n_max)
 struct TcArgs {
     ContractArgs<float> c;
     int groups;        // nz^3 * groups_per_zt(n_max): index space of the partial sums
-    int pair;          // 1: two sides per tile (4 nb <= 128 rows), 0: one side (2 nb <= 128)
+    int sides;         // sides of a tile: 4 (8 nb <= 128 rows), 2 (4 nb <= 128) or 1 (2 nb <= 128)
     int npad;          // MMA N: 2 nb columns per side, rounded up to 32 (8 TMEM columns per part)
     int nbp;           // bins padded to even (the moment rows)
     int fixed_slices;  // > 0: this many centre slices instead of the automatic choice
@@ -246,13 +256,13 @@ struct TcArgs {
     unsigned long long* err;
 };
 
-// one raw slot: boxes X_0 [X_1] Y_0 [Y_1], each one order row [KT centres][nbp bins] complex,
+// one raw slot: boxes X_0 .. X_{sides-1} Y_0 .. Y_{sides-1}, each one order row [KT centres][nbp bins] complex,
 // then the coefficients [KT]
 struct RawLayout {
     int box_bytes, slot_bytes, sides;
-    __host__ __device__ RawLayout(int kt, int nbp, int pair)
+    __host__ __device__ RawLayout(int kt, int nbp, int n_sides)
     {
-        sides = pair ? 2 : 1;
+        sides = n_sides;
         box_bytes = kt * nbp * 8;
         slot_bytes = ((2 * sides * box_bytes + kt * 16) + 127) / 128 * 128;
     }
@@ -282,9 +292,9 @@ constexpr int kRaw = 3;    // raw slots: the TMA copies run two stages ahead of 
 constexpr int kDqs = 129;  // floats between the columns of the block sums (rows 0..127, padded)
 
 template <class SP>
-static size_t smem_bytes(int kt, int nbp, int pair, int npad)
+static size_t smem_bytes(int kt, int nbp, int sides, int npad)
 {
-    const RawLayout R(kt, nbp, pair);
+    const RawLayout R(kt, nbp, sides);
     return (size_t)kRaw * R.slot_bytes + kStages * (size_t)Layout<SP>::STAGE_BYTES +
            (size_t)(npad / 2) * kDqs * sizeof(float);
 }
@@ -381,7 +391,7 @@ __global__ void __launch_bounds__(kThreads, 2) contract_tc_kernel(const __grid_c
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nb = A.nb, nz = A.nz, n_max = A.n_max;
     const int nbb = nb * nb, nb2 = 2 * nb, nbp = a.nbp;
-    const RawLayout R(KT, nbp, a.pair);
+    const RawLayout R(KT, nbp, a.sides);
     unsigned char* raw = smem;
     unsigned char* ops = smem + kRaw * R.slot_bytes;
     // FP32 block sums: column pair p (Re R, Im R of one bin) of row r at dq[p * kDqs + r]; even
@@ -395,7 +405,7 @@ __global__ void __launch_bounds__(kThreads, 2) contract_tc_kernel(const __grid_c
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
-        make_tile(ts, blockIdx.x, a.pair, nz, n_max);
+        make_tile(ts, blockIdx.x, a.sides, nz, n_max);
         for (int i = 0; i < kRaw; ++i) {
             mbar_init(smem_u32(&rawfull[i]), 1);
             mbar_init(smem_u32(&rawempty[i]), kConvWarps);
@@ -534,7 +544,7 @@ __global__ void __launch_bounds__(kThreads, 2) contract_tc_kernel(const __grid_c
         const int quarter = warp & 3, part = warp >> 2;
         const int row = quarter * 32 + lane;
         const int ncol = a.npad / kParts, colb = part * ncol;  // ncol: a multiple of 8
-        const float sx = ts.xs[min(row / nb2, 1)];
+        const float sx = ts.xs[min(row / nb2, 3)];
 
         // adds chain c's accumulator to dq and hands it back to the MMA warp. The lanes of the A
         // rows Re and Im of a bin are neighbours: with (e0, e1) = (A_re B_re, A_re B_im) and
@@ -557,7 +567,7 @@ __global__ void __launch_bounds__(kThreads, 2) contract_tc_kernel(const __grid_c
                 float* d = dq + cp0 * kDqs + row;
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const float sy = ts.ys[min((cp0 + j) / nb, 1)];
+                    const float sy = ts.ys[min((cp0 + j) / nb, 3)];
                     const float e = __uint_as_float(v[2 * j]);
                     const float t = __shfl_xor_sync(0xffffffffu, __uint_as_float(v[2 * j + 1]), 1);
                     d[j * kDqs] += (lane & 1) ? sy * t + sx * e : e - sx * sy * t;
@@ -776,7 +786,7 @@ template <class SP>
 static cudaError_t launch_tc(TcArgs a, float4* coef, int n_sm, int* splits_out, bool plan_only, cudaStream_t st)
 {
     const ContractArgs<float>& c = a.c;
-    const size_t smem = smem_bytes<SP>(SP::KT, a.nbp, a.pair, a.npad);
+    const size_t smem = smem_bytes<SP>(SP::KT, a.nbp, a.sides, a.npad);
     if (smem > 227 * 1024) return cudaErrorInvalidValue;
     cudaError_t e = set_smem_attr(contract_tc_kernel<SP>, smem);
     if (e != cudaSuccess) return e;
@@ -784,7 +794,7 @@ static cudaError_t launch_tc(TcArgs a, float4* coef, int n_sm, int* splits_out, 
     e = occupancy(&per_sm, contract_tc_kernel<SP>, kThreads, smem);
     if (e != cudaSuccess) return e;
     per_sm = std::max(1, std::min(per_sm, 512 / (2 * kTmemCols)));
-    const int tiles = c.nz * c.nz * c.nz * tiles_per_zt(a.pair, c.n_max);
+    const int tiles = c.nz * c.nz * c.nz * tiles_per_zt(a.sides, c.n_max);
     const int slices = a.fixed_slices > 0 ? (int)std::min<int64_t>(a.fixed_slices, std::max<int64_t>(1, c.n_centres))
                                           : pick_slices(tiles, per_sm * n_sm, c.n_centres, SP::KT);
     *splits_out = slices;
@@ -827,9 +837,17 @@ cudaError_t launch_contract_tc(const ContractArgs<float>& c, bool tf32, int n_sm
     a.c = c;
     a.groups = c.nz * c.nz * c.nz * groups_per_zt(c.n_max);
     if (2 * c.nb > tc::kM) return cudaErrorInvalidValue;
-    a.pair = 4 * c.nb <= tc::kM ? 1 : 0;
-    a.npad = (((a.pair ? 2 : 1) * 2 * c.nb + 31) / 32) * 32;
     a.nbp = nb_pad(c.nb);
+    auto use = [&](int sides) {
+        a.sides = sides;
+        a.npad = (sides * 2 * c.nb + 31) / 32 * 32;
+    };
+    use(8 * c.nb <= tc::kM ? 4 : 4 * c.nb <= tc::kM ? 2 : 1);
+    // quad tiles only while two blocks fit an SM (BF16 with 15 or 16 bins: the copy ring is too large)
+    if (a.sides == 4 && 2 * (1024 + 2048 + (tf32 ? tc::smem_bytes<tc::Tf32Split>(tc::Tf32Split::KT, a.nbp, 4, a.npad)
+                                                : tc::smem_bytes<tc::Bf16Split>(tc::Bf16Split::KT, a.nbp, 4, a.npad))) >
+                            228 * 1024)
+        use(2);
     a.err = err;
     return tf32 ? tc::launch_tc<tc::Tf32Split>(a, coef, n_sm, splits, plan_only, st)
                 : tc::launch_tc<tc::Bf16Split>(a, coef, n_sm, splits, plan_only, st);
