@@ -785,7 +785,7 @@ static unsigned grid1d(int64_t n, int n_sm)
 // faster than the block-per-centre form: about 300 + (5 + 6 SW + 4 SAB) N warp instructions a bin
 // against 300 n_max + n_max N / 2 (lines measured at n_max 10, 20 and 30 in FP32; in FP64, where a
 // warp-wide instruction takes 16 cycles, the line lies lower).
-static double near_line(int n_max, bool fp64) { return fp64 ? 100.0 : std::max(60.0, 24.0 * n_max); }
+static double near_line(int n_max, bool fp64) { return fp64 ? 100.0 : std::max(60.0, 36.0 * n_max); }
 
 // estimated warp instructions of a (centre, bin) with N neighbours, by the cheaper of those two forms
 static double small_cost(int n_max, double N)
@@ -819,7 +819,7 @@ static FarPlan plan_far(const mp3pcf_ctx* ctx, int64_t n, int64_t nc, double are
         while (b > b_lo && (double)ctx->e2q[b - 1] >= r_min * r_min) {
             // per centre: the sectors' enumeration and reduction, the FFT and orders, the pairs
             const double N = M_PI * rho * (double)(ctx->e2q[b] - ctx->e2q[b - 1]);
-            const double cost = 75.0 * t.sectors + 0.35 * t.terms * t.sectors + N * (1.25 * t.terms + 30.0) / 24.0;
+            const double cost = 150.0 * t.sectors + 0.35 * t.terms * t.sectors + N * (1.25 * t.terms + 30.0) / 24.0;
             if (cost >= small_cost(c.n_max, N)) break;
             --b;
         }

@@ -45,9 +45,10 @@ struct Plan {
     static constexpr int S = S_, PW = PW_, PAB = PAB_, PT = PW + 2 * PAB;
     static constexpr int KS = PT * kC + ((PT * kC) % 32 == 0 ? 8 : 0);  // floats per sector (bank spread)
 };
-using Wide = Plan<64, 16, 12>;    // few terms: the centre group must subtend a small angle
+using Wide = Plan<64, 18, 14>;    // few terms: the centre group must subtend a small angle
 using Middle = Plan<64, 20, 16>;
 using Close = Plan<32, 28, 20>;   // bins nearer to the group
+using Tight = Plan<32, 32, 24>;   // the nearest
 
 // cos(2 pi k / 64); folds to a literal once the loops are unrolled
 __device__ __forceinline__ float cos64(int k)
@@ -697,7 +698,7 @@ static cudaError_t launch(const FarArgs& a, int n_sm, cudaStream_t st)
 // functions J_p, p >= P, sum to half of that
 static double dmax_of(int n_max, int PW, int PAB)
 {
-    auto x = [](int P) { return P >= 28 ? 12.7 : P >= 20 ? 7.0 : P >= 16 ? 4.5 : 2.35; };
+    auto x = [](int P) { return P >= 32 ? 15.5 : P >= 28 ? 12.5 : P >= 24 ? 9.6 : P >= 20 ? 6.9 : P >= 18 ? 5.6 : P >= 16 ? 4.45 : 3.3; };
     return std::min({0.5, x(PW) / std::max(2 * n_max, 1), x(PAB) / (n_max + 3)});
 }
 
@@ -787,6 +788,7 @@ void far_tables(int n_max, FarTables (&t)[kFarPlans], std::vector<float>* v)
     far::tables<far::Wide>(n_max, &t[0], v);
     far::tables<far::Middle>(n_max, &t[1], v);
     far::tables<far::Close>(n_max, &t[2], v);
+    far::tables<far::Tight>(n_max, &t[3], v);
 }
 
 cudaError_t launch_moments_far(const FarArgs& a, int plan, int n_sm, cudaStream_t st)
@@ -794,7 +796,8 @@ cudaError_t launch_moments_far(const FarArgs& a, int plan, int n_sm, cudaStream_
     switch (plan) {
         case 0: return far::launch<far::Wide, false>(a, n_sm, st);
         case 1: return far::launch<far::Middle, false>(a, n_sm, st);
-        default: return far::launch<far::Close, false>(a, n_sm, st);
+        case 2: return far::launch<far::Close, false>(a, n_sm, st);
+        default: return far::launch<far::Tight, false>(a, n_sm, st);
     }
 }
 
@@ -803,7 +806,8 @@ cudaError_t launch_moments_far_adjoint(const FarArgs& a, int plan, int n_sm, cud
     switch (plan) {
         case 0: return far::launch<far::Wide, true>(a, n_sm, st);
         case 1: return far::launch<far::Middle, true>(a, n_sm, st);
-        default: return far::launch<far::Close, true>(a, n_sm, st);
+        case 2: return far::launch<far::Close, true>(a, n_sm, st);
+        default: return far::launch<far::Tight, true>(a, n_sm, st);
     }
 }
 

@@ -17,7 +17,7 @@ struct BinGeom {
 std::vector<BinGeom> bin_geometry(const std::vector<long long>& e2q);
 
 // tables of a context (they depend on n_max only): offsets into one float array of all variants
-constexpr int kFarPlans = 3;  // variants, widest bins first
+constexpr int kFarPlans = 4;  // variants, widest bins first
 struct FarTables {
     int sectors = 0, terms = 0;
     double dmax = 0.0, half_width = 0.0;  // largest angle from a sector's axis; half a sector
