@@ -37,7 +37,7 @@ constexpr int kWarps = 8, kThreads = kWarps * 32;
 constexpr int kC = 8;       // centres of a group
 constexpr int kSub = 4;     // candidate streams of a warp (kC * kSub = 32 lanes)
 constexpr int kQueue = 128; // candidates listed at a time per warp
-constexpr int kAhead = 3;   // candidates of a lane in flight
+constexpr int kAhead = 6;   // filler entries of a lane behind the list
 
 // S sectors, PW terms of W, PAB terms of A and B
 template <int S_, int PW_, int PAB_>
@@ -509,21 +509,28 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
                                 odd += d < d_out && !in ? 1 : 0;
                                 add(i, in && mine, fmaf(fmaf(dy, ax.x, -dx * ax.y), rsqrt_approx(r2), ax.z));
                             };
-                            const int its = (n + kSub - 1) / kSub;
                             const int* q = qu + sub;
-                            int i0 = q[0], i1 = q[kSub], i2 = q[2 * kSub];
-                            float2 p0 = at32(m.posf, i0), p1 = at32(m.posf, i1), p2 = at32(m.posf, i2);
-                            for (int it = 0;;) {
+                            int i0, i1, i2, i3;
+                            float2 p0, p1, p2, p3;
+                            auto fetch = [&](int at, int& i, float2& p) {
+                                i = q[at * kSub];
+                                p = at32(m.posf, i);
+                            };
+                            fetch(0, i0, p0);
+                            fetch(1, i1, p1);
+                            fetch(2, i2, p2);
+                            fetch(3, i3, p3);
+                            for (int rest = n; ; q += 4 * kSub) {
                                 one(i0, p0);
-                                if (++it >= its) break;
-                                p0 = at32(m.posf, i0 = q[3 * kSub]);
                                 one(i1, p1);
-                                if (++it >= its) break;
-                                p1 = at32(m.posf, i1 = q[4 * kSub]);
+                                if ((rest -= 2 * kSub) <= 0) break;
+                                fetch(4, i0, p0);
+                                fetch(5, i1, p1);
                                 one(i2, p2);
-                                if (++it >= its) break;
-                                p2 = at32(m.posf, i2 = q[5 * kSub]);
-                                q += kAhead * kSub;
+                                one(i3, p3);
+                                if ((rest -= 2 * kSub) <= 0) break;
+                                fetch(6, i2, p2);
+                                fetch(7, i3, p3);
                             }
                             if (__any_sync(FULL, odd))  // rare: the candidates near an edge, by the integers
                                 for (int t = sub; t < n + sub; t += kSub) {
@@ -542,7 +549,7 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
                         int count = 0, maybe = 0;
                         sector_batches(g, upper, sp == 0, sp == S / 2 - 1, ray[sp], ray[sp + 1], sn0, sn1, row_start, A.none, qu, lane,
                                        [&](int n) {
-                            // candidates sub, sub + 4, ...: three loads in flight
+                            // candidates sub, sub + 4, ...: two to four loads ahead
                             auto one = [&](float2 p, const Pay<float>& v) {
                                 const float dx = p.x - pc.x, dy = p.y - pc.y;  // exact
                                 const float r2 = fmaf(dx, dx, dy * dy), d = fabsf(r2 - mid);
@@ -552,28 +559,31 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
                                 const float u = fmaf(fmaf(dy, ax.x, -dx * ax.y), rsqrt_approx(r2), ax.z);
                                 sum.add(in ? v.a : 0.f, in ? v.b : 0.f, in ? v.w : 0.f, u);
                             };
-                            const int its = (n + kSub - 1) / kSub;
+                            // two at a time in one stretch of code, so that the direction of one is
+                            // formed while the other is added
                             const int* q = qu + sub;
-                            int i0 = q[0], i1 = q[kSub], i2 = q[2 * kSub];
-                            float2 p0 = at32(m.posf, i0), p1 = at32(m.posf, i1), p2 = at32(m.posf, i2);
-                            Pay<float> v0 = at32(m.pay, i0), v1 = at32(m.pay, i1), v2 = at32(m.pay, i2);
-                            for (int it = 0;;) {
+                            float2 p0, p1, p2, p3;
+                            Pay<float> v0, v1, v2, v3;
+                            auto fetch = [&](int at, float2& p, Pay<float>& v) {
+                                const int i = q[at * kSub];
+                                p = at32(m.posf, i);
+                                v = at32(m.pay, i);
+                            };
+                            fetch(0, p0, v0);
+                            fetch(1, p1, v1);
+                            fetch(2, p2, v2);
+                            fetch(3, p3, v3);
+                            for (int rest = n; ; q += 4 * kSub) {
                                 one(p0, v0);
-                                if (++it >= its) break;
-                                i0 = q[3 * kSub];
-                                p0 = at32(m.posf, i0);
-                                v0 = at32(m.pay, i0);
                                 one(p1, v1);
-                                if (++it >= its) break;
-                                i1 = q[4 * kSub];
-                                p1 = at32(m.posf, i1);
-                                v1 = at32(m.pay, i1);
+                                if ((rest -= 2 * kSub) <= 0) break;
+                                fetch(4, p0, v0);
+                                fetch(5, p1, v1);
                                 one(p2, v2);
-                                if (++it >= its) break;
-                                i2 = q[5 * kSub];
-                                p2 = at32(m.posf, i2);
-                                v2 = at32(m.pay, i2);
-                                q += kAhead * kSub;
+                                one(p3, v3);
+                                if ((rest -= 2 * kSub) <= 0) break;
+                                fetch(6, p2, v2);
+                                fetch(7, p3, v3);
                             }
                             if (__any_sync(FULL, maybe != count)) {
                                 // rare: the candidates near an edge, by the integers
