@@ -75,32 +75,106 @@ __global__ void grad_tables(const AdjArgs<T> a, int64_t n_ups_groups, int64_t to
     }
 }
 
+template <int B>
+__device__ __forceinline__ void cp_async(void* dst, const void* src)
+{
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(B) : "memory");
+}
+
+// (r, i) += t (y.x, y.y) with t's real and imaginary part apart: t y = (r.x - i.y, r.y + i.x) and
+// t conj(y) = (r.x + i.y, i.x - r.y), so the partners are staged as they lie in memory
+__device__ __forceinline__ void mac_parts(cx<float>& r, cx<float>& i, cx<float> t, cx<float> y)
+{
+    const float2 v = make_float2(y.x, y.y);
+    const float2 a = __ffma2_rn(make_float2(t.x, t.x), v, make_float2(r.x, r.y));
+    const float2 b = __ffma2_rn(make_float2(t.y, t.y), v, make_float2(i.x, i.y));
+    r = cx<float>{a.x, a.y};
+    i = cx<float>{b.x, b.y};
+}
+
+__device__ __forceinline__ void mac_parts(cx<double>& r, cx<double>& i, cx<double> t, cx<double> y)
+{
+    r.x = fma(t.x, y.x, r.x);
+    r.y = fma(t.x, y.y, r.y);
+    i.x = fma(t.y, y.x, i.x);
+    i.y = fma(t.y, y.y, i.y);
+}
+
+constexpr int kTileC = 64, kPer = 4, kAdjThreads = 320;
+
+// one role of an order slot: the gradient table at g (X role: transposed), the partner's order slot and
+// z-bin, pconj: the partner enters conjugated, mconj: this moment does
+struct Role {
+    size_t g;
+    int qp, z1, zo, kind;
+    bool is_x, pconj, mconj;
+};
+
+// role r (0..7) of order slot q and z-bin z with centres of z-bin z1 and partners of z-bin zo
+__device__ __forceinline__ bool role_of(int r, int q, int z, int z1, int zo, int nz, int nmax, int nbb, Role& o)
+{
+    const int MG = 2 * nmax + 3, NN = nmax + 1, NW = 2 * nmax + 1, of = nmax + 3;
+    o.is_x = (r & 1) == 0;
+    o.z1 = z1;
+    o.zo = zo;
+    // as X this moment is of Z2 and the partner of Z3, as Y the other way round
+    const size_t zt = o.is_x ? (size_t)(z1 * nz + z) * nz + zo : (size_t)(z1 * nz + zo) * nz + z;
+    if (q >= MG) {
+        // N_n: w W_n(b1) conj(W_n(b2))
+        const int m = q - MG;
+        o.kind = 4;
+        o.qp = m;
+        o.pconj = o.is_x;
+        o.mconj = !o.is_x;
+        o.g = ((size_t)nz * nz * nz * 4 * NN + zt * NW + m) * nbb;
+        return r < 2;
+    }
+    const int m = q - of;
+    int n, p;
+    o.kind = r >> 1;
+    switch (r) {
+        case 0: n = m + 3; p = -n - 3; break;   // kind 0: -v G_{n-3}(b1) G_{-n-3}(b2)
+        case 1: n = -m - 3; p = n - 3; break;
+        case 2: n = m + 1; p = -n - 1; break;   // kind 1: -conj(v) G_{n-1}(b1) G_{-n-1}(b2)
+        case 3: n = -m - 1; p = n - 1; break;
+        case 4: n = -m - 1; p = -n - 3; break;  // kind 2: -v conj(G_{-n-1}(b1)) G_{-n-3}(b2)
+        case 5: n = -m - 3; p = -n - 1; break;
+        case 6: n = m + 3; p = n - 1; break;    // kind 3: -v G_{n-3}(b1) conj(G_{n-1}(b2))
+        default: n = m + 1; p = n - 3; break;
+    }
+    o.qp = p + of;
+    o.pconj = r == 5 || r == 6;
+    o.mconj = r == 4 || r == 7;
+    o.g = ((zt * 4 + o.kind) * NN + n) * nbb;
+    return n >= 0 && n <= nmax;
+}
+
 // grid: x = centre tiles, y = output order slot (G slots 0..MG-1, then W slots), z = z-bin. Per role of the
 // slot (X or Y of one group, at most eight a partner z-bin) the block stages the group's dL/dy, transposed
-// for the X role, and the partner rows of its kTileC centres in shared memory; a thread owns one bin of
-// kPer centres, so a table element serves kPer products. The X role also gives the gradient of the
-// centre's own coefficient, sum_b1 conj(X(b1)) sum_b2 dL/dy conj(Y(b2)): the inner sum is the role's. It is
-// reduced over the bins and added atomically (every group has exactly one X role). 100 000 centres, 20
-// bins, n_max 30: 10.4 ms, against 22.5 with table and partner elements from global memory (4 FMAs
-// per two loads) and the coefficients' gradient in a kernel of its own that formed every inner sum
-// again.
-constexpr int kTileC = 64, kPer = 4, kAdjThreads = 512;
-
+// for the X role, and the partner rows of its kTileC centres in shared memory, the next role's while this
+// one is worked on (stages 2; 1 where two do not fit); a thread owns one bin of kPer centres, so a table
+// element serves kPer products. The X role also gives the gradient of the centre's own coefficient, sum_b1
+// conj(X(b1)) sum_b2 dL/dy conj(Y(b2)): the inner sum is the role's. It is reduced over the bins and added
+// atomically (every group has exactly one X role). Bound by shared-memory reads and issue. 100 000 centres,
+// 20 bins, n_max 30: 7.7 ms; one stage, scalar products and shared atomics 10.4; table and partner elements from
+// global memory and the coefficients' gradient in a kernel of its own 22.5.
 template <typename T>
-__global__ void __launch_bounds__(kAdjThreads) contract_adjoint_moments(const AdjArgs<T> a)
+__global__ void __launch_bounds__(kAdjThreads, sizeof(T) == 4 ? 2 : 1) contract_adjoint_moments(const AdjArgs<T> a, int stages)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int nb = a.nb, nz = a.nz, nmax = a.n_max, nbp = nb_pad(nb), nbb = nb * nb;
-    const int MG = 2 * nmax + 3, o = nmax + 3, NN = nmax + 1, NW = 2 * nmax + 1;
-    cx<T>* tab = reinterpret_cast<cx<T>*>(smem_raw);  // [nb][nb], the summed bin first
-    cx<T>* part = tab + nbb;                          // [kTileC][nb] partner rows
-    T* gc = reinterpret_cast<T*>(part + kTileC * nb);  // [kTileC][3]: dL/dv (re, im), dL/dw of the centres
+    const int nb = a.nb, nz = a.nz, nmax = a.n_max, nbp = nb_pad(nb), nbb = nb * nb, nbbp = nbb + (nbb & 1);
+    const int MG = 2 * nmax + 3;
+    // per stage: [nb][nb] table, the summed bin first, then [kTileC][nbp] partner rows
+    cx<T>* buf = reinterpret_cast<cx<T>*>(smem_raw);
+    const int stage_len = nbbp + kTileC * nbp;
+    __shared__ T gc[3 * kTileC];  // dL/dv (re, im), dL/dw of the centres
     __shared__ cx<T> s_v[kTileC];
     __shared__ T s_w[kTileC];
     __shared__ int s_z[kTileC];
     const int q = blockIdx.y, z = blockIdx.z, c0 = blockIdx.x * kTileC, nc = min(kTileC, a.n_centres - c0);
     const bool isG = q < MG;
-    const int m = isG ? q - o : q - MG;
+    const int slot = isG ? q : q - MG;
     const size_t plane = (size_t)a.n_centres * nz * nbp;
     for (int i = threadIdx.x; i < kTileC; i += blockDim.x) {
         cx<T> v{T(0), T(0)};
@@ -119,110 +193,142 @@ __global__ void __launch_bounds__(kAdjThreads) contract_adjoint_moments(const Ad
     }
     for (int i = threadIdx.x; i < 3 * kTileC; i += blockDim.x) gc[i] = T(0);
     __syncthreads();
-    const int z_lo = s_z[0], z_hi = s_z[nc - 1];  // the centres are sorted by z-bin
+    const int z_lo = s_z[0], roles = (s_z[nc - 1] - z_lo + 1) * nz * 8;  // the centres are sorted by z-bin
     const cx<T>* M = isG ? a.G : a.W;
-    cx<T>* out = isG ? a.gG + (size_t)q * plane : a.gW + (size_t)m * plane;
-    const size_t n_off = (size_t)nz * nz * nz * 4 * NN * nbb;
-    // thread -> (bin b, centres i0 .. i0 + kPer - 1), in passes over the items
-    const int groups = kTileC / kPer;
-    for (int it0 = 0; it0 < groups * nb; it0 += blockDim.x) {
+    cx<T>* out = (isG ? a.gG : a.gW) + (size_t)slot * plane;
+    // the first role from k on (roles: none)
+    auto find = [&](int k, Role& o) {
+        for (; k < roles; ++k)
+            if (role_of(k & 7, q, z, z_lo + (k >> 3) / nz, (k >> 3) % nz, nz, nmax, nbb, o)) break;
+        return k;
+    };
+    auto stage_in = [&](cx<T>* dst, const Role& o) {
+        const cx<T>* src = (o.is_x ? a.tabX : a.tabY) + o.g;
+        for (int i = threadIdx.x; i < nbb; i += blockDim.x) cp_async<sizeof(cx<T>)>(dst + i, src + i);
+        const cx<T>* pr = M + (size_t)o.qp * plane + ((size_t)c0 * nz + o.zo) * nbp;
+        cx<T>* part = dst + nbbp;
+        constexpr int E = 16 / sizeof(cx<T>);  // elements per 16 bytes
+        if (nz == 1) {                         // the rows follow one another
+            for (int i = threadIdx.x * E; i < nc * nbp; i += blockDim.x * E) cp_async<16>(part + i, pr + i);
+        } else {
+            for (int r = threadIdx.x >> 5; r < nc; r += blockDim.x >> 5)
+                for (int i = (threadIdx.x & 31) * E; i < nbp; i += 32 * E)
+                    cp_async<16>(part + r * nbp + i, pr + (size_t)r * nz * nbp + i);
+        }
+    };
+    // thread -> (bin b, centres i0 + j kTileC / kPer), in passes over the items
+    constexpr int kGroups = kTileC / kPer;
+    for (int it0 = 0; it0 < kGroups * nb; it0 += blockDim.x) {
         const int it = it0 + threadIdx.x;
-        const bool on = it < groups * nb;
-        const int b = on ? it % nb : 0, i0 = on ? it / nb * kPer : 0;
+        const bool on = it < kGroups * nb;
+        const int b = on ? it % nb : 0, i0 = on ? it / nb : 0;
         cx<T> acc[kPer], own[kPer];
-        T gr[kPer], gi[kPer], gw[kPer];
+        T gr[kPer], gi[kPer];  // the coefficient's gradient (W slots: gr, of the weight)
 #pragma unroll
         for (int j = 0; j < kPer; ++j) {
+            const int i = i0 + j * kGroups;
             acc[j] = own[j] = cx<T>{T(0), T(0)};
-            gr[j] = gi[j] = gw[j] = T(0);
-            if (on && i0 + j < nc) own[j] = M[(size_t)(isG ? q : m) * plane + ((size_t)(c0 + i0 + j) * nz + z) * nbp + b];
+            gr[j] = gi[j] = T(0);
+            if (on && i < nc) own[j] = M[(size_t)slot * plane + ((size_t)(c0 + i) * nz + z) * nbp + b];
         }
-        // one role: group table at g (X: transposed), partner order slot qp of z-bin zo, pconj: the
-        // partner enters conjugated, mconj: this moment does; kind as in the groups' list
-        auto role = [&](size_t g, bool is_x, int z1, int zo, int qp, bool pconj, bool mconj, int kind) {
-            __syncthreads();
-            const cx<T>* src = (is_x ? a.tabX : a.tabY) + g;
-            for (int i = threadIdx.x; i < nbb; i += blockDim.x) tab[i] = src[i];
-            const cx<T>* pr = M + (size_t)qp * plane + ((size_t)c0 * nz + zo) * nbp;
-            for (int i = threadIdx.x; i < nc * nb; i += blockDim.x) {
-                cx<T> y = pr[(size_t)(i / nb) * nz * nbp + i % nb];
-                if (!pconj) y.y = -y.y;  // conj(partner) (conj(conj(G)) = G when it enters conjugated)
-                part[i] = y;
+        Role cur, next;
+        int k = find(0, cur), at = 0;
+        if (k < roles) stage_in(buf, cur);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        while (k < roles) {
+            const int kn = find(k + 1, next);
+            if (stages == 2) {
+                if (kn < roles) stage_in(buf + (at ^ 1) * stage_len, next);
+                asm volatile("cp.async.commit_group;" ::: "memory");
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
             }
             __syncthreads();
-            cx<T> s[kPer];
+            const cx<T>* tab = buf + at * stage_len + b;
+            const cx<T>* part = buf + at * stage_len + nbbp + i0 * nbp;
+            cx<T> re[kPer], im[kPer];
 #pragma unroll
-            for (int j = 0; j < kPer; ++j) s[j] = cx<T>{T(0), T(0)};
-            if (on)
-                for (int b2 = 0; b2 < nb; ++b2) {
-                    const cx<T> t = tab[b2 * nb + b];
+            for (int j = 0; j < kPer; ++j) re[j] = im[j] = cx<T>{T(0), T(0)};
+            int b2 = 0;
+            for (; b2 + 1 < nb; b2 += 2) {
+                const cx<T> t0 = tab[b2 * nb], t1 = tab[(b2 + 1) * nb];
 #pragma unroll
-                    for (int j = 0; j < kPer; ++j) cfma(s[j], t, part[(i0 + j) * nb + b2]);
+                for (int j = 0; j < kPer; ++j) {
+                    const cx<T>* y = part + j * kGroups * nbp + b2;
+                    cx<T> y0, y1;
+                    if constexpr (sizeof(T) == 4) {
+                        const float4 v = *reinterpret_cast<const float4*>(y);  // nbp and b2 are even
+                        y0 = cx<T>{v.x, v.y};
+                        y1 = cx<T>{v.z, v.w};
+                    } else {
+                        y0 = y[0];
+                        y1 = y[1];
+                    }
+                    mac_parts(re[j], im[j], t0, y0);
+                    mac_parts(re[j], im[j], t1, y1);
                 }
+            }
+            if (b2 < nb) {
+                const cx<T> t = tab[b2 * nb];
+#pragma unroll
+                for (int j = 0; j < kPer; ++j) mac_parts(re[j], im[j], t, part[j * kGroups * nbp + b2]);
+            }
 #pragma unroll
             for (int j = 0; j < kPer; ++j) {
-                if (!on || s_z[i0 + j] != z1) continue;
-                const cx<T> v = s_v[i0 + j];
-                // the coefficient: -v, -conj(v) (kind 1) or w (kind 4)
-                const cx<T> cc = kind == 4 ? cx<T>{s_w[i0 + j], T(0)} : kind == 1 ? cx<T>{-v.x, -v.y} : cx<T>{-v.x, v.y};
-                const cx<T> gx = cmul(s[j], cc);  // times conj(coefficient)
-                acc[j] = cadd(acc[j], mconj ? cconj(gx) : gx);
-                if (is_x) {
-                    const cx<T> x = mconj ? own[j] : cconj(own[j]);
-                    const cx<T> p = cmul(x, s[j]);
-                    if (kind == 4) {
-                        gw[j] += p.x;  // c = w
+                const int i = i0 + j * kGroups;
+                if (!on || s_z[i] != cur.z1) continue;
+                // sum of the table and the conjugate of the partner as it enters the product
+                const cx<T> s = cur.pconj ? cx<T>{re[j].x - im[j].y, re[j].y + im[j].x}
+                                          : cx<T>{re[j].x + im[j].y, im[j].x - re[j].y};
+                const cx<T> v = s_v[i];
+                // times conj(coefficient): of w (kind 4), -conj(v) (kind 1) or -v
+                const cx<T> cc = cur.kind == 4 ? cx<T>{s_w[i], T(0)} : cx<T>{-v.x, cur.kind == 1 ? -v.y : v.y};
+                const cx<T> gx = cmul(s, cc);
+                acc[j] = cadd(acc[j], cur.mconj ? cconj(gx) : gx);
+                if (cur.is_x) {
+                    const cx<T> p = cmul(cur.mconj ? own[j] : cconj(own[j]), s);
+                    if (cur.kind == 4) {
+                        gr[j] += p.x;  // c = w
                     } else {
                         gr[j] -= p.x;  // c = -v, or -conj(v): grad v = -conj(grad c)
-                        gi[j] += kind == 1 ? p.y : -p.y;
+                        gi[j] += cur.kind == 1 ? p.y : -p.y;
                     }
                 }
             }
-        };
-        auto ub = [&](int zt, int kind, int n) { return (((size_t)zt * 4 + kind) * NN + n) * nbb; };
-        for (int z1 = z_lo; z1 <= z_hi; ++z1)
-            for (int zo = 0; zo < nz; ++zo) {
-                const int ztX = (z1 * nz + z) * nz + zo;  // this element as X (Z2 = z), partner Z3 = zo
-                const int ztY = (z1 * nz + zo) * nz + z;  // this element as Y (Z3 = z), partner Z2 = zo
-                if (isG) {
-                    int n;
-                    // kind 0: G_{n-3}(b1) G_{-n-3}(b2), coef -v
-                    n = m + 3;
-                    if (n >= 0 && n <= nmax) role(ub(ztX, 0, n), true, z1, zo, -n - 3 + o, false, false, 0);
-                    n = -m - 3;
-                    if (n >= 0 && n <= nmax) role(ub(ztY, 0, n), false, z1, zo, n - 3 + o, false, false, 0);
-                    // kind 1: G_{n-1}(b1) G_{-n-1}(b2), coef -conj(v)
-                    n = m + 1;
-                    if (n >= 0 && n <= nmax) role(ub(ztX, 1, n), true, z1, zo, -n - 1 + o, false, false, 1);
-                    n = -m - 1;
-                    if (n >= 0 && n <= nmax) role(ub(ztY, 1, n), false, z1, zo, n - 1 + o, false, false, 1);
-                    // kind 2: conj(G_{-n-1}(b1)) G_{-n-3}(b2), coef -v
-                    n = -m - 1;
-                    if (n >= 0 && n <= nmax) role(ub(ztX, 2, n), true, z1, zo, -n - 3 + o, false, true, 2);
-                    n = -m - 3;
-                    if (n >= 0 && n <= nmax) role(ub(ztY, 2, n), false, z1, zo, -n - 1 + o, true, false, 2);
-                    // kind 3: G_{n-3}(b1) conj(G_{n-1}(b2)), coef -v
-                    n = m + 3;
-                    if (n >= 0 && n <= nmax) role(ub(ztX, 3, n), true, z1, zo, n - 1 + o, true, false, 3);
-                    n = m + 1;
-                    if (n >= 0 && n <= nmax) role(ub(ztY, 3, n), false, z1, zo, n - 3 + o, false, true, 3);
-                } else {
-                    // N_n: w W_n(b1) conj(W_n(b2))
-                    role(n_off + ((size_t)ztX * NW + m) * nbb, true, z1, zo, m, true, false, 4);
-                    role(n_off + ((size_t)ztY * NW + m) * nbb, false, z1, zo, m, false, true, 4);
-                }
+            __syncthreads();
+            if (stages == 1) {
+                if (kn < roles) stage_in(buf, next);
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            } else {
+                at ^= 1;
             }
+            cur = next;
+            k = kn;
+        }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        // the bins' parts of the coefficient's gradient through shared memory, added per centre (shared
+        // atomics on one address by all bins cost more than the roles)
+        T* red = reinterpret_cast<T*>(buf);
 #pragma unroll
-        for (int j = 0; j < kPer; ++j)
-            if (on && i0 + j < nc) {
-                out[((size_t)(c0 + i0 + j) * nz + z) * nbp + b] = acc[j];
-                if (isG) {
-                    atomicAdd(&gc[3 * (i0 + j)], gr[j]);
-                    atomicAdd(&gc[3 * (i0 + j) + 1], gi[j]);
-                } else {
-                    atomicAdd(&gc[3 * (i0 + j) + 2], gw[j]);
-                }
+        for (int j = 0; j < kPer; ++j) {
+            const int i = i0 + j * kGroups;
+            if (on && i < nc) {
+                out[((size_t)(c0 + i) * nz + z) * nbp + b] = acc[j];
+                red[i * nb + b] = gr[j];
+                if (isG) red[(kTileC + i) * nb + b] = gi[j];
             }
+        }
+        __syncthreads();
+        for (int e = threadIdx.x; e < (isG ? 2 : 1) * kTileC; e += blockDim.x) {
+            const int i = e % kTileC, first = (i % kGroups) * nb;  // the centre's first item
+            if (i >= nc) continue;
+            T sum = T(0);
+            for (int b2 = max(0, it0 - first); b2 < min(nb, it0 + (int)blockDim.x - first); ++b2) sum += red[e * nb + b2];
+            gc[3 * i + (isG ? e / kTileC : 2)] += sum;
+        }
+        __syncthreads();
     }
     __syncthreads();
     for (int i = threadIdx.x; i < 3 * nc; i += blockDim.x)
@@ -662,12 +768,15 @@ static cudaError_t run(const AdjArgs<T>& a, int64_t n, const int* perm, const fl
         const int64_t nU = z3 * 4 * (a.n_max + 1), tot = (nU + z3 * (2 * a.n_max + 1)) * nbb;
         grad_tables<T><<<(unsigned)std::min<int64_t>((tot + 255) / 256, (int64_t)n_sm * 16), 256, 0, st>>>(a, nU, tot);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        const size_t sm_mom = sizeof(cx<T>) * ((size_t)nbb + (size_t)kTileC * a.nb) + sizeof(T) * 3 * kTileC;
+        // two stages where they leave room for two blocks on an SM
+        const size_t stage = sizeof(cx<T>) * ((size_t)nbb + (nbb & 1) + (size_t)kTileC * nb_pad(a.nb));
+        const int stages = stage <= 54 * 1024 ? 2 : 1;
+        const size_t sm_mom = stages * stage;
         if ((e = set_smem_attr(contract_adjoint_moments<T>, sm_mom)) != cudaSuccess) return e;
         // threads: the items in as few, equally full passes as kAdjThreads allows
         const int items = kTileC / kPer * a.nb, passes = (items + kAdjThreads - 1) / kAdjThreads;
         const int threads = ((items + passes - 1) / passes + 31) / 32 * 32;
-        contract_adjoint_moments<T><<<g1d, threads, sm_mom, st>>>(a);
+        contract_adjoint_moments<T><<<g1d, threads, sm_mom, st>>>(a, stages);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         const size_t sm_pair = sizeof(cx<T>) * (size_t)kPairWarps * (a.nz * (MG + MW) + kQueue) +
                                sizeof(int) * (size_t)kPairWarps * kQueue;
