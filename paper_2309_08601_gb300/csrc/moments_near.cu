@@ -2,12 +2,15 @@
 //
 // The block-per-centre form spends some 9000 warp instructions per (centre, bin) on barriers, range
 // set-up, half-empty batches and the reduction over lanes, whatever the bin holds. Here a warp works
-// on a centre by itself and its lanes are the orders: lane l keeps W_m, A_m and B_m of
-// m = l, l + 32, ... The warp tests 32 candidates at a time, one per lane; once 32 members are found
-// (or the bin ends) the lanes store the powers of their directions, and the members are added one
-// after the other, every lane forming its own z^m from two of the stored powers. About 27 warp
-// instructions a member at n_max = 30, no reduction, no barrier; the direct form's 14 a member plus its
-// overhead are less from a few hundred members on. The order of the sums is fixed.
+// on a centre by itself and its lanes are the orders: lane l of either half keeps W_m, A_m and B_m of
+// m = l, l + 16, ... The warp tests 32 candidates at a time, one per lane; once 32 members are found
+// (or the bin ends) the lanes store the powers of their directions, and the members are added two at a
+// time, one by each half, every lane stepping from z^l by z^16: about 16 warp instructions a member at
+// n_max = 30, no barrier, one exchange between the halves at a bin's end. (All 32 lanes on one member took
+// 27, as 34 and 61 orders fill two words of 32 badly and each power was a product first: 20 000 galaxies,
+// 20 bins, n_max 30 4.69 -> 4.43 ms, 3 000 galaxies, 10 bins, n_max 10 0.233 -> 0.221.) The direct form's
+// 14 a member plus its overhead are less from a few hundred members on. Bound by issue and the latency of
+// the chains in small bins. The order of the sums is fixed.
 #include <algorithm>
 
 #include "moments_far.cuh"
@@ -18,6 +21,7 @@ namespace mp3 {
 namespace near {
 
 constexpr int kQueue = 128;
+static_assert(kMaxNmax <= 55, "launch() needs more orders a lane");
 
 // warps of a block (the stored powers take 3.3 KB a warp in FP32) and blocks per SM the registers are
 // sized for
@@ -44,13 +48,35 @@ __device__ __forceinline__ cx<double> direction(float dx, float dy, double)
     return {x * inv, y * inv};
 }
 
-template <typename T>
-__device__ __forceinline__ void cacc(cx<T>& s, T v, cx<T> c)
+__device__ __forceinline__ void cacc(cx<float>& s, float v, cx<float> c)
 {
-    s.x += v * c.x;
-    s.y += v * c.y;
+    const float2 r = __ffma2_rn(make_float2(v, v), make_float2(c.x, c.y), make_float2(s.x, s.y));
+    s = cx<float>{r.x, r.y};
+}
+__device__ __forceinline__ void cacc(cx<double>& s, double v, cx<double> c)
+{
+    s.x = fma(v, c.x, s.x);
+    s.y = fma(v, c.y, s.y);
 }
 
+// stored powers of a member: z^0..z^16; in FP64 with up to 32 orders all of them, as an FP64 instruction
+// takes 16 cycles whatever the number of lanes that need it
+template <typename T, int SW>
+struct Powers {
+    static constexpr bool kAll = sizeof(T) == 8 && SW <= 2;
+    static constexpr int kPow = kAll ? 16 * SW + 1 : 17;
+};
+
+// the halves' sums of x[2 k] and x[2 k + 1], the even one to the lower half, the odd one to the upper
+template <typename T, int S>
+__device__ __forceinline__ cx<T> exchange(const cx<T> (&x)[S], int k, bool upper)
+{
+    const cx<T> even = x[2 * k], odd = 2 * k + 1 < S ? x[2 * k + 1 < S ? 2 * k + 1 : 0] : cx<T>{T(0), T(0)};
+    const cx<T> keep = upper ? odd : even, send = upper ? even : odd;
+    return {keep.x + __shfl_xor_sync(0xffffffffu, send.x, 16), keep.y + __shfl_xor_sync(0xffffffffu, send.y, 16)};
+}
+
+// SW, SAB: orders of W and of A, B a lane
 template <typename T, int SW, int SAB>
 __global__ void __launch_bounds__(Block<T>::kThreads, Block<T>::kMin) near_moments_kernel(const NearArgs<T> A)
 {
@@ -58,16 +84,13 @@ __global__ void __launch_bounds__(Block<T>::kThreads, Block<T>::kMin) near_momen
     constexpr unsigned FULL = 0xffffffffu;
     const MomentArgs<T>& m = A.m;
     __shared__ BinGeom bins[kMaxBins];
-    // stored powers of a member: z^0..z^7, z^0, z^8, z^16, z^24, z^32, of which a lane forms its own by a
-    // product; in FP64 with up to 31 orders all of them, as an FP64 instruction takes 16 cycles whatever the
-    // number of lanes that need it
-    constexpr bool kAll = sizeof(T) == 8 && SW == 1;
-    constexpr int kPow = kAll ? 33 : 13;
+    constexpr bool kAll = Powers<T, SW>::kAll;
+    constexpr int kPow = Powers<T, SW>::kPow;
     extern __shared__ __align__(16) unsigned char smem_raw[];  // powers [kWarps][32 kPow]
     __shared__ int queue[kWarps][kQueue], founds[kWarps][64];
     __shared__ Member<T> mem[kWarps][32];
     const int mtop = max(2 * A.m.n_max, A.m.n_max + 3);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, half = lane >> 4;
     const unsigned lt_mask = (1u << lane) - 1u;
     const int nz = m.nz, n_max = m.n_max;
     const size_t plane = (size_t)m.n_centres * nz * m.nbp;
@@ -106,51 +129,36 @@ __global__ void __launch_bounds__(Block<T>::kThreads, Block<T>::kMin) near_momen
                 for (int s = 0; s < SAB; ++s) aa[s] = ab[s] = cx<T>{T(0), T(0)};
                 // the first cnt members found: their powers by the lanes, then one member after the other
                 auto add_members = [&](int cnt) {
-                    if (lane < cnt) {
-                        const int i = found[lane];
+                    if (lane < cnt + (cnt & 1)) {  // an odd last one is paired with itself at weight zero
+                        const int i = found[min(lane, cnt - 1)];
                         const float2 p = A.m.posf[i];
                         const Pay<T> v = m.pay[i];
-                        V[lane] = Member<T>{v.a, v.b, v.w, T(0)};
+                        V[lane] = lane < cnt ? Member<T>{v.a, v.b, v.w, T(0)} : Member<T>{T(0), T(0), T(0), T(0)};
                         const cx<T> z1 = direction(p.x - pc.x, p.y - pc.y, T(0));
                         cx<T>* q = P + lane * kPow;
-                        const cx<T> z2 = cmul(z1, z1), z4 = cmul(z2, z2), z3 = cmul(z2, z1);
-                        q[0] = cx<T>{T(1), T(0)};
-                        q[1] = z1;
-                        q[2] = z2;
-                        q[3] = z3;
-                        q[4] = z4;
-                        const cx<T> z5 = cmul(z4, z1), z6 = cmul(z4, z2), z7 = cmul(z4, z3), z8 = cmul(z4, z4);
-                        q[5] = z5;
-                        q[6] = z6;
-                        q[7] = z7;
-                        if constexpr (kAll) {  // every power up to the highest order
-                            cx<T> lo[8] = {q[0], z1, z2, z3, z4, z5, z6, z7}, hi = z8;
+                        cx<T> lo[8];
+                        lo[0] = cx<T>{T(1), T(0)};
+                        lo[1] = z1;
 #pragma unroll
-                            for (int k = 8; k < kPow; ++k) {
-                                if (k > mtop) break;
-                                if (k % 8 == 0 && k > 8) hi = cmul(hi, z8);
-                                q[k] = k % 8 == 0 ? hi : cmul(hi, lo[k % 8]);
-                            }
-                        } else {
-                            const cx<T> z16 = cmul(z8, z8);
-                            q[8] = cx<T>{T(1), T(0)};
-                            q[9] = z8;
-                            q[10] = z16;
-                            q[11] = cmul(z16, z8);
-                            if (SW > 1) q[12] = cmul(z16, z16);
+                        for (int k = 2; k < 8; ++k) lo[k] = cmul(lo[k / 2], lo[k - k / 2]);
+                        cx<T> hi = cmul(lo[4], lo[4]);
+                        const cx<T> z8 = hi;
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) q[k] = lo[k];
+#pragma unroll
+                        for (int k = 8; k < kPow; ++k) {
+                            if (kAll && k > mtop) break;
+                            if (k % 8 == 0 && k > 8) hi = cmul(hi, z8);
+                            q[k] = k % 8 == 0 ? hi : cmul(hi, lo[k % 8]);
                         }
                     }
                     __syncwarp();
                     my_pairs += cnt;
+                    const cx<T>* q = P + half * kPow;
 #pragma unroll 2
-                    for (int j = 0; j < cnt; ++j) {
-                        const cx<T>* q = P + j * kPow;
+                    for (int j = half; j < cnt + half; j += 2, q += 2 * kPow) {
                         const Member<T> v = V[j];
-                        cx<T> zc;
-                        if constexpr (kAll)
-                            zc = q[min(lane, mtop)];
-                        else
-                            zc = cmul(q[lane & 7], q[8 + (lane >> 3)]);
+                        cx<T> zc = q[lane & 15];
 #pragma unroll
                         for (int s = 0; s < SW; ++s) {
                             cacc(aw[s], v.w, zc);
@@ -158,7 +166,7 @@ __global__ void __launch_bounds__(Block<T>::kThreads, Block<T>::kMin) near_momen
                                 cacc(aa[s], v.a, zc);
                                 cacc(ab[s], v.b, zc);
                             }
-                            if (s + 1 < SW) zc = cmul(zc, q[12]);
+                            if (s + 1 < SW) zc = kAll ? q[(lane & 15) + 16 * (s + 1)] : cmul(zc, q[16]);
                         }
                     }
                     __syncwarp();
@@ -219,11 +227,13 @@ __global__ void __launch_bounds__(Block<T>::kThreads, Block<T>::kMin) near_momen
                 if (nm > 0) add_members(nm);
                 const size_t row = ((size_t)c * nz + z) * m.nbp + b;
 #pragma unroll
-                for (int s = 0; s < SW; ++s) {
-                    const int mm = lane + 32 * s;
-                    if (mm <= 2 * n_max) m.W[(size_t)mm * plane + row] = aw[s];
-                    if (s < SAB) {
-                        const cx<T> a = aa[s < SAB ? s : 0], bb = ab[s < SAB ? s : 0];
+                for (int k = 0; k < (SW + 1) / 2; ++k) {
+                    const int mm = lane + 32 * k;
+                    const cx<T> wm = exchange(aw, k, half != 0);
+                    if (mm <= 2 * n_max) m.W[(size_t)mm * plane + row] = wm;
+                    if (2 * k < SAB) {
+                        const int ka = 2 * k < SAB ? k : 0;
+                        const cx<T> a = exchange(aa, ka, half != 0), bb = exchange(ab, ka, half != 0);
                         if (mm <= n_max - 1) m.G[(size_t)(mm + n_max + 3) * plane + row] = cx<T>{a.x - bb.y, a.y + bb.x};
                         if (mm >= 1 && mm <= n_max + 3)
                             m.G[(size_t)(n_max + 3 - mm) * plane + row] = cx<T>{a.x + bb.y, bb.x - a.y};
@@ -242,7 +252,7 @@ template <typename T, int SW, int SAB>
 static cudaError_t launch(NearArgs<T> a, int n_sm, cudaStream_t st)
 {
     constexpr int kWarps = Block<T>::kWarps, kThreads = Block<T>::kThreads;
-    const size_t smem = sizeof(cx<T>) * kWarps * 32 * (sizeof(T) == 8 && SW == 1 ? 33 : 13);
+    const size_t smem = sizeof(cx<T>) * kWarps * 32 * Powers<T, SW>::kPow;
     int per_sm = 0;
     cudaError_t e = set_smem_attr(near_moments_kernel<T, SW, SAB>, smem);
     if (e != cudaSuccess) return e;
@@ -260,12 +270,15 @@ static cudaError_t launch(NearArgs<T> a, int n_sm, cudaStream_t st)
 template <typename T>
 static cudaError_t dispatch(const NearArgs<T>& a, int n_sm, cudaStream_t st)
 {
-    const int sw = std::max(2 * a.m.n_max, a.m.n_max + 3) / 32 + 1, sab = (a.m.n_max + 3) / 32 + 1;
+    // orders 0 .. max(2 n_max, n_max + 3) of W and 0 .. n_max + 3 of A, B, 16 lanes
+    const int sw = std::max(2 * a.m.n_max, a.m.n_max + 3) / 16 + 1, sab = (a.m.n_max + 3) / 16 + 1;
     if (sw == 1) return launch<T, 1, 1>(a, n_sm, st);
     if (sw == 2 && sab == 1) return launch<T, 2, 1>(a, n_sm, st);
     if (sw == 2) return launch<T, 2, 2>(a, n_sm, st);
     if (sw == 3) return launch<T, 3, 2>(a, n_sm, st);
-    return launch<T, 4, 2>(a, n_sm, st);
+    if (sw == 4) return launch<T, 4, 3>(a, n_sm, st);
+    if (sw <= 6) return launch<T, 6, 4>(a, n_sm, st);
+    return launch<T, 7, 4>(a, n_sm, st);  // kMaxNmax is 50
 }
 
 }  // namespace near
