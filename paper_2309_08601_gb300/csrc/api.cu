@@ -782,16 +782,19 @@ static unsigned grid1d(int64_t n, int n_sm)
 }
 
 // Expected neighbours of a (centre, bin) below which the warp-per-centre form (moments_near.cu) is
-// faster than the block-per-centre form: about 300 + (5 + 6 SW + 4 SAB) N warp instructions a bin
-// against 300 n_max + n_max N / 2 (lines measured at n_max 10, 20 and 30 in FP32; in FP64, where a
-// warp-wide instruction takes 16 cycles, the line lies lower).
-static double near_line(int n_max, bool fp64) { return fp64 ? 100.0 : std::max(60.0, 36.0 * n_max); }
+// faster than the block-per-centre form. FP32: about 300 + 16 N warp instructions a bin against 300 n_max +
+// n_max N / 2 at n_max 30; the line is flat (36 to 150 n_max: within 1 %). FP64: both form about as many of the
+// 16-cycle instructions a member, the block-per-centre form has its reduction on top. Lines at 100, 400,
+// 800, 1600, 3200 neighbours: 12 000 galaxies, n_max 10 14.6, 14.3, 14.23, 14.20, 14.19 ms, six catalogs in
+// three z-bins 55.2, 54.0, 52.95, 52.96, 53.0; 20 000 galaxies up to 40', n_max 20 164.5, 164.4, -, 165.4, 167.5,
+// n_max 30 263, 260, -, 258.6, 258.0.
+static double near_line(int n_max, bool fp64) { return fp64 ? 1000.0 : std::max(60.0, 36.0 * n_max); }
 
 // estimated warp instructions of a (centre, bin) with N neighbours, by the cheaper of those two forms
 static double small_cost(int n_max, double N)
 {
-    const int sw = std::max(2 * n_max, n_max + 3) / 32 + 1, sab = (n_max + 3) / 32 + 1;
-    return std::min(300.0 + (5 + 6 * sw + 4 * sab) * N, 300.0 * n_max + 0.5 * n_max * N);
+    const int sw = std::max(2 * n_max, n_max + 3) / 16 + 1, sab = (n_max + 3) / 16 + 1;
+    return std::min(300.0 + (2.0 + 2.5 * sw + sab) * N, 300.0 * n_max + 0.5 * n_max * N);
 }
 
 static FarPlan plan_far(const mp3pcf_ctx* ctx, int64_t n, int64_t nc, double area, double carea, int b_lo, int b_hi)
