@@ -1283,7 +1283,7 @@ mp3pcf_status mp3pcf_contract_multipoles(mp3pcf_ctx* ctx, double* d_upsilon, dou
             ctx->launches[ST_CONTRACT] += 1;
             MP3_CK(launch_contract_diag(a, ctx->st));
         }
-        MP3_CK(launch_contract_reduce(ctx->partial.as<double>(), splits, nz, nb, c.n_max, d_upsilon, d_norm,
+        MP3_CK(launch_contract_reduce(ctx->partial.as<double>(), splits, nz, nb, c.n_max, false, d_upsilon, d_norm,
                                       ctx->st));
         if (c.exclude_degenerate) return degenerate_t<float>(ctx, d_upsilon, d_norm);
         return MP3PCF_OK;
@@ -1308,7 +1308,8 @@ mp3pcf_status mp3pcf_contract_multipoles(mp3pcf_ctx* ctx, double* d_upsilon, dou
         e = launch_contract_f32(a, ctx->st);
     }
     MP3_CK(e);
-    MP3_CK(launch_contract_reduce(ctx->partial.as<double>(), splits, nz, nb, c.n_max, d_upsilon, d_norm, ctx->st));
+    MP3_CK(launch_contract_reduce(ctx->partial.as<double>(), splits, nz, nb, c.n_max, ctx->fp64, d_upsilon, d_norm,
+                                  ctx->st));
     if (c.exclude_degenerate)
         return ctx->fp64 ? degenerate_t<double>(ctx, d_upsilon, d_norm) : degenerate_t<float>(ctx, d_upsilon, d_norm);
     return MP3PCF_OK;

@@ -131,7 +131,7 @@ cudaError_t launch_contract_tc(const ContractArgs<float>& a, bool tf32, int n_sm
 // exclude_degenerate with a tensor-core form: recomputes the b1 = b2 slice partials of the
 // Z-triplets with Z2 = Z3 in FP64 (a.partial, a.splits as filled by launch_contract_tc)
 cudaError_t launch_contract_diag(const ContractArgs<float>& a, cudaStream_t st);
-cudaError_t launch_contract_reduce(const double* partial, int splits, int nz, int nb, int n_max,
+cudaError_t launch_contract_reduce(const double* partial, int splits, int nz, int nb, int n_max, bool mirror,
                                    double* ups, double* norm, cudaStream_t st);
 
 // ------------------------------------------------------------------ post-processing (FP64)
