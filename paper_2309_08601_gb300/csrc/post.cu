@@ -1069,8 +1069,8 @@ __global__ void __launch_bounds__(kM3Threads) map3_sum_kernel(const PostArgs p, 
         for (int a = 0; a < kMapGroup; ++a)
             if (a < na) {
                 const cx<double> v = f[(size_t)a * 4 * pts + t];
-                acc[a][0] += g.x * v.x - g.y * v.y;
-                acc[a][1] += g.x * v.y + g.y * v.x;
+                acc[a][0] = fma(g.x, v.x, fma(-g.y, v.y, acc[a][0]));  // two FP64 instructions each, not three
+                acc[a][1] = fma(g.x, v.y, fma(g.y, v.x, acc[a][1]));
             }
     }
     __shared__ double red[kM3Threads / 32][kMapGroup * 2];
