@@ -38,7 +38,6 @@ UNIT = "pair-accumulations/s"
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2070e6 / 1e12
 PEAK_NOTE = "152 SMs x 128 FP32 lanes x 2 flop/FMA x 2070 MHz (derived from unit counts and clock)"
 DEFAULT_WORKLOAD = "masked_lognormal_1m"
-MOMENT_KERNEL_NMAX = (4, 10, 20, 30, 40, 50)  # compiled order sets of moments_kernel<T, NMAX>
 
 
 def _measured_hbm_gbs():
@@ -55,26 +54,12 @@ HBM_PEAK_GBS, HBM_PEAK_NOTE = _measured_hbm_gbs()
 # the same density (the traffic of both kernels is proportional to the centres); None until the
 # kernel has been captured since its last change.
 TRAFFIC_BYTES = {
-    # moments_kernel<float,40>: capture at 100 000 galaxies of the same density, x10
-    # (profiles/moments_kernel_masked_lognormal_100k.md)
-    ("moments", "masked_lognormal_1m"): 10 * (630.813440e6 + 4.473916e9),
-    # moments_kernel<float,30>: capture at 50 000 galaxies of the same density, x4
-    # (profiles/moments_kernel_lognormal_50k.md)
-    ("moments", "lognormal_200k"): 4 * (147.244544e6 + 1.073786e9),
     # contract_tc_kernel<Bf16Split>: captures at 50 000 galaxies of each density, x20 and x4
     # (profiles/contract_tc_bf16x3_traffic_50k.md)
     ("contract", "masked_lognormal_1m"): 20 * (1.981240576e9 + 35.888640e6),
     ("contract", "lognormal_200k"): 4 * (993.852928e6 + 19.601408e6),
 }
 TRAFFIC_NOTE = "ncu dram__bytes_read.sum + dram__bytes_write.sum per launch (profiles/)"
-
-
-def compiled_nmax(n_max: int) -> int:
-    """n_max of the moment kernel instantiation that serves n_max (the smallest compiled set)."""
-    for k in MOMENT_KERNEL_NMAX:
-        if n_max <= k:
-            return k
-    raise ValueError("n_max above the compiled range")
 
 
 def flops_per_pair(n_max: int) -> int:
@@ -85,12 +70,16 @@ def flops_per_pair(n_max: int) -> int:
     return 15 + 6 * 2 * n_max + 8 * (2 * n_max + 3) + 4 * (2 * n_max + 1)
 
 
-def kernel_flops_per_pair(n_max: int) -> int:
-    """The flops the moment kernel's own formulation needs per pair (fewer than the plain form:
-    with real weights, G_m and G_-m come from the same two real sums A_m = sum w g1 z^m and
-    B_m = sum w g2 z^m): unit vector (6), powers z^2..z^{2 n_max} (6 each), A_m and B_m for
-    m <= n_max + 3 (4 each), W_m for m <= 2 n_max (4 each)."""
-    return 6 + 6 * (2 * n_max - 1) + 8 * (n_max + 4) + 4 * (2 * n_max + 1)
+def kernel_flops_per_pair(n_max: int, precision: str) -> int:
+    """The fewest flops that the moment kernels spend on a pair. FP32: the sector form with its shortest
+    series (moments_far.cu): the Chebyshev polynomials of the angle (18) and three real series (18 terms
+    of w, 14 of w g1 and of w g2), a multiply-add each, and the geometry (6), whatever n_max; narrower
+    bins take more. FP64: per pair and order as the direct form counts them (with real weights, G_m and
+    G_-m come from the same two real sums A_m = sum w g1 z^m and B_m = sum w g2 z^m): unit vector (6),
+    powers z^2..z^{2 n_max} (6 each), A_m and B_m for m <= n_max + 3 (4 each), W_m for m <= 2 n_max (4
+    each)."""
+    direct = 6 + 6 * (2 * n_max - 1) + 8 * (n_max + 4) + 4 * (2 * n_max + 1)
+    return direct if precision == "fp64" else min(direct, 6 + 2 * (18 + 18 + 2 * 14))
 
 
 class ClockSampler:
@@ -582,18 +571,19 @@ def time_steps(step, steps, stream):
 
 
 def moment_roofline(name, n_max, pairs, k1_ms, precision, peaks):
-    """Roofline of stage (a) on the FP32 FMA pipe: algorithmic flops (the plain form of
-    Eq. Gn_disc, flops_per_pair) x pairs per launch / launch time, against the derived peak;
-    the kernel's own flop count and the measured probe peaks are reported beside it."""
-    fpp = flops_per_pair(n_max)
+    """Roofline of stage (a) on the FP32 FMA pipe: the fewest flops that the kernels spend on a pair
+    x pairs per launch / time of the stage, against the derived peak. The rate of the plain form of
+    Eq. Gn_disc (flops_per_pair), which the sector form does not carry out, is reported beside it."""
+    fpp = kernel_flops_per_pair(n_max, precision)
     achieved = fpp * pairs / (k1_ms / 1e3) / 1e12
-    kfl = kernel_flops_per_pair(n_max) * pairs / (k1_ms / 1e3) / 1e12
-    r = {"bound": "alu", "kernel": "moments_kernel<float,%d>" % compiled_nmax(n_max), "achieved": achieved,
+    plain = flops_per_pair(n_max)
+    kernel = "moments_kernel, near_moments_kernel" + ("" if precision == "fp64" else ", far_moments_kernel")
+    r = {"bound": "alu", "kernel": kernel, "achieved": achieved,
          "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": achieved / FP32_PEAK_TFLOPS,
          "traffic": TRAFFIC_BYTES.get(("moments", name)) if precision != "fp64" else None,
          "traffic_note": TRAFFIC_NOTE, "flops_per_pair": fpp, "pairs_per_launch": pairs,
-         "kernel_flops_per_pair": kernel_flops_per_pair(n_max),
-         "frac_kernel_flops": kfl / FP32_PEAK_TFLOPS, "launch_ms": k1_ms, "peak_source": PEAK_NOTE}
+         "plain_form_flops_per_pair": plain, "plain_form_tflops": plain * pairs / (k1_ms / 1e3) / 1e12,
+         "launch_ms": k1_ms, "peak_source": PEAK_NOTE}
     if peaks:
         meas = max(peaks["fp32_fma_tflops"], peaks["fp32_ffma2_tflops"])
         r["peak_measured"] = meas

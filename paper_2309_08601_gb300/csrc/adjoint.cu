@@ -12,7 +12,7 @@
 //   grad Y_i(b2) = conj(c_i) sum_b1 grad y(b1, b2) conj(X_i(b1)),
 //   grad c_i     = sum_b1 conj(X_i(b1)) sum_b2 grad y(b1, b2) conj(Y_i(b2)),
 // with an extra conjugation where the moment enters conjugated. dL/dG and dL/dW are gathered per
-// output moment element (each written once, no atomics): an element receives the X or Y role of
+// output moment element (each written once): an element receives the X or Y role of
 // at most eight (component, n) groups.
 //
 // Stage (a): G_m(i, b) = sum_k v_k e^{i m phi_ik} and W_m(i, b) = sum_k w_k e^{i m phi_ik}, so
@@ -23,7 +23,8 @@
 // z = e^{i phi} for m < 0), one neighbour per lane, and added to the neighbour's gradient with
 // atomics (the gradient is therefore not bit-reproducible). Neighbours are found per bin from
 // the cell grid of the forward pass: for every cell row, the one or two runs of cells that meet
-// the annulus.
+// the annulus. The bins that the forward took by angular sectors go through the transpose of that
+// form instead (far_moments_kernel<PL, 1>, moments_far.cu).
 #include <math.h>
 
 #include <algorithm>

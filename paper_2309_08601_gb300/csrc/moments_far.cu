@@ -18,8 +18,8 @@
 // centre and the order of the sums is fixed (reproducible run to run).
 //
 // Measured with the narrow bins in moments_near.cu, moments of the whole call: 200 000 galaxies, 20
-// bins to 120', n_max 30: 314 -> 101 ms; 10 000 centres of 400 000 galaxies, 30 bins to 240',
-// n_max 40: 98.5 -> 26 ms. The candidate loop is 80 % of it, bound by issue (64 %) and the FMA and
+// bins to 120', n_max 30: 314 -> 84 ms; 10 000 centres of 400 000 galaxies, 30 bins to 240',
+// n_max 40: 98.5 -> 19 ms. The candidate loop is 80 % of it, bound by issue (64 %) and the FMA and
 // ALU pipes (50 % each); the loads of the next candidates come from L2.
 #include <math.h>
 
