@@ -371,8 +371,10 @@ __global__ void k_gather(int64_t n, const int* __restrict__ perm, const int32_t*
     for (int64_t d = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; d < n;
          d += (int64_t)gridDim.x * blockDim.x) {
         const int i = perm[d];
-        if (d == 0) {  // the sector form's filler entry: twice the largest extent away
-            posf[n] = make_float2(67108864.0f, 67108864.0f);
+        if (d == 0) {
+            // the sector form's filler entry, beyond every bin: edges are below 3e9 quanta (config_valid),
+            // and its r^2 = 2e36 is finite in FP32
+            posf[n] = make_float2(1e18f, 1e18f);
             pay[n] = Pay<T>{T(0), T(0), T(0), T(0)};
         }
         pos[d] = make_int2(xq[i], yq[i]);
