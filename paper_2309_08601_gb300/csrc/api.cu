@@ -340,22 +340,83 @@ __global__ void k_scatter(int64_t n, const int* __restrict__ key, const int* __r
     }
 }
 
-// atomics leave the order inside a cell arbitrary; restore increasing galaxy index so that the
-// whole pipeline is deterministic
-__global__ void k_cell_order(int64_t K, const int* __restrict__ start, int* __restrict__ perm)
+// Ascending order of v[0 .. n) by the whole block: bitonic network in the form whose comparators all put
+// the smaller value first, so that entries beyond n need not exist. Four pairs a thread at a time, as the
+// pairs of a pass are disjoint and the loads' latency is what it waits for.
+__device__ void block_sort(int* v, int n)
 {
-    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < K;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        const int a = start[c], b = start[c + 1];
-        for (int i = a + 1; i < b; ++i) {
-            const int v = perm[i];
-            int j = i - 1;
-            while (j >= a && perm[j] > v) {
-                perm[j + 1] = perm[j];
-                --j;
+    auto pass = [&](int pairs, auto pair) {
+        for (int t0 = threadIdx.x; t0 < pairs; t0 += 4 * (int)blockDim.x) {
+            int i[4], j[4], x[4], y[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int t = t0 + q * (int)blockDim.x;
+                i[q] = j[q] = n;
+                if (t < pairs) pair(t, i[q], j[q]);
+                x[q] = y[q] = 0;
+                if (j[q] < n) {
+                    x[q] = v[i[q]];
+                    y[q] = v[j[q]];
+                }
             }
-            perm[j + 1] = v;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (x[q] > y[q]) {
+                    v[i[q]] = y[q];
+                    v[j[q]] = x[q];
+                }
         }
+        __syncthreads();
+    };
+    for (int h = 1; h < n; h *= 2) {
+        pass((n + 2 * h - 1) / (2 * h) * h, [&](int t, int& i, int& j) {
+            const int b = t / h * 2 * h, o = t % h;
+            i = b + o;
+            j = b + 2 * h - 1 - o;
+        });
+        for (int s = h / 2; s > 0; s /= 2)
+            pass((n + 2 * s - 1) / (2 * s) * s, [&](int t, int& i, int& j) {
+                i = t / s * 2 * s + t % s;
+                j = i + s;
+            });
+    }
+}
+
+// atomics leave the order inside a cell arbitrary; restore increasing galaxy index so that the
+// whole pipeline is deterministic. A cell of up to kLightCell entries is sorted by insertion by one
+// thread (a few entries in a field of even density), a fuller one by the block: a distant outlier or
+// a steep cluster can put the whole catalog into one cell, where insertion takes n^2 / 4 dependent steps
+// (200 000 entries: 10^10). The direct estimator of 200 000 galaxies, 900 apertures x 3 triples, with one
+// galaxy at the far end of the fixed-point range takes 34 ms with the network (even field: 1.9).
+constexpr int kLightCell = 64;
+
+__global__ void __launch_bounds__(256) k_cell_order(int64_t K, const int* __restrict__ start, int* perm)
+{
+    __shared__ int heavy[256], n_heavy;
+    for (int64_t c0 = blockIdx.x * (int64_t)blockDim.x; c0 < K; c0 += (int64_t)gridDim.x * blockDim.x) {
+        if (threadIdx.x == 0) n_heavy = 0;
+        __syncthreads();
+        const int64_t c = c0 + threadIdx.x;
+        const int a = c < K ? start[c] : 0, b = c < K ? start[c + 1] : 0;
+        if (b - a > kLightCell) {
+            heavy[atomicAdd(&n_heavy, 1)] = threadIdx.x;
+        } else {
+            for (int i = a + 1; i < b; ++i) {
+                const int v = perm[i];
+                int j = i - 1;
+                while (j >= a && perm[j] > v) {
+                    perm[j + 1] = perm[j];
+                    --j;
+                }
+                perm[j + 1] = v;
+            }
+        }
+        __syncthreads();
+        for (int h = 0; h < n_heavy; ++h) {
+            const int64_t cell = c0 + heavy[h];
+            block_sort(perm + start[cell], start[cell + 1] - start[cell]);
+        }
+        __syncthreads();
     }
 }
 

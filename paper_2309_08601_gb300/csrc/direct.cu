@@ -94,6 +94,11 @@ __global__ void __launch_bounds__(kDirThreads) map3_direct_kernel(int64_t n, con
 // galaxies. Bound by FP64 arithmetic on the galaxies inside (two FP64 lanes per SM and cycle), so a
 // radius that occurs twice in a triple is evaluated once, and equal radii need three powers of one
 // factor. 200 000 galaxies, 900 apertures x 3 triples: 67.5 ms by scanning the catalog, 2.7 ms by cells.
+// A row with more than kDirLong galaxies in the circle (a strip, an outlier that makes the cells huge, a
+// cluster) is left to the whole block, which would else wait for the one warp that has it. Uneven fields of
+// 200 000 galaxies, by scanning and by cells: an outlier 50 and 34 ms, a strip 79 and 12, a cluster 23 and 7.5.
+constexpr int kDirLong = 1024;
+
 template <int R>  // distinct radii of the triple: 1 (all equal), 2 (the first two equal) or 3
 __device__ __forceinline__ void direct_sums(double (&s)[14], const double (&b)[3], double gt)
 {
@@ -133,13 +138,18 @@ __device__ __forceinline__ void direct_cells(double (&s)[14], const int2* __rest
     const double is = 1.0 / (double)g.side, xc = (cx / quantum - (double)g.x0) * is, yc = (cy / quantum - (double)g.y0) * is;
     const double rc = (rcut / quantum + 2.0) * is * (1.0 + 1e-9);
     const int iy0 = (int)fmin(fmax(floor(yc - rc), 0.0), (double)g.ncy), iy1 = (int)fmax(fmin(floor(yc + rc), (double)g.ncy - 1.0), -1.0);
-    for (int iy = iy0 + warp; iy <= iy1; iy += kDirThreads / 32) {
+    // the run [k0, k1) of row iy
+    auto run = [&](int iy, int& k0, int& k1) {
+        k0 = k1 = 0;
         const double dy = fmax(fmax((double)iy - yc, yc - (double)iy - 1.0), 0.0);
         const double hx = sqrt(fmax(rc * rc - dy * dy, 0.0)) + 1e-6 * rc;
         const int ix0 = (int)fmin(fmax(floor(xc - hx), 0.0), (double)g.ncx), ix1 = (int)fmax(fmin(floor(xc + hx), (double)g.ncx - 1.0), -1.0);
-        if (ix0 > ix1) continue;
-        const int k1 = start[iy * g.ncx + ix1 + 1];
-        for (int k = start[iy * g.ncx + ix0] + lane; k < k1; k += 32) {
+        if (ix0 > ix1) return;
+        k0 = start[iy * g.ncx + ix0];
+        k1 = start[iy * g.ncx + ix1 + 1];
+    };
+    auto add = [&](int k0, int k1, int first, int step) {
+        for (int k = k0 + first; k < k1; k += step) {
             const int2 p = pos[k];
             const double dx = (double)p.x * quantum - cx, dyk = (double)p.y * quantum - cy;
             const double r2 = dx * dx + dyk * dyk;
@@ -154,6 +164,24 @@ __device__ __forceinline__ void direct_cells(double (&s)[14], const int2* __rest
                 b[l] = wr * nrm[i] * exp(-r2 * inv2[i]);
             }
             direct_sums<R>(s, b, gt);
+        }
+    };
+    bool later = false;
+    for (int iy = iy0 + warp; iy <= iy1; iy += kDirThreads / 32) {
+        int k0, k1;
+        run(iy, k0, k1);
+        if (k1 - k0 > kDirLong)
+            later = true;
+        else
+            add(k0, k1, lane, 32);
+    }
+    if (!__syncthreads_or(later)) return;
+    for (int r0 = iy0; r0 <= iy1; r0 += 32) {
+        int k0 = 0, k1 = 0;
+        if (r0 + lane <= iy1) run(r0 + lane, k0, k1);
+        for (unsigned m = __ballot_sync(0xffffffffu, k1 - k0 > kDirLong); m; m &= m - 1) {
+            const int l = __ffs(m) - 1;
+            add(__shfl_sync(0xffffffffu, k0, l), __shfl_sync(0xffffffffu, k1, l), threadIdx.x, kDirThreads);
         }
     }
 }
