@@ -16,7 +16,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "common.cuh"
-#include "moments_far.cuh"
+#include "moments_plan.cuh"
 
 namespace mp3 {
 
@@ -549,14 +549,6 @@ using namespace mp3;
 
 // ------------------------------------------------------------------ context
 
-// The sector form of the moments (moments_far.cu) for the bins [b_far, b_hi): groups of kFarGroup
-// centres in strips of `rows` cell rows and at most `cols` columns, on cells of side `side`.
-struct FarPlan {
-    int b_far = 0, rows = 1, cols = 1;
-    int b[kFarPlans + 1] = {0};  // bins [b[v + 1], b[v]) take variant v (b[0] = b_hi)
-    double side = 1.0;
-};
-
 struct mp3pcf_ctx {
     mp3pcf_config cfg;
     cudaStream_t st = nullptr;
@@ -844,57 +836,6 @@ static unsigned grid1d(int64_t n, int n_sm)
     return (unsigned)(g < 1 ? 1 : g);
 }
 
-// Expected neighbours of a (centre, bin) below which the warp-per-centre form (moments_near.cu) is
-// faster than the block-per-centre form. FP32: about 300 + 16 N warp instructions a bin against 300 n_max +
-// n_max N / 2 at n_max 30; the line is flat (36 to 150 n_max: within 1 %). FP64: both form about as many of the
-// 16-cycle instructions a member, the block-per-centre form has its reduction on top. Lines at 100, 400,
-// 800, 1600, 3200 neighbours: 12 000 galaxies, n_max 10 14.6, 14.3, 14.23, 14.20, 14.19 ms, six catalogs in
-// three z-bins 55.2, 54.0, 52.95, 52.96, 53.0; 20 000 galaxies up to 40', n_max 20 164.5, 164.4, -, 165.4, 167.5,
-// n_max 30 263, 260, -, 258.6, 258.0.
-static double near_line(int n_max, bool fp64) { return fp64 ? 1000.0 : std::max(60.0, 36.0 * n_max); }
-
-// estimated warp instructions of a (centre, bin) with N neighbours, by the cheaper of those two forms
-static double small_cost(int n_max, double N)
-{
-    const int sw = std::max(2 * n_max, n_max + 3) / 16 + 1, sab = (n_max + 3) / 16 + 1;
-    return std::min(300.0 + (2.0 + 2.5 * sw + sab) * N, 300.0 * n_max + 0.5 * n_max * N);
-}
-
-static FarPlan plan_far(const mp3pcf_ctx* ctx, int64_t n, int64_t nc, double area, double carea, int b_lo, int b_hi)
-{
-    const mp3pcf_config& c = ctx->cfg;
-    FarPlan f;
-    f.b_far = b_hi;
-    if (nc < 1 || n >= (1 << 27)) return f;  // 32-bit byte offsets into the sorted catalog
-    const double rho = (double)n / c.n_z / area;  // galaxies per quantum^2 and z-bin
-    const double occ = c.cell_occupancy > 0 ? (double)c.cell_occupancy : 1.0;
-    f.side = std::max(1.0, std::max(sqrt(occ / rho), sqrt(area * c.n_z / (double)(1 << 26))));
-    const double per_cell = (double)nc / carea * f.side * f.side;  // centres
-    f.rows = (int)std::min(4.0, std::max(1.0, floor(sqrt(8.0 / per_cell) + 0.5)));
-    f.cols = (int)std::min(5.0, ceil(8.0 / (per_cell * f.rows)) + 1.0);
-    // sparse centres would leave most lanes of a group empty
-    if (per_cell * f.rows * f.cols < 4.0) return f;
-    // the direction from a centre to a galaxy differs from the sector's axis by at most half a
-    // sector plus the angle the cell's and the group's extents subtend
-    const double reach = f.side * (0.7072 + 0.5 * sqrt((double)f.rows * f.rows + (double)f.cols * f.cols)) + 8.0;
-    int b = b_hi;
-    f.b[0] = b_hi;
-    for (int v = 0; v < kFarPlans; ++v) {
-        const FarTables& t = ctx->far[v];
-        const double r_min = t.dmax > t.half_width ? reach / sin(t.dmax - t.half_width) : 1e300;
-        while (b > b_lo && (double)ctx->e2q[b - 1] >= r_min * r_min) {
-            // per centre: the sectors' enumeration and reduction, the FFT and orders, the pairs
-            const double N = M_PI * rho * (double)(ctx->e2q[b] - ctx->e2q[b - 1]);
-            const double cost = 150.0 * t.sectors + 0.35 * t.terms * t.sectors + N * (1.25 * t.terms + 30.0) / 24.0;
-            if (cost >= small_cost(c.n_max, N)) break;
-            --b;
-        }
-        f.b[v + 1] = b;
-    }
-    f.b_far = b;
-    return f;
-}
-
 // arguments of variant v for its bins (false: none); a: the whole range's, from bin b_lo
 static bool far_args(mp3pcf_ctx* ctx, const MomentArgs<float>& a, const FarPlan& fp, int v, int b_lo, FarArgs* f)
 {
@@ -1001,32 +942,28 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
         return fail(ctx, MP3PCF_EINVAL, "patch extent must be below 2^24 position quanta");
     }
 
-    // ---- cell grid: ~4 galaxies per cell and bin, and at most kMaxRows rows per annulus of the
-    // bins of the direct form; the sector form takes bins [b_far, b_hi) (plan_far)
+    // ---- the forms of the bins and the cell grid
     const int64_t nc64 = mask ? hb[9] : n;
-    const double area = (double)(ex + 1) * (double)(ey + 1);
-    const double occ = c.cell_occupancy > 0 ? (double)c.cell_occupancy : 4.0;
-    double side = sqrt(area * occ / std::max(1.0, (double)n / nz));
-    FarPlan fp;
-    fp.b_far = b_hi;
-    if constexpr (sizeof(T) == 4) {
-        const double carea = mask ? (double)((long long)hb[7] - hb[5] + 1) * (double)((long long)hb[8] - hb[6] + 1) : area;
-        fp = plan_far(ctx, n, nc64, area, carea, b_lo, b_hi);
-        if (fp.b_far < b_hi) side = fp.side;
-    }
+    MomentsPlanInput in;
+    in.n_max = c.n_max;
+    in.nz = nz;
+    in.fp64 = ctx->fp64;
+    in.occupancy = c.cell_occupancy;
+    in.e2q = ctx->e2q.data();
+    in.b_lo = b_lo;
+    in.b_hi = b_hi;
+    in.n = n;
+    in.nc = nc64;
+    in.area = (double)(ex + 1) * (double)(ey + 1);
+    in.carea = mask ? (double)((long long)hb[7] - hb[5] + 1) * (double)((long long)hb[8] - hb[6] + 1) : in.area;
+    const MomentsPlan plan = plan_moments(in);
+    const FarPlan& fp = plan.far;
+    const int b_near = plan.b_near;
     ctx->fplan = fp;
-    int b_near = b_lo;
-    while (b_near < fp.b_far &&
-           M_PI * (double)n / nz / area * (double)(ctx->e2q[b_near + 1] - ctx->e2q[b_near]) < near_line(c.n_max, ctx->fp64))
-        ++b_near;
-    const double R = sqrt((double)ctx->e2q[fp.b_far]);
-    side = std::max(side, (2.0 * R + 16.0) / (kMaxRows - 4));
-    side = std::max(side, sqrt(area * nz / (double)(1 << 26)));
-    side = std::max(side, 1.0);
     GridDesc g;
     g.x0 = bb[0];
     g.y0 = bb[1];
-    g.side = (int32_t)ceil(side);
+    g.side = (int32_t)ceil(plan.side);
     g.ncx = (int32_t)(ex / g.side + 1);
     g.ncy = (int32_t)(ey / g.side + 1);
     g.ncells = g.ncx * g.ncy;

@@ -9,7 +9,7 @@
 // its sector's sums M_{s,p} (about 25 packed FMAs at n_max = 30), and per (centre, bin) a real FFT over the sectors and a
 // short sum over p give every order:
 //   W_m = e^{i pi m / S} sum_p i^{p mod 2} c_{m,p} F_{m,p},  F_{m,p} = sum_s M_{s,p} e^{2 pi i m s / S}.
-// delta_max follows from n_max, PW and PAB so that the dropped terms stay below 3e-8 (sector_dmax), so
+// delta_max follows from n_max, PW and PAB so that the dropped terms stay below 3e-8 (far_dmax), so
 // the result differs from the direct form's by FP32 rounding only.
 //
 // A block of eight warps works on a group of up to eight neighbouring centres; a warp takes a sector
@@ -26,7 +26,7 @@
 #include <algorithm>
 #include <vector>
 
-#include "moments_far.cuh"
+#include "moments_plan.cuh"
 #include "sector.cuh"
 
 namespace mp3 {
@@ -45,10 +45,8 @@ struct Plan {
     static constexpr int S = S_, PW = PW_, PAB = PAB_, PT = PW + 2 * PAB;
     static constexpr int KS = PT * kC + ((PT * kC) % 32 == 0 ? 8 : 0);  // floats per sector (bank spread)
 };
-using Wide = Plan<64, 18, 14>;    // few terms: the centre group must subtend a small angle
-using Middle = Plan<64, 20, 16>;
-using Close = Plan<32, 28, 20>;   // bins nearer to the group
-using Tight = Plan<32, 32, 24>;   // the nearest
+template <int V>
+using Variant = Plan<kFarSectors[V], kFarPW[V], kFarPAB[V]>;
 
 // cos(2 pi k / 64); folds to a literal once the loops are unrolled
 __device__ __forceinline__ float cos64(int k)
@@ -703,25 +701,13 @@ static cudaError_t launch(const FarArgs& a, int n_sm, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// largest angle from a sector's axis for which the terms beyond PW (PAB) of every order up to
-// 2 n_max (n_max + 3) stay below 3e-8: m delta_max <= x(P), the argument at which the Bessel
-// functions J_p, p >= P, sum to half of that
-static double dmax_of(int n_max, int PW, int PAB)
-{
-    auto x = [](int P) { return P >= 32 ? 15.5 : P >= 28 ? 12.5 : P >= 24 ? 9.6 : P >= 20 ? 6.9 : P >= 18 ? 5.6 : P >= 16 ? 4.45 : 3.3; };
-    return std::min({0.5, x(PW) / std::max(2 * n_max, 1), x(PAB) / (n_max + 3)});
-}
-
-template <class PL>
+template <int V>
 static void tables(int n_max, FarTables* t, std::vector<float>* out)
 {
+    using PL = Variant<V>;
     constexpr int S = PL::S, K = 48;  // K Chebyshev nodes, symmetric: half of them are needed
-    const double dmax = dmax_of(n_max, PL::PW, PL::PAB), sd = sin(dmax);
+    const double sd = sin(far_dmax(n_max, V));
     const int mtop = std::max(2 * n_max, n_max + 3);
-    t->sectors = S;
-    t->terms = PL::PT;
-    t->dmax = dmax;
-    t->half_width = M_PI / S;
     t->off_ray = (int)out->size();
     t->off_sin = t->off_ray + S / 2 + 4;
     t->off_axis = (t->off_sin + S + 3) / 4 * 4;
@@ -795,29 +781,29 @@ std::vector<BinGeom> bin_geometry(const std::vector<long long>& e2q)
 
 void far_tables(int n_max, FarTables (&t)[kFarPlans], std::vector<float>* v)
 {
-    far::tables<far::Wide>(n_max, &t[0], v);
-    far::tables<far::Middle>(n_max, &t[1], v);
-    far::tables<far::Close>(n_max, &t[2], v);
-    far::tables<far::Tight>(n_max, &t[3], v);
+    far::tables<0>(n_max, &t[0], v);
+    far::tables<1>(n_max, &t[1], v);
+    far::tables<2>(n_max, &t[2], v);
+    far::tables<3>(n_max, &t[3], v);
 }
 
 cudaError_t launch_moments_far(const FarArgs& a, int plan, int n_sm, cudaStream_t st)
 {
     switch (plan) {
-        case 0: return far::launch<far::Wide, false>(a, n_sm, st);
-        case 1: return far::launch<far::Middle, false>(a, n_sm, st);
-        case 2: return far::launch<far::Close, false>(a, n_sm, st);
-        default: return far::launch<far::Tight, false>(a, n_sm, st);
+        case 0: return far::launch<far::Variant<0>, false>(a, n_sm, st);
+        case 1: return far::launch<far::Variant<1>, false>(a, n_sm, st);
+        case 2: return far::launch<far::Variant<2>, false>(a, n_sm, st);
+        default: return far::launch<far::Variant<3>, false>(a, n_sm, st);
     }
 }
 
 cudaError_t launch_moments_far_adjoint(const FarArgs& a, int plan, int n_sm, cudaStream_t st)
 {
     switch (plan) {
-        case 0: return far::launch<far::Wide, true>(a, n_sm, st);
-        case 1: return far::launch<far::Middle, true>(a, n_sm, st);
-        case 2: return far::launch<far::Close, true>(a, n_sm, st);
-        default: return far::launch<far::Tight, true>(a, n_sm, st);
+        case 0: return far::launch<far::Variant<0>, true>(a, n_sm, st);
+        case 1: return far::launch<far::Variant<1>, true>(a, n_sm, st);
+        case 2: return far::launch<far::Variant<2>, true>(a, n_sm, st);
+        default: return far::launch<far::Variant<3>, true>(a, n_sm, st);
     }
 }
 

@@ -18,9 +18,11 @@ std::vector<BinGeom> bin_geometry(const std::vector<long long>& e2q);
 
 // tables of a context (they depend on n_max only): offsets into one float array of all variants
 constexpr int kFarPlans = 4;  // variants, widest bins first
+// Their sectors, terms of W, terms of A and B. Widest: few terms, the centre group must subtend a small
+// angle; last: the bins nearest to the group.
+constexpr int kFarSectors[kFarPlans] = {64, 64, 32, 32}, kFarPW[kFarPlans] = {18, 20, 28, 32},
+              kFarPAB[kFarPlans] = {14, 16, 20, 24};
 struct FarTables {
-    int sectors = 0, terms = 0;
-    double dmax = 0.0, half_width = 0.0;  // largest angle from a sector's axis; half a sector
     int off_ray = 0, off_sin = 0, off_axis = 0, off_rot = 0, off_coef = 0;
 };
 void far_tables(int n_max, FarTables (&t)[kFarPlans], std::vector<float>* v);

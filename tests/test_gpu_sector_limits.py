@@ -1,7 +1,8 @@
 """The sector form of the moments (csrc/moments_far.cu) at the limits of its plan: binnings, fields and
 orders at the edge of what a context accepts. Pair counts are whole numbers and equal to the FP64 form's
 (which has no sectors). Tolerances, normwise against FP64: 1e-4 for gradients, the differentiation form's in
-FP32."""
+FP32; moments of sector bins 1e-5 (a direction in FP32 is off by at most 1.5 2^-24, an order m <= 100 by m times
+that, 9e-6; the dropped Chebyshev terms add 3e-8)."""
 import numpy as np
 import pytest
 import torch
@@ -47,3 +48,41 @@ def test_a_bin_wider_than_any_extent(gpu):
     assert out["fp32"][0] == out["fp64"][0]
     for a, b in zip(out["fp32"][1:], out["fp64"][1:]):
         assert rel_err(a, b) < 1e-4
+
+
+@pytest.mark.parametrize("n_max, lo, bins", [(50, 200.0, 2), (45, 200.0, 4)])
+def test_first_bin_hundreds_of_cells_away(gpu, n_max, lo, bins):
+    """8.6 galaxies per arcmin^2, bins from 200' (590 cells) up, half of the patch with few centres, so that
+    groups extend over all the rows and columns allowed: cells and groups must be as narrow as the expansion in
+    the angle from a sector's axis assumes. One galaxy of every bin carries weight, near the y axis (a sector's
+    boundary) as seen from the groups, so each moment is that galaxy's phase and an error of its direction
+    shows in full."""
+    rng = np.random.default_rng(n_max)
+    width, height = 60.0, 860.0
+    n = int(8.6 * width * height)
+    xy = rng.uniform(0, 1, (n, 2)) * [width, height]
+    with gpu.Estimator(bins, lo, 400.0, n_max) as est:
+        edges, _ = est.bin_edges()
+    cat = hand_catalog(xy, 0.3 * np.exp(1j * rng.uniform(0, 2 * np.pi, n)), np.ones(n))
+    dev = gpu.catalog_to_device(cat)
+    x, y = xy.T
+    share = np.where((x > 5) & (x < 25), 0.6, np.where((x > 30) & (x < 50), 0.066, 0.0))
+    mask = (np.abs(y - 0.5 * height) < 30.0) & (rng.uniform(size=n) < share)
+    mask = torch.as_tensor(mask.astype(np.uint8)).cuda()
+    worst = 0.0
+    for x0 in (36.5, 43.5):
+        w = np.zeros(n, np.float32)
+        for i in range(bins):
+            at = [x0, 0.5 * height + (-1) ** i * (edges[i] + 33.0)]
+            w[np.argmin(np.hypot(*(xy - at).T))] = 1.0
+        w = torch.as_tensor(w).cuda()
+        out = {}
+        for precision in ("fp64", "fp32"):
+            with gpu.Estimator(bins, lo, 400.0, n_max, precision=precision) as est:
+                est.accumulate_moments(*dev[:4], w, centre_mask=mask)
+                out[precision] = [est.counts(), *est.moments()]
+        assert out["fp32"][0] == out["fp64"][0]
+        for a, b, unit in zip(out["fp32"][1:], out["fp64"][1:], (0.3, 1.0)):
+            worst = max(worst, float((a.to(torch.complex128) - b).abs().max()) / unit)
+    print(n_max, lo, bins, worst)
+    assert worst < 1e-5
