@@ -954,6 +954,7 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
     in.b_hi = b_hi;
     in.n = n;
     in.nc = nc64;
+    in.extent = (double)(std::max(ex, ey) + 1);
     in.area = (double)(ex + 1) * (double)(ey + 1);
     in.carea = mask ? (double)((long long)hb[7] - hb[5] + 1) * (double)((long long)hb[8] - hb[6] + 1) : in.area;
     const MomentsPlan plan = plan_moments(in);

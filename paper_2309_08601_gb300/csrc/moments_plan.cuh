@@ -25,6 +25,7 @@ struct MomentsPlanInput {
     const long long* e2q;  // all bins' squared edges
     int b_lo, b_hi;        // bins computed
     int64_t n, nc;         // galaxies, centres
+    double extent;         // the longer side of the galaxies' extent, quanta
     double area, carea;    // of the extents of the galaxies and of the centres, quanta^2
 };
 
@@ -107,7 +108,8 @@ inline MomentsPlan plan_moments(const MomentsPlanInput& in)
 {
     MomentsPlan p;
     const double occ = in.occupancy > 0 ? (double)in.occupancy : 4.0;
-    double least = std::max(1.0, sqrt(in.area * in.nz / (double)(1 << 26)));
+    // at most 2^26 cells and 2^22 - 4 columns or rows: the column arithmetic of sector.cuh (near_int) is FP32
+    double least = std::max({1.0, sqrt(in.area * in.nz / (double)(1 << 26)), in.extent / (double)((1 << 22) - 5)});
     for (;;) {
         p.far = plan_far(in, least);
         const bool sectors = p.far.b_far < in.b_hi;

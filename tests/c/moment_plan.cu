@@ -26,6 +26,7 @@ int main(int argc, char** argv)
         in.fp64 = rng() % 8 == 0;
         in.occupancy = rng() % 2 ? 0 : 1 + rng() % 64;
         const double ex = floor(logu(1.0, 16777215.0)), ey = rng() % 3 ? ex : floor(logu(1.0, 16777215.0));
+        in.extent = std::max(ex, ey) + 1.0;
         in.area = (ex + 1.0) * (ey + 1.0);
         in.n = (int64_t)logu(1.0, 2e7);
         in.nc = (int64_t)ceil(in.n * logu(1e-3, 1.0));
@@ -45,6 +46,7 @@ int main(int argc, char** argv)
         if (!(in.b_lo <= p.b_near && p.b_near <= f.b_far && f.b_far <= in.b_hi)) return printf("ranges of bins\n"), 1;
         const double side = ceil(p.side);
         if (side < 1.0 || (ex / side) * (ey / side) * in.nz > 2.0 * (1 << 26) + ex + ey) return printf("too many cells\n"), 1;
+        if (floor(in.extent / side) + 2.0 >= (1 << 22)) return printf("columns beyond near_int's range\n"), 1;
         if ((2.0 * sqrt((double)e2[f.b_far]) + 16.0) / side > kMaxRows - 4) return printf("more cell rows than listed\n"), 1;
         if (f.b_far == in.b_hi) continue;
         if (in.fp64 || f.b[0] != in.b_hi || f.b[kFarPlans] != f.b_far) return printf("ranges of variants\n"), 1;

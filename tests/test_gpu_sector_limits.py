@@ -86,3 +86,22 @@ def test_first_bin_hundreds_of_cells_away(gpu, n_max, lo, bins):
             worst = max(worst, float((a.to(torch.complex128) - b).abs().max()) / unit)
     print(n_max, lo, bins, worst)
     assert worst < 1e-5
+
+
+def test_line_over_the_whole_extent(gpu):
+    """2.2e6 galaxies on a line of 2^24 quanta: without a limit the grid would have 5.6e6 columns, more than
+    the FP32 column arithmetic holds. Pair counts of the three forms against sorted positions."""
+    rng = np.random.default_rng(8)
+    n, q = 2_200_000, 2.0 ** -13
+    x = np.sort(rng.integers(0, 2 ** 24 - 1, n)).astype(np.int64)
+    x[0], x[-1] = 0, 2 ** 24 - 1
+    ones = torch.ones(n).cuda()
+    dev = [torch.as_tensor(rng.permutation(x).astype(np.int32)).cuda(), torch.zeros(n, dtype=torch.int32).cuda(), ones, ones, ones]
+    for b0, b1 in ((5.0, 21.5), (21.5, 92.8), (92.8, 400.0)):  # narrow, middle and sector bins
+        for precision in ("fp32", "fp64"):
+            with gpu.Estimator(1, b0 * q, b1 * q, 10, precision=precision, cell_occupancy=1) as est:
+                e2 = est.bin_edges()[1]
+                lo, hi = (int(np.ceil(np.sqrt(float(e)))) for e in e2)  # dx^2 in [e2_0, e2_1), dx >= lo, dx < hi
+                want = 2 * int((np.searchsorted(x, x + hi) - np.searchsorted(x, x + lo)).sum())
+                est.accumulate_moments(*dev)
+                assert est.counts() == (n, want), (b0, precision)
