@@ -199,7 +199,7 @@ __device__ __forceinline__ bool toeplitz_solve4(const cx<double>* t, const cx<do
     }
     cx<double> p = t[0], ip = crecip(p);
     const double p0 = p.x * p.x + p.y * p.y, floor2 = kToeplitzFloor * kToeplitzFloor * p0;
-    bool good = p0 > 0.0 && p0 < 1e300;
+    bool good = p0 > 1e-280 && p0 < 1e300;  // 1 / |p|^2 stays in range (the elimination scales its divisions)
     if (l == 0) {
         f[0] = b[0] = cx<double>{1.0, 0.0};
 #pragma unroll
