@@ -128,12 +128,16 @@ __device__ __forceinline__ cx<double> coupling(const PostArgs& p, const cx<doubl
 
 // ---- the same by the Toeplitz structure: N_{l-n} depends on l - n only, so the Levinson recursion (the
 // forward and backward vectors of the leading blocks, extended by one row at a time) solves the four
-// right-hand sides in about 6 D^2 complex multiply-adds instead of D^3 / 3 (toeplitz_solve4). Without pivoting it is as accurate
-// as elimination while the leading blocks stay well conditioned, which holds for sums of neighbour
-// weights (a positive definite matrix) in filled bins: a system whose pivots fall below kToeplitzFloor of
-// the first one, or whose reflection coefficients leave [0, 10], is listed for the pivoted elimination.
+// right-hand sides in about 6 D^2 complex multiply-adds instead of D^3 / 3 (toeplitz_solve4). It does not pivot, so its
+// error grows with the leading blocks' conditioning where elimination's follows the system's own. Each step multiplies
+// the norm of the inverse by at most (1 + |k|) / (1 - |k|), k the larger of the two reflection coefficients; a
+// system whose product exceeds kToeplitzGrowth is listed for the pivoted elimination. Systems of sums over
+// neighbours in filled bins are diagonally dominant: of 2000 galaxies, of 100 000 and of 125 triplets of five
+// z-bins all products are below 1100. Against extended precision, 500 random systems below the line, n_max 5 to
+// 50: the recursion's error is at most 7e-14, elimination's 4e-14; above it the recursion is off by 4 to 6 times
+// as much as elimination in the median and up to 80 times (couplings concentrated in angle, few neighbours).
 // FP64-bound. 125 triplets, 20 x 20 bins, n_max 30 (50 000 systems): 170 -> 16 ms.
-constexpr double kToeplitzFloor = 1e-4;
+constexpr float kToeplitzGrowth = 1e4f;
 constexpr int kToepWarps = 4, kToepSystems = 2 * kToepWarps;  // half a warp per system
 
 __device__ __forceinline__ cx<double> shfl16(cx<double> v, int src)
@@ -198,7 +202,8 @@ __device__ __forceinline__ bool toeplitz_solve4(const cx<double>* t, const cx<do
         for (int mu = 0; mu < 4; ++mu) x[mu][r] = cx<double>{0.0, 0.0};
     }
     cx<double> p = t[0], ip = crecip(p);
-    const double p0 = p.x * p.x + p.y * p.y, floor2 = kToeplitzFloor * kToeplitzFloor * p0;
+    const double p0 = p.x * p.x + p.y * p.y;
+    float growth = 1.f;
     bool good = p0 > 1e-280 && p0 < 1e300;  // 1 / |p|^2 stays in range (the elimination scales its divisions)
     if (l == 0) {
         f[0] = b[0] = cx<double>{1.0, 0.0};
@@ -226,8 +231,10 @@ __device__ __forceinline__ bool toeplitz_solve4(const cx<double>* t, const cx<do
             const cx<double> ae = cmul(al, e[1]);
             p = csub(p, ae);
             ip = crecip(p);
-            const double pp = p.x * p.x + p.y * p.y, aa = al.x * al.x + al.y * al.y, bb = be.x * be.x + be.y * be.y;
-            good = good && pp >= floor2 && pp < 1e300 && aa < 100.0 && bb < 100.0;
+            const double aa = al.x * al.x + al.y * al.y, bb = be.x * be.x + be.y * be.y;
+            const float refl = sqrtf((float)fmax(aa, bb));
+            growth *= (1.f + refl) / (1.f - refl);
+            good = good && aa < 1.0 && bb < 1.0 && growth < kToeplitzGrowth;  // false for NaN
             const cx<double> na{-al.x, -al.y}, nbt{-be.x, -be.y};
             cx<double> d[4], w[R];
 #pragma unroll
