@@ -77,6 +77,16 @@ struct DevBuf {
     }
 };
 
+// part of another buffer
+struct DevSlice {
+    void* p = nullptr;
+    template <typename U>
+    U* as() const
+    {
+        return reinterpret_cast<U*>(p);
+    }
+};
+
 // ------------------------------------------------------------------ a0: cell sort kernels
 
 // fixed-extent mode: every position inside [x0, x1] x [y0, y1] and zbin < nz, else bit 4 of err
@@ -571,10 +581,12 @@ struct mp3pcf_ctx {
     // fault injection on the host side (tests of failure detection): see mp3pcf_inject
     bool inject_wait_timeout = false, inject_alloc_failure = false;
     cudaEvent_t batch_ev[2] = {nullptr, nullptr};
-    DevBuf d_edges, d_nodes;
-    DevBuf bb, key, count, fill, scan_sums, scan_total, perm, pos, pay, zs;
+    // made by mp3pcf_create, in one allocation
+    DevBuf fixed;
+    DevSlice d_edges, d_nodes, bingeom, bb, pairs, singular, edgelist;
+    DevBuf key, count, fill, scan_sums, scan_total, perm, pos, pay, zs;
     DevBuf cflag, crank, oflag, orank, centre_idx, crow;
-    DevBuf G, W, pairs, partial, singular, edgelist, m3partial, m3filter, m3four, ccoef;
+    DevBuf G, W, partial, m3partial, m3filter, m3four, ccoef;
     DevBuf gG, gW, gv, gtab, adjscratch;  // adjoint workspace
     DevBuf degen;                       // exclude_degenerate sums per (centre, z, bin)
     DevBuf degen_grad;                  // their gradient sums per (Z1, z, bin) in the adjoint
@@ -582,7 +594,7 @@ struct mp3pcf_ctx {
     // wide bins by angular sectors (moments_far.cu): tables, FP32 positions, centres in strip order
     FarTables far[kFarPlans];
     FarPlan fplan;  // of the last accumulate call
-    DevBuf bingeom, ftable, posf, fkey, fstart, ffill, forder;
+    DevBuf ftable, posf, fkey, fstart, ffill, forder;
     DevBuf fftwork;                     // FFT grid moments: padded fields, kernels, products
     FftPlanCache* fft = nullptr;        // cuFFT plans of the FFT grid moments
     DevBuf gridsum;                     // per-pixel FP64 sums of the grid-based approximation
@@ -746,25 +758,33 @@ mp3pcf_status mp3pcf_create(const mp3pcf_config* cfg, void* stream, mp3pcf_ctx**
     if (cudaGetDevice(&ctx->device) != cudaSuccess) return cleanup(MP3PCF_ECUDA);
     if (cudaDeviceGetAttribute(&ctx->n_sm, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess)
         return cleanup(MP3PCF_ECUDA);
-    const int nb = cfg->n_bins;
-    if (ctx->d_edges.ensure(sizeof(double) * (nb + 1)) != cudaSuccess ||
-        ctx->d_nodes.ensure(sizeof(double) * nb) != cudaSuccess ||
-        ctx->bingeom.ensure(sizeof(BinGeom) * nb) != cudaSuccess ||
-        ctx->edgelist.ensure(sizeof(int) * (1 + (size_t)cfg->n_z * cfg->n_z * cfg->n_z * nb * nb)) != cudaSuccess ||
-        ctx->bb.ensure(sizeof(int) * 10) != cudaSuccess || ctx->pairs.ensure(8 * (4 + kFarPlans)) != cudaSuccess ||
-        ctx->singular.ensure(8) != cudaSuccess)
-        return cleanup(MP3PCF_ENOMEM);
-    if (cudaMemcpy(ctx->d_edges.p, ctx->edges.data(), sizeof(double) * (nb + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(ctx->bingeom.p, bin_geometry(ctx->e2q).data(), sizeof(BinGeom) * nb, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(ctx->d_nodes.p, ctx->nodes.data(), sizeof(double) * nb, cudaMemcpyHostToDevice) != cudaSuccess)
-        return cleanup(MP3PCF_ECUDA);
-    if (!ctx->fp64) {
-        std::vector<float> v;
-        far_tables(cfg->n_max, ctx->far, &v);
-        if (ctx->ftable.ensure(sizeof(float) * v.size()) != cudaSuccess) return cleanup(MP3PCF_ENOMEM);
-        if (cudaMemcpy(ctx->ftable.p, v.data(), sizeof(float) * v.size(), cudaMemcpyHostToDevice) != cudaSuccess)
-            return cleanup(MP3PCF_ECUDA);
+    // one allocation and one copy: a program that makes a context per small field pays for them each time
+    const size_t nb = cfg->n_bins, z3 = (size_t)cfg->n_z * cfg->n_z * cfg->n_z;
+    const std::vector<BinGeom> geom = bin_geometry(ctx->e2q);
+    struct Part {
+        DevSlice* s;
+        const void* src;
+        size_t bytes, at;
+    } parts[] = {{&ctx->bingeom, geom.data(), sizeof(BinGeom) * nb, 0},
+                 {&ctx->d_edges, ctx->edges.data(), sizeof(double) * (nb + 1), 0},
+                 {&ctx->d_nodes, ctx->nodes.data(), sizeof(double) * nb, 0},
+                 {&ctx->bb, nullptr, sizeof(int) * 10, 0},
+                 {&ctx->pairs, nullptr, 8 * (4 + kFarPlans), 0},
+                 {&ctx->singular, nullptr, 8, 0},
+                 {&ctx->edgelist, nullptr, sizeof(int) * (1 + z3 * nb * nb), 0}};
+    size_t total = 0, copied = 0;
+    for (Part& q : parts) {
+        q.at = total;
+        total += (q.bytes + 255) / 256 * 256;
+        if (q.src) copied = total;
     }
+    if (ctx->fixed.ensure(total) != cudaSuccess) return cleanup(MP3PCF_ENOMEM);
+    std::vector<char> host(copied);
+    for (Part& q : parts) {
+        q.s->p = ctx->fixed.as<char>() + q.at;
+        if (q.src) memcpy(host.data() + q.at, q.src, q.bytes);
+    }
+    if (cudaMemcpy(ctx->fixed.p, host.data(), copied, cudaMemcpyHostToDevice) != cudaSuccess) return cleanup(MP3PCF_ECUDA);
     *out = ctx;
     return MP3PCF_OK;
 }
@@ -773,13 +793,13 @@ mp3pcf_status mp3pcf_destroy(mp3pcf_ctx* ctx)
 {
     if (!ctx) return MP3PCF_OK;
     cudaStreamSynchronize(ctx->st);
-    DevBuf* bufs[] = {&ctx->d_edges, &ctx->d_nodes, &ctx->bb, &ctx->key,
+    DevBuf* bufs[] = {&ctx->fixed, &ctx->key,
                       &ctx->count, &ctx->fill, &ctx->scan_sums, &ctx->scan_total, &ctx->perm,
                       &ctx->pos, &ctx->pay, &ctx->zs, &ctx->cflag,
                       &ctx->crank, &ctx->oflag, &ctx->orank, &ctx->centre_idx, &ctx->crow,
-                      &ctx->G, &ctx->W, &ctx->pairs, &ctx->partial, &ctx->singular,
-                      &ctx->edgelist, &ctx->m3partial, &ctx->m3filter, &ctx->m3four, &ctx->fftwork, &ctx->ccoef, &ctx->gG, &ctx->gW, &ctx->gv, &ctx->gtab,
-                      &ctx->adjscratch, &ctx->degen, &ctx->degen_grad, &ctx->zrange, &ctx->dkey, &ctx->dcell, &ctx->dperm, &ctx->dpos, &ctx->dgw, &ctx->dgrid, &ctx->bingeom, &ctx->ftable, &ctx->posf, &ctx->fkey, &ctx->fstart, &ctx->ffill, &ctx->forder, &ctx->gridsum, &ctx->gridflag, &ctx->bups, &ctx->bnorm,
+                      &ctx->G, &ctx->W, &ctx->partial,
+                      &ctx->m3partial, &ctx->m3filter, &ctx->m3four, &ctx->fftwork, &ctx->ccoef, &ctx->gG, &ctx->gW, &ctx->gv, &ctx->gtab,
+                      &ctx->adjscratch, &ctx->degen, &ctx->degen_grad, &ctx->zrange, &ctx->dkey, &ctx->dcell, &ctx->dperm, &ctx->dpos, &ctx->dgw, &ctx->dgrid, &ctx->ftable, &ctx->posf, &ctx->fkey, &ctx->fstart, &ctx->ffill, &ctx->forder, &ctx->gridsum, &ctx->gridflag, &ctx->bups, &ctx->bnorm,
                       &ctx->bgam, &ctx->bgcen, &ctx->berr, &ctx->pix, &ctx->pixinv};
     for (DevBuf* b : bufs) b->release();
     if (ctx->fft) fft_cache_destroy(ctx->fft);
@@ -834,6 +854,26 @@ static unsigned grid1d(int64_t n, int n_sm)
     const int64_t cap = (int64_t)n_sm * 16;
     if (g > cap) g = cap;
     return (unsigned)(g < 1 ? 1 : g);
+}
+
+// The sector form's tables, made when a plan first has sector bins (25 us at n_max 10, 78 at 50, an allocation
+// and a copy: as much as a small call, which never has any, takes in all). *ready: false inside a stream capture,
+// which may not allocate.
+static mp3pcf_status ensure_far_tables(mp3pcf_ctx* ctx, bool* ready)
+{
+    *ready = ctx->ftable.p != nullptr;
+    if (*ready) return MP3PCF_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    MP3_CK(cudaStreamIsCapturing(ctx->st, &cap));
+    if (cap != cudaStreamCaptureStatusNone) return MP3PCF_OK;
+    std::vector<float> v;
+    far_tables(ctx->cfg.n_max, ctx->far, &v);
+    MP3_CK(ctx->ftable.ensure(sizeof(float) * v.size()));
+    const cudaError_t e = cudaMemcpy(ctx->ftable.p, v.data(), sizeof(float) * v.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) ctx->ftable.release();
+    MP3_CK(e);
+    *ready = true;
+    return MP3PCF_OK;
 }
 
 // arguments of variant v for its bins (false: none); a: the whole range's, from bin b_lo
@@ -948,6 +988,7 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
     in.n_max = c.n_max;
     in.nz = nz;
     in.fp64 = ctx->fp64;
+    in.sectors = !ctx->fp64;
     in.occupancy = c.cell_occupancy;
     in.e2q = ctx->e2q.data();
     in.b_lo = b_lo;
@@ -957,7 +998,14 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
     in.extent = (double)(std::max(ex, ey) + 1);
     in.area = (double)(ex + 1) * (double)(ey + 1);
     in.carea = mask ? (double)((long long)hb[7] - hb[5] + 1) * (double)((long long)hb[8] - hb[6] + 1) : in.area;
-    const MomentsPlan plan = plan_moments(in);
+    MomentsPlan plan = plan_moments(in);
+    if (plan.far.b_far < b_hi) {
+        if (mp3pcf_status s = ensure_far_tables(ctx, &in.sectors)) {
+            stage_end(ctx, ST_SORT, t_sort);
+            return s;
+        }
+        if (!in.sectors) plan = plan_moments(in);
+    }
     const FarPlan& fp = plan.far;
     const int b_near = plan.b_near;
     ctx->fplan = fp;
@@ -1617,6 +1665,10 @@ mp3pcf_status mp3pcf_run_batch(mp3pcf_ctx* ctx, const mp3pcf_catalog_view* h_cat
         return s;
     };
     cudaError_t e;
+    if (!ctx->fp64) {  // before any capture
+        bool ready = false;
+        if (mp3pcf_status s = ensure_far_tables(ctx, &ready)) return restore(s);
+    }
     if ((e = ctx->bups.ensure(sizeof(double) * 2 * z3 * 4 * (c.n_max + 1) * nbb)) != cudaSuccess ||
         (e = ctx->bnorm.ensure(sizeof(double) * 2 * z3 * D * nbb)) != cudaSuccess ||
         (e = ctx->bgam.ensure(sizeof(double) * 2 * z3 * 4 * D * nbb)) != cudaSuccess ||

@@ -20,7 +20,7 @@ struct FarPlan {
 
 struct MomentsPlanInput {
     int n_max, nz;
-    bool fp64;
+    bool fp64, sectors;    // sectors: the sector form may be taken (FP32 only)
     int occupancy;         // configured galaxies per cell (0: automatic)
     const long long* e2q;  // all bins' squared edges
     int b_lo, b_hi;        // bins computed
@@ -67,7 +67,7 @@ inline FarPlan plan_far(const MomentsPlanInput& in, double least)
 {
     FarPlan f;
     f.b_far = in.b_hi;
-    if (in.fp64 || in.nc < 1 || in.n >= (1 << 27)) return f;  // 32-bit byte offsets into the sorted catalog
+    if (!in.sectors || in.nc < 1 || in.n >= (1 << 27)) return f;  // 32-bit byte offsets into the sorted catalog
     const double rho = (double)in.n / in.nz / in.area;  // galaxies per quantum^2 and z-bin
     const double occ = in.occupancy > 0 ? (double)in.occupancy : 1.0;
     f.side = std::max(least, sqrt(occ / rho));

@@ -24,6 +24,7 @@ int main(int argc, char** argv)
         in.n_max = rng() % (kMaxNmax + 1);
         in.nz = rng() % 3 ? 1 : 1 + rng() % kMaxNz;
         in.fp64 = rng() % 8 == 0;
+        in.sectors = !in.fp64 && rng() % 8;
         in.occupancy = rng() % 2 ? 0 : 1 + rng() % 64;
         const double ex = floor(logu(1.0, 16777215.0)), ey = rng() % 3 ? ex : floor(logu(1.0, 16777215.0));
         in.extent = std::max(ex, ey) + 1.0;
@@ -49,7 +50,7 @@ int main(int argc, char** argv)
         if (floor(in.extent / side) + 2.0 >= (1 << 22)) return printf("columns beyond near_int's range\n"), 1;
         if ((2.0 * sqrt((double)e2[f.b_far]) + 16.0) / side > kMaxRows - 4) return printf("more cell rows than listed\n"), 1;
         if (f.b_far == in.b_hi) continue;
-        if (in.fp64 || f.b[0] != in.b_hi || f.b[kFarPlans] != f.b_far) return printf("ranges of variants\n"), 1;
+        if (!in.sectors || f.b[0] != in.b_hi || f.b[kFarPlans] != f.b_far) return printf("ranges of variants\n"), 1;
         // a cell's half diagonal and the group's, as seen from the inner edge
         const double reach = side * (sqrt(0.5) + 0.5 * sqrt((double)f.rows * f.rows + (double)f.cols * f.cols));
         for (int v = 0; v < kFarPlans; ++v)
