@@ -27,6 +27,8 @@
 // and hence the result, reproducible run to run.
 #pragma once
 
+#include <type_traits>
+
 #include "moments_far.cuh"
 
 // Tiling parameters (compile-time; the defaults are the tuned values).
@@ -95,7 +97,10 @@ struct MomSmem {
     Pay<T> spay[P][SCR];      // staged candidate payloads
     int2 seg[2 * kMaxRows];   // (first sorted index, count) of the current bin's ranges
     int pre[2 * kMaxRows + 1];  // exclusive prefix sums of the range lengths
-    unsigned char found[P][SCR];  // staged candidates that are members
+    // staged candidates that are members
+    using Index = typename std::conditional<(SCR <= 256), unsigned char, unsigned short>::type;
+    static_assert(SCR <= 65536, "staged candidates are indexed by 16 bits at most");
+    Index found[P][SCR];
     int cnt[8];   // members in each warp's region this round
     int wtot[8];  // per-warp partial sums of the prefix scan
     int claim;    // the CTA's next centre from the work queue
@@ -358,7 +363,7 @@ __global__ void __launch_bounds__(MomPlan<T, NMAX>::NT, MomPlan<T, NMAX>::MINB) 
     const uint32_t aP = zp_base + (uint32_t)((P - 1) * CH * sizeof(cx<T>));
     const uint32_t aq = zp_base + (uint32_t)(zsel * CH * sizeof(cx<T>));
     float2* my_pos = s.spos[warp];
-    unsigned char* my_found = s.found[warp];
+    auto* my_found = s.found[warp];
     Pay<T>* my_pay = s.spay[warp];
     unsigned long long my_pairs = 0;
 
@@ -499,7 +504,7 @@ __global__ void __launch_bounds__(MomPlan<T, NMAX>::NT, MomPlan<T, NMAX>::MINB) 
                         }
                         in = in && ok;
                         const unsigned m = __ballot_sync(FULL, in);
-                        if (in) my_found[mycnt + __popc(m & lt_mask)] = (unsigned char)(u * 32 + lane);
+                        if (in) my_found[mycnt + __popc(m & lt_mask)] = u * 32 + lane;
                         mycnt += __popc(m);
                     }
                     __syncwarp();
