@@ -19,8 +19,7 @@ CASES = {
     "strip": dict(n=20011, side=150.0, lo=0.5, hi=70.0, bins=12, n_max=30, flat=True, variants=4),
     "coarse cells": dict(n=20011, side=60.0, lo=0.5, hi=40.0, bins=12, n_max=30, cell_occupancy=9, variants=2),
     "patch": dict(n=60011, side=120.0, lo=1.0, hi=50.0, bins=14, n_max=30, centres=True, variants=4),
-    "holes, degenerate triplets left out": dict(n=20011, side=60.0, lo=0.5, hi=40.0, bins=16, n_max=30, holes=True,
-                                                exclude_degenerate=True, variants=3),
+    "holes": dict(n=20011, side=60.0, lo=0.5, hi=40.0, bins=16, n_max=30, holes=True, variants=3),
 }
 
 
@@ -46,8 +45,7 @@ def test_gradient_of_every_galaxy(name):
     grad = {}
     for precision in ("fp64", "fp32"):
         with api.Estimator(c["bins"], c["lo"], c["hi"], c["n_max"], n_z=nz, precision=precision,
-                           cell_occupancy=c.get("cell_occupancy", 0),
-                           exclude_degenerate=c.get("exclude_degenerate", False)) as est:
+                           cell_occupancy=c.get("cell_occupancy", 0)) as est:
             est.accumulate_moments(*dev, centre_mask=mask)
             if precision == "fp64":
                 gu, gn = (torch.complex(*[torch.as_tensor(rng.normal(size=tuple(t.shape))) for _ in range(2)]).cuda()
