@@ -36,12 +36,6 @@ namespace mp3 {
 
 namespace adj {
 
-template <typename T>
-__device__ __forceinline__ cx<T> ld(const cx<T>* p, size_t i)
-{
-    return p[i];
-}
-
 __device__ __forceinline__ cx<double> ldd(const double* p, size_t i)
 {
     return cx<double>{p[2 * i], p[2 * i + 1]};
@@ -51,13 +45,6 @@ template <typename T>
 __device__ __forceinline__ cx<T> to_t(cx<double> v)
 {
     return cx<T>{(T)v.x, (T)v.y};
-}
-
-template <typename T>
-__device__ __forceinline__ void cfma(cx<T>& acc, cx<T> a, cx<T> b)
-{
-    acc.x += a.x * b.x - a.y * b.y;
-    acc.y += a.x * b.y + a.y * b.x;
 }
 
 // ------------------------------------------------------------------ stage (b): dL/dG, dL/dW

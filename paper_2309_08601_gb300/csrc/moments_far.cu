@@ -623,58 +623,58 @@ __global__ void __launch_bounds__(kThreads, 2) far_moments_kernel(const FarArgs 
                     s = __shfl_sync(FULL, nx, 0);
                 }
                 __syncthreads();
-                if constexpr (ADJ) continue;
+                if constexpr (!ADJ) {
+                    // ---- FFT over the sectors of every (term, centre)
+                    for (int q = tid; q < PT * kC; q += kThreads) {
+                        float x[S];
+    #pragma unroll
+                        for (int s = 0; s < S; ++s) x[s] = M[s * KS + q];
+                        real_fft<S>(x);
+    #pragma unroll
+                        for (int s = 0; s < S; ++s) M[s * KS + q] = x[s];
+                    }
+                    __syncthreads();
 
-                // ---- FFT over the sectors of every (term, centre)
-                for (int q = tid; q < PT * kC; q += kThreads) {
-                    float x[S];
-#pragma unroll
-                    for (int s = 0; s < S; ++s) x[s] = M[s * KS + q];
-                    real_fft<S>(x);
-#pragma unroll
-                    for (int s = 0; s < S; ++s) M[s * KS + q] = x[s];
-                }
-                __syncthreads();
-
-                // ---- the orders: thread (centre, m)
-                const int c8 = tid & (kC - 1);
-                if ((act >> c8) & 1u) {
-                    const size_t at = ((size_t)s_row[c8] * nz + z) * m.nbp + b;
-                    const int mtop = max(2 * n_max, n_max + 3);
-                    for (int mm = tid / kC; mm <= mtop; mm += kThreads / kC) {
-                        int k = mm & (S - 1);
-                        const bool cj = k > S / 2;
-                        if (cj) k = S - k;
-                        const float* Fr = M + k * KS + c8;
-                        const float* Fi = M + ((S - k) & (S - 1)) * KS + c8;
-                        const float fi = (k == 0 || k == S / 2) ? 0.f : (cj ? -1.f : 1.f);
-                        const float* cm = coef + mm * PW;
-                        const float2 ro = rot[mm];
-                        auto order = [&](int base, int P) {
-                            float er = 0.f, ei = 0.f, orr = 0.f, oi = 0.f;
-#pragma unroll 4
-                            for (int p = 0; p < P; p += 2) {
-                                const float ca = cm[p], cb = cm[p + 1];
-                                er = fmaf(ca, Fr[(base + p) * kC], er);
-                                ei = fmaf(ca, Fi[(base + p) * kC], ei);
-                                orr = fmaf(cb, Fr[(base + p + 1) * kC], orr);
-                                oi = fmaf(cb, Fi[(base + p + 1) * kC], oi);
+                    // ---- the orders: thread (centre, m)
+                    const int c8 = tid & (kC - 1);
+                    if ((act >> c8) & 1u) {
+                        const size_t at = ((size_t)s_row[c8] * nz + z) * m.nbp + b;
+                        const int mtop = max(2 * n_max, n_max + 3);
+                        for (int mm = tid / kC; mm <= mtop; mm += kThreads / kC) {
+                            int k = mm & (S - 1);
+                            const bool cj = k > S / 2;
+                            if (cj) k = S - k;
+                            const float* Fr = M + k * KS + c8;
+                            const float* Fi = M + ((S - k) & (S - 1)) * KS + c8;
+                            const float fi = (k == 0 || k == S / 2) ? 0.f : (cj ? -1.f : 1.f);
+                            const float* cm = coef + mm * PW;
+                            const float2 ro = rot[mm];
+                            auto order = [&](int base, int P) {
+                                float er = 0.f, ei = 0.f, orr = 0.f, oi = 0.f;
+    #pragma unroll 4
+                                for (int p = 0; p < P; p += 2) {
+                                    const float ca = cm[p], cb = cm[p + 1];
+                                    er = fmaf(ca, Fr[(base + p) * kC], er);
+                                    ei = fmaf(ca, Fi[(base + p) * kC], ei);
+                                    orr = fmaf(cb, Fr[(base + p + 1) * kC], orr);
+                                    oi = fmaf(cb, Fi[(base + p + 1) * kC], oi);
+                                }
+                                // even terms + i odd terms, then the half-sector rotation
+                                const float vr = er - fi * oi, vi = fi * ei + orr;
+                                return cx<float>{vr * ro.x - vi * ro.y, vr * ro.y + vi * ro.x};
+                            };
+                            if (mm <= 2 * n_max) m.W[(size_t)mm * plane + at] = order(0, PW);
+                            if (mm <= n_max + 3) {
+                                const cx<float> a = order(PW, PAB), bb = order(PW + PAB, PAB);
+                                if (mm <= n_max - 1)
+                                    m.G[(size_t)(mm + n_max + 3) * plane + at] = cx<float>{a.x - bb.y, a.y + bb.x};
+                                if (mm >= 1)
+                                    m.G[(size_t)(n_max + 3 - mm) * plane + at] = cx<float>{a.x + bb.y, bb.x - a.y};
                             }
-                            // even terms + i odd terms, then the half-sector rotation
-                            const float vr = er - fi * oi, vi = fi * ei + orr;
-                            return cx<float>{vr * ro.x - vi * ro.y, vr * ro.y + vi * ro.x};
-                        };
-                        if (mm <= 2 * n_max) m.W[(size_t)mm * plane + at] = order(0, PW);
-                        if (mm <= n_max + 3) {
-                            const cx<float> a = order(PW, PAB), bb = order(PW + PAB, PAB);
-                            if (mm <= n_max - 1)
-                                m.G[(size_t)(mm + n_max + 3) * plane + at] = cx<float>{a.x - bb.y, a.y + bb.x};
-                            if (mm >= 1)
-                                m.G[(size_t)(n_max + 3 - mm) * plane + at] = cx<float>{a.x + bb.y, bb.x - a.y};
                         }
                     }
+                    __syncthreads();
                 }
-                __syncthreads();
             }
         }
         if (tid == 0) s_item = (int)min(atomicAdd(A.queue, 1ull) + gridDim.x, (unsigned long long)nitems);
