@@ -397,7 +397,7 @@ __device__ void block_sort(int* v, int n)
 // thread (a few entries in a field of even density), a fuller one by the block: a distant outlier or
 // a steep cluster can put the whole catalog into one cell, where insertion takes n^2 / 4 dependent steps
 // (200 000 entries: 10^10). The direct estimator of 200 000 galaxies, 900 apertures x 3 triples, with one
-// galaxy at the far end of the fixed-point range takes 34 ms with the network (even field: 1.9).
+// galaxy at the far end of the fixed-point range takes 33 ms with the network (even field: 1.9).
 constexpr int kLightCell = 64;
 
 __global__ void __launch_bounds__(256) k_cell_order(int64_t K, const int* __restrict__ start, int* perm)
@@ -599,7 +599,7 @@ struct mp3pcf_ctx {
     FftPlanCache* fft = nullptr;        // cuFFT plans of the FFT grid moments
     DevBuf gridsum;                     // per-pixel FP64 sums of the grid-based approximation
     DevBuf gridflag;                    // its non-empty flags and their exclusive scan
-    DevBuf dkey, dcell, dperm, dpos, dgw, dgrid;  // cell-sorted copy of the direct estimator's catalog
+    DevBuf dkey, dcell, dperm, dpos, dgw, dgrid, dagain;  // cell-sorted copy of the direct estimator's catalog
     // combined estimator: the moments of the last accumulate call mix discrete and grid bins
     bool combined = false;
     long long bbox[4] = {0, 0, 0, 0};   // extent (x0, y0, x1, y1) of the last accumulate call
@@ -799,7 +799,7 @@ mp3pcf_status mp3pcf_destroy(mp3pcf_ctx* ctx)
                       &ctx->crank, &ctx->oflag, &ctx->orank, &ctx->centre_idx, &ctx->crow,
                       &ctx->G, &ctx->W, &ctx->partial,
                       &ctx->m3partial, &ctx->m3filter, &ctx->m3four, &ctx->fftwork, &ctx->ccoef, &ctx->gG, &ctx->gW, &ctx->gv, &ctx->gtab,
-                      &ctx->adjscratch, &ctx->degen, &ctx->degen_grad, &ctx->zrange, &ctx->dkey, &ctx->dcell, &ctx->dperm, &ctx->dpos, &ctx->dgw, &ctx->dgrid, &ctx->ftable, &ctx->posf, &ctx->fkey, &ctx->fstart, &ctx->ffill, &ctx->forder, &ctx->gridsum, &ctx->gridflag, &ctx->bups, &ctx->bnorm,
+                      &ctx->adjscratch, &ctx->degen, &ctx->degen_grad, &ctx->zrange, &ctx->dkey, &ctx->dcell, &ctx->dperm, &ctx->dpos, &ctx->dgw, &ctx->dgrid, &ctx->dagain, &ctx->ftable, &ctx->posf, &ctx->fkey, &ctx->fstart, &ctx->ffill, &ctx->forder, &ctx->gridsum, &ctx->gridflag, &ctx->bups, &ctx->bnorm,
                       &ctx->bgam, &ctx->bgcen, &ctx->berr, &ctx->pix, &ctx->pixinv};
     for (DevBuf* b : bufs) b->release();
     if (ctx->fft) fft_cache_destroy(ctx->fft);
@@ -1527,6 +1527,7 @@ mp3pcf_status mp3pcf_map3_direct(mp3pcf_ctx* ctx, int64_t n, const int32_t* d_xq
         MP3_CK(ctx->dpos.ensure(sizeof(int2) * n));
         MP3_CK(ctx->dgw.ensure(sizeof(float4) * n));
         MP3_CK(ctx->dgrid.ensure(sizeof(GridDesc)));
+        MP3_CK(ctx->dagain.ensure((size_t)n_centres * n_ap));
         int* start = ctx->dcell.as<int>();
         int* fill = start + K + 1;
         GridDesc* g = ctx->dgrid.as<GridDesc>();
@@ -1544,8 +1545,9 @@ mp3pcf_status mp3pcf_map3_direct(mp3pcf_ctx* ctx, int64_t n, const int32_t* d_xq
         k_gather_raw<<<gr, 256, 0, st>>>(n, ctx->dperm.as<int>(), d_xq, d_yq, d_g1, d_g2, d_w, ctx->dpos.as<int2>(),
                                          ctx->dgw.as<float4>());
         MP3_CK(cudaGetLastError());
-        MP3_CK(launch_map3_direct_cells(ctx->dpos.as<int2>(), ctx->dgw.as<float4>(), start, g, ctx->cfg.quantum, n_centres,
-                                        d_centres, (int)n_ap, d_theta_ap, rcut_factor, d_out, st));
+        MP3_CK(launch_map3_direct_cells(n, ctx->dpos.as<int2>(), ctx->dgw.as<float4>(), start, g, ctx->cfg.quantum, n_centres,
+                                        d_centres, (int)n_ap, d_theta_ap, rcut_factor, d_out, ctx->dagain.as<uint8_t>(), ctx->n_sm,
+                                        st));
         return MP3PCF_OK;
     }
     MP3_CK(launch_map3_direct(n, d_xq, d_yq, d_g1, d_g2, d_w, ctx->cfg.quantum, n_centres, d_centres, (int)n_ap,

@@ -186,10 +186,11 @@ cudaError_t grid_fft_moments(FftPlanCache* cache, int64_t nc, int nz, int nb, in
 cudaError_t launch_map3_direct(int64_t n, const int32_t* xq, const int32_t* yq, const float* g1, const float* g2,
                                const float* w, double quantum, int64_t n_cen, const double* centres, int n_ap,
                                const double* theta, double rcut_factor, double* out, cudaStream_t st);
-// the same from a cell-sorted copy: pos, (gamma_1, gamma_2, w, -), cell offsets and the grid (device)
-cudaError_t launch_map3_direct_cells(const int2* pos, const float4* gw, const int* start, const GridDesc* grid,
+// the same from a cell-sorted copy: pos, (gamma_1, gamma_2, w, -), cell offsets and the grid (device); again
+// [n_cen * n_ap]: scratch
+cudaError_t launch_map3_direct_cells(int64_t n, const int2* pos, const float4* gw, const int* start, const GridDesc* grid,
                                      double quantum, int64_t n_cen, const double* centres, int n_ap, const double* theta,
-                                     double rcut_factor, double* out, cudaStream_t st);
+                                     double rcut_factor, double* out, uint8_t* again, int n_sm, cudaStream_t st);
 cudaError_t launch_to_map3(const PostArgs& p, const double* gcen, int n_ap, const double* theta,
                            double* partial, int chunks, double* corr, double* m8,
                            cudaStream_t st);

@@ -13,6 +13,8 @@
 // over the galaxies, FP64 sums reduced over the block.
 #include <math.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace mp3 {
@@ -94,11 +96,11 @@ __global__ void __launch_bounds__(kDirThreads) map3_direct_kernel(int64_t n, con
 // galaxies. Bound by FP64 arithmetic on the galaxies inside (two FP64 lanes per SM and cycle), so a
 // radius that occurs twice in a triple is evaluated once, and equal radii need three powers of one
 // factor. 200 000 galaxies, 900 apertures x 3 triples: 67.5 ms by scanning the catalog, 2.7 ms by cells.
-// A row with more than kDirLong galaxies in the circle (a strip, an outlier that makes the cells huge, a
-// cluster) is left to the whole block, which would else wait for the one warp that has it. Uneven fields of
-// 200 000 galaxies, by scanning and by cells: an outlier 50 and 34 ms, a strip 79 and 12, a cluster 23 and 7.5.
-constexpr int kDirLong = 1024;
-
+// A row with more than `limit` galaxies in the circle (a strip, an outlier that makes the cells huge, a cluster) is
+// left out by this kernel, as the block would wait for the one warp that has it; the aperture is noted and
+// map3_direct_long_kernel does it again with such rows taken by the whole block. Uneven fields of 200 000 galaxies,
+// by scanning and by cells: an outlier 50 and 33 ms, a strip 79 and 13, a cluster 23 and 12. (With both
+// loops in one kernel the even field took 1 to 2 % longer.)
 template <int R>  // distinct radii of the triple: 1 (all equal), 2 (the first two equal) or 3
 __device__ __forceinline__ void direct_sums(double (&s)[14], const double (&b)[3], double gt)
 {
@@ -127,8 +129,9 @@ __device__ __forceinline__ void direct_sums(double (&s)[14], const double (&b)[3
     }
 }
 
-template <int R>
-__device__ __forceinline__ void direct_cells(double (&s)[14], const int2* __restrict__ pos,
+// BLOCK: long rows by the block, else not at all; returns whether the calling warp has left one out
+template <int R, bool BLOCK>
+__device__ __forceinline__ bool direct_cells(double (&s)[14], int limit, const int2* __restrict__ pos,
                                              const float4* __restrict__ gw, const int* __restrict__ start,
                                              const GridDesc& g, double quantum, double cx, double cy, double rcut,
                                              double r2max, const double (&inv2)[3], const double (&nrm)[3])
@@ -138,64 +141,50 @@ __device__ __forceinline__ void direct_cells(double (&s)[14], const int2* __rest
     const double is = 1.0 / (double)g.side, xc = (cx / quantum - (double)g.x0) * is, yc = (cy / quantum - (double)g.y0) * is;
     const double rc = (rcut / quantum + 2.0) * is * (1.0 + 1e-9);
     const int iy0 = (int)fmin(fmax(floor(yc - rc), 0.0), (double)g.ncy), iy1 = (int)fmax(fmin(floor(yc + rc), (double)g.ncy - 1.0), -1.0);
-    // the run [k0, k1) of row iy
-    auto run = [&](int iy, int& k0, int& k1) {
-        k0 = k1 = 0;
-        const double dy = fmax(fmax((double)iy - yc, yc - (double)iy - 1.0), 0.0);
-        const double hx = sqrt(fmax(rc * rc - dy * dy, 0.0)) + 1e-6 * rc;
-        const int ix0 = (int)fmin(fmax(floor(xc - hx), 0.0), (double)g.ncx), ix1 = (int)fmax(fmin(floor(xc + hx), (double)g.ncx - 1.0), -1.0);
-        if (ix0 > ix1) return;
-        k0 = start[iy * g.ncx + ix0];
-        k1 = start[iy * g.ncx + ix1 + 1];
-    };
-    auto add = [&](int k0, int k1, int first, int step) {
-        for (int k = k0 + first; k < k1; k += step) {
-            const int2 p = pos[k];
-            const double dx = (double)p.x * quantum - cx, dyk = (double)p.y * quantum - cy;
-            const double r2 = dx * dx + dyk * dyk;
-            if (r2 == 0.0 || r2 > r2max) continue;
-            const float4 v = gw[k];
-            const double gt = -((double)v.x * (dx * dx - dyk * dyk) + 2.0 * (double)v.y * dx * dyk) / r2;
-            const double wr = (double)v.z * r2;
-            double b[3];
-#pragma unroll
-            for (int l = 0; l < R; ++l) {
-                const int i = R == 2 && l == 1 ? 2 : l;
-                b[l] = wr * nrm[i] * exp(-r2 * inv2[i]);
-            }
-            direct_sums<R>(s, b, gt);
-        }
-    };
     bool later = false;
-    for (int iy = iy0 + warp; iy <= iy1; iy += kDirThreads / 32) {
-        int k0, k1;
-        run(iy, k0, k1);
-        if (k1 - k0 > kDirLong)
-            later = true;
-        else
-            add(k0, k1, lane, 32);
-    }
-    if (!__syncthreads_or(later)) return;
-    for (int r0 = iy0; r0 <= iy1; r0 += 32) {
-        int k0 = 0, k1 = 0;
-        if (r0 + lane <= iy1) run(r0 + lane, k0, k1);
-        for (unsigned m = __ballot_sync(0xffffffffu, k1 - k0 > kDirLong); m; m &= m - 1) {
-            const int l = __ffs(m) - 1;
-            add(__shfl_sync(0xffffffffu, k0, l), __shfl_sync(0xffffffffu, k1, l), threadIdx.x, kDirThreads);
+#pragma unroll 1
+    for (int pass = 0; pass < (BLOCK ? 2 : 1); ++pass) {
+        const int first = pass ? (int)threadIdx.x : lane, step = pass ? kDirThreads : 32;
+        for (int iy = iy0 + (pass ? 0 : warp); iy <= iy1; iy += pass ? 1 : kDirThreads / 32) {
+            const double dy = fmax(fmax((double)iy - yc, yc - (double)iy - 1.0), 0.0);
+            const double hx = sqrt(fmax(rc * rc - dy * dy, 0.0)) + 1e-6 * rc;
+            const int ix0 = (int)fmin(fmax(floor(xc - hx), 0.0), (double)g.ncx), ix1 = (int)fmax(fmin(floor(xc + hx), (double)g.ncx - 1.0), -1.0);
+            if (ix0 > ix1) continue;
+            const int k0 = start[iy * g.ncx + ix0], k1 = start[iy * g.ncx + ix1 + 1];
+            if ((k1 - k0 > limit) != (pass == 1)) {
+                later = true;
+                continue;
+            }
+            for (int k = k0 + first; k < k1; k += step) {
+                const int2 p = pos[k];
+                const double dx = (double)p.x * quantum - cx, dyk = (double)p.y * quantum - cy;
+                const double r2 = dx * dx + dyk * dyk;
+                if (r2 == 0.0 || r2 > r2max) continue;
+                const float4 v = gw[k];
+                const double gt = -((double)v.x * (dx * dx - dyk * dyk) + 2.0 * (double)v.y * dx * dyk) / r2;
+                const double wr = (double)v.z * r2;
+                double b[3];
+#pragma unroll
+                for (int l = 0; l < R; ++l) {
+                    const int i = R == 2 && l == 1 ? 2 : l;
+                    b[l] = wr * nrm[i] * exp(-r2 * inv2[i]);
+                }
+                direct_sums<R>(s, b, gt);
+            }
         }
     }
+    return !BLOCK && later;
 }
 
-__global__ void __launch_bounds__(kDirThreads) map3_direct_cells_kernel(const int2* __restrict__ pos,
-                                                                        const float4* __restrict__ gw,
-                                                                        const int* __restrict__ start,
-                                                                        const GridDesc* __restrict__ grid, double quantum,
-                                                                        int n_ap, const double* __restrict__ centres,
-                                                                        const double* __restrict__ theta,
-                                                                        double rcut_factor, double* __restrict__ out)
+// one (aperture, radii triple) by the block; returns whether a row was left out
+template <bool BLOCK>
+__device__ __forceinline__ bool direct_aperture(int64_t job, int limit, const int2* __restrict__ pos,
+                                                const float4* __restrict__ gw, const int* __restrict__ start,
+                                                const GridDesc* __restrict__ grid, double quantum, int n_ap,
+                                                const double* __restrict__ centres, const double* __restrict__ theta,
+                                                double rcut_factor, double* __restrict__ out)
 {
     __shared__ double red[14][kDirThreads / 32];
-    const int64_t job = blockIdx.x;
     const int64_t t = job / n_ap;
     const int a = (int)(job % n_ap);
     double th[3], inv2[3], nrm[3];
@@ -231,21 +220,22 @@ __global__ void __launch_bounds__(kDirThreads) map3_direct_cells_kernel(const in
     for (int v = 0; v < 14; ++v) s[v] = 0.0;
     const GridDesc g = *grid;
     const double cx = centres[2 * t], cy = centres[2 * t + 1];
+    bool later;
     const bool e01 = th[0] == th[1], e12 = th[1] == th[2];
     if (e01 && e12) {
-        direct_cells<1>(s, pos, gw, start, g, quantum, cx, cy, rcut, r2max, inv2, nrm);
+        later = direct_cells<1, BLOCK>(s, limit, pos, gw, start, g, quantum, cx, cy, rcut, r2max, inv2, nrm);
         s[1] = s[2] = s[0];
         s[4] = s[5] = s[3];
         s[8] = s[9] = s[7];
         s[11] = s[12] = s[10];
     } else if (e01) {
-        direct_cells<2>(s, pos, gw, start, g, quantum, cx, cy, rcut, r2max, inv2, nrm);
+        later = direct_cells<2, BLOCK>(s, limit, pos, gw, start, g, quantum, cx, cy, rcut, r2max, inv2, nrm);
         s[1] = s[0];
         s[5] = s[4];
         s[8] = s[7];
         s[12] = s[11];
     } else {
-        direct_cells<3>(s, pos, gw, start, g, quantum, cx, cy, rcut, r2max, inv2, nrm);
+        later = direct_cells<3, BLOCK>(s, limit, pos, gw, start, g, quantum, cx, cy, rcut, r2max, inv2, nrm);
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -254,7 +244,7 @@ __global__ void __launch_bounds__(kDirThreads) map3_direct_cells_kernel(const in
         for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
         if (lane == 0) red[v][warp] = x;
     }
-    __syncthreads();
+    later = __syncthreads_or(later) != 0;
     if (threadIdx.x == 0) {
         double q[14];
         for (int v = 0; v < 14; ++v) {
@@ -264,14 +254,55 @@ __global__ void __launch_bounds__(kDirThreads) map3_direct_cells_kernel(const in
         out[2 * job] = q[0] * q[1] * q[2] - q[3] * q[2] - q[4] * q[1] - q[5] * q[0] + 2.0 * q[6];
         out[2 * job + 1] = q[7] * q[8] * q[9] - q[10] * q[9] - q[11] * q[8] - q[12] * q[7] + 2.0 * q[13];
     }
+    return later;
 }
 
-cudaError_t launch_map3_direct_cells(const int2* pos, const float4* gw, const int* start, const GridDesc* grid,
-                                     double quantum, int64_t n_cen, const double* centres, int n_ap, const double* theta,
-                                     double rcut_factor, double* out, cudaStream_t st)
+__global__ void __launch_bounds__(kDirThreads) map3_direct_cells_kernel(const int2* __restrict__ pos,
+                                                                        const float4* __restrict__ gw,
+                                                                        const int* __restrict__ start,
+                                                                        const GridDesc* __restrict__ grid, double quantum,
+                                                                        int limit, int n_ap,
+                                                                        const double* __restrict__ centres,
+                                                                        const double* __restrict__ theta,
+                                                                        double rcut_factor, double* __restrict__ out,
+                                                                        uint8_t* __restrict__ again)
 {
-    map3_direct_cells_kernel<<<(unsigned)(n_cen * n_ap), kDirThreads, 0, st>>>(pos, gw, start, grid, quantum, n_ap, centres,
-                                                                               theta, rcut_factor, out);
+    const int64_t job = blockIdx.x;
+    const bool later = direct_aperture<false>(job, limit, pos, gw, start, grid, quantum, n_ap, centres, theta, rcut_factor, out);
+    if (threadIdx.x == 0) again[job] = later;
+}
+
+__global__ void __launch_bounds__(kDirThreads) map3_direct_long_kernel(int64_t jobs, const int2* __restrict__ pos,
+                                                                       const float4* __restrict__ gw,
+                                                                       const int* __restrict__ start,
+                                                                       const GridDesc* __restrict__ grid, double quantum,
+                                                                       int limit, int n_ap,
+                                                                       const double* __restrict__ centres,
+                                                                       const double* __restrict__ theta,
+                                                                       double rcut_factor, double* __restrict__ out,
+                                                                       const uint8_t* __restrict__ again)
+{
+    for (int64_t job = blockIdx.x; job < jobs; job += gridDim.x) {
+        if (!again[job]) continue;
+        direct_aperture<true>(job, limit, pos, gw, start, grid, quantum, n_ap, centres, theta, rcut_factor, out);
+        __syncthreads();  // the reduction's buffer
+    }
+}
+
+cudaError_t launch_map3_direct_cells(int64_t n, const int2* pos, const float4* gw, const int* start, const GridDesc* grid,
+                                     double quantum, int64_t n_cen, const double* centres, int n_ap, const double* theta,
+                                     double rcut_factor, double* out, uint8_t* again, int n_sm, cudaStream_t st)
+{
+    // long: a row by a warp takes as long as the scan of an eighth of the catalog by the block; 128 steps of a
+    // warp are not worth the second kernel
+    const int limit = (int)std::min<int64_t>(4096, std::max<int64_t>(256, n / 8));
+    const int64_t jobs = n_cen * n_ap;
+    map3_direct_cells_kernel<<<(unsigned)jobs, kDirThreads, 0, st>>>(pos, gw, start, grid, quantum, limit, n_ap, centres, theta,
+                                                                     rcut_factor, out, again);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    map3_direct_long_kernel<<<(unsigned)std::min<int64_t>(jobs, 2 * n_sm), kDirThreads, 0, st>>>(
+        jobs, pos, gw, start, grid, quantum, limit, n_ap, centres, theta, rcut_factor, out, again);
     return cudaGetLastError();
 }
 
