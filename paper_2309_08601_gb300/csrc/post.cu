@@ -232,9 +232,12 @@ __device__ __forceinline__ bool toeplitz_solve4(const cx<double>* t, const cx<do
             p = csub(p, ae);
             ip = crecip(p);
             const double aa = al.x * al.x + al.y * al.y, bb = be.x * be.x + be.y * be.y;
-            const float refl = sqrtf((float)fmax(aa, bb));
+            // the larger by the high words (none is negative; the FP64 comparisons would take the pipe that bounds this),
+            // rounded up; a NaN's is above 1's
+            const unsigned big = max((unsigned)__double2hiint(aa), (unsigned)__double2hiint(bb));
+            const float refl = sqrtf((float)__hiloint2double((int)big, -1));
             growth *= (1.f + refl) / (1.f - refl);
-            good = good && aa < 1.0 && bb < 1.0 && growth < kToeplitzGrowth;  // false for NaN
+            good = good && big < 0x3ff00000u && growth < kToeplitzGrowth;
             const cx<double> na{-al.x, -al.y}, nbt{-be.x, -be.y};
             cx<double> d[4], w[R];
 #pragma unroll
