@@ -58,6 +58,10 @@ TRAFFIC_BYTES = {
     # (profiles/contract_tc_bf16x3_traffic_50k.md)
     ("contract", "masked_lognormal_1m"): 20 * (1.981240576e9 + 35.888640e6),
     ("contract", "lognormal_200k"): 4 * (993.852928e6 + 19.601408e6),
+    # the stage's five moment kernels: captures at 100 000 and 50 000 galaxies of each density, x10 and x4
+    # (profiles/moments_kernels_50k_100k.md)
+    ("moments", "masked_lognormal_1m"): 10 * (5.431272e9 + 9.957754e9),
+    ("moments", "lognormal_200k"): 4 * (1.411256e9 + 2.327457e9),
 }
 TRAFFIC_NOTE = "ncu dram__bytes_read.sum + dram__bytes_write.sum per launch (profiles/)"
 

@@ -6,8 +6,8 @@
 //   e^{i m phi} = e^{i m phi_s} sum_p i^{p mod 2} c_{m,p} T_p(u),  u = sin(delta) / sin(delta_max),
 // T_p the Chebyshev polynomials and c_{m,p} the (real) expansion coefficients of cos and sin of
 // m asin(sin(delta_max) u). A pair then only adds w T_p, w gamma_1 T_p (p < PAB) and w gamma_2 T_p to
-// its sector's sums M_{s,p} (about 25 packed FMAs at n_max = 30), and per (centre, bin) a real FFT over the sectors and a
-// short sum over p give every order:
+// its sector's sums M_{s,p} (30 packed FMAs in the variant for the widest bins, 54 for the nearest), and per (centre,
+// bin) a real FFT over the sectors and a short sum over p give every order:
 //   W_m = e^{i pi m / S} sum_p i^{p mod 2} c_{m,p} F_{m,p},  F_{m,p} = sum_s M_{s,p} e^{2 pi i m s / S}.
 // delta_max follows from n_max, PW and PAB so that the dropped terms stay below 3e-8 (far_dmax), so
 // the result differs from the direct form's by FP32 rounding only.
@@ -19,8 +19,8 @@
 //
 // Measured with the narrow bins in moments_near.cu, moments of the whole call: 200 000 galaxies, 20
 // bins to 120', n_max 30: 314 -> 84 ms; 10 000 centres of 400 000 galaxies, 30 bins to 240',
-// n_max 40: 98.5 -> 19 ms. The candidate loop is 80 % of it, bound by issue (64 %) and the FMA and
-// ALU pipes (50 % each); the loads of the next candidates come from L2.
+// n_max 40: 98.5 -> 19 ms. The candidate loop is 80 % of it, bound by issue (53 to 63 % of the slots with 16
+// warps an SM) and latency; FMA pipe 47 to 58 %, ALU pipe 25 to 44 %; the next candidates' loads come from L2.
 #include <math.h>
 
 #include <algorithm>
