@@ -141,8 +141,9 @@ mp3pcf_status mp3pcf_copy_moments(mp3pcf_ctx* ctx, void* d_G, void* d_W);
 mp3pcf_status mp3pcf_contract_multipoles(mp3pcf_ctx* ctx, double* d_upsilon, double* d_norm);
 
 /* Edge correction, Eqs. ModeCoupling and GammaMultipolesWithEC, Sec. 3.4: per (zt, b1, b2)
- * solves sum_n N_{l-n} Gamma_{mu,n} = Upsilon_{mu,l}, l, n in [-n_max, n_max], in FP64 with
- * partial pivoting. Negative orders come from the symmetries of App. A
+ * solves sum_n N_{l-n} Gamma_{mu,n} = Upsilon_{mu,l}, l, n in [-n_max, n_max], in FP64: by the
+ * Levinson recursion where the couplings keep its error at elimination's, else by elimination
+ * with partial pivoting. Negative orders come from the symmetries of App. A
  * (Upsilon_{0,-n}(i,j) = Upsilon_{0,n}(j,i), Upsilon_{1,-n}(i,j) = Upsilon_{1,n}(j,i),
  * Upsilon_{2,-n}(i,j) = Upsilon_{3,n}(j,i), N_{-n}(i,j) = N_n(j,i), with Z2 <-> Z3).
  * Output d_gamma_n [n_z^3][4][2 n_max+1][n_bins][n_bins] complex double, n = -n_max..n_max;

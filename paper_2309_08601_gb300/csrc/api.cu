@@ -857,22 +857,16 @@ static unsigned grid1d(int64_t n, int n_sm)
 }
 
 // The sector form's tables, made when a plan first has sector bins (25 us at n_max 10, 78 at 50, an allocation
-// and a copy: as much as a small call, which never has any, takes in all). *ready: false inside a stream capture,
-// which may not allocate.
-static mp3pcf_status ensure_far_tables(mp3pcf_ctx* ctx, bool* ready)
+// and a copy: as much as a small call, which never has any, takes in all).
+static mp3pcf_status make_far_tables(mp3pcf_ctx* ctx)
 {
-    *ready = ctx->ftable.p != nullptr;
-    if (*ready) return MP3PCF_OK;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    MP3_CK(cudaStreamIsCapturing(ctx->st, &cap));
-    if (cap != cudaStreamCaptureStatusNone) return MP3PCF_OK;
+    if (ctx->ftable.p) return MP3PCF_OK;
     std::vector<float> v;
     far_tables(ctx->cfg.n_max, ctx->far, &v);
     MP3_CK(ctx->ftable.ensure(sizeof(float) * v.size()));
-    const cudaError_t e = cudaMemcpy(ctx->ftable.p, v.data(), sizeof(float) * v.size(), cudaMemcpyHostToDevice);
+    const cudaError_t e = cudaMemcpyAsync(ctx->ftable.p, v.data(), sizeof(float) * v.size(), cudaMemcpyHostToDevice, ctx->st);
     if (e != cudaSuccess) ctx->ftable.release();
     MP3_CK(e);
-    *ready = true;
     return MP3PCF_OK;
 }
 
@@ -999,12 +993,17 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
     in.area = (double)(ex + 1) * (double)(ey + 1);
     in.carea = mask ? (double)((long long)hb[7] - hb[5] + 1) * (double)((long long)hb[8] - hb[6] + 1) : in.area;
     MomentsPlan plan = plan_moments(in);
-    if (plan.far.b_far < b_hi) {
-        if (mp3pcf_status s = ensure_far_tables(ctx, &in.sectors)) {
-            stage_end(ctx, ST_SORT, t_sort);
-            return s;
+    const bool make_tables = plan.far.b_far < b_hi && !ctx->ftable.p;
+    if (make_tables) {
+        // a stream capture may not allocate: without the tables the other forms take all bins
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        const cudaError_t e = cudaStreamIsCapturing(st, &cap);
+        if (e != cudaSuccess) stage_end(ctx, ST_SORT, t_sort);
+        MP3_CK(e);
+        if (cap != cudaStreamCaptureStatusNone) {
+            in.sectors = false;
+            plan = plan_moments(in);
         }
-        if (!in.sectors) plan = plan_moments(in);
     }
     const FarPlan& fp = plan.far;
     const int b_near = plan.b_near;
@@ -1095,11 +1094,16 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
     a.queue = ctx->pairs.as<unsigned long long>() + 2;
     if (b_lo >= b_hi) return MP3PCF_OK;
     StageScope sc(ctx, ST_MOMENTS);
-    if (fp.b_far < b_hi) {
+    const MomentArgs<T> all = a;
+    auto sectors = [&]() {
         if constexpr (sizeof(T) == 4) {
-            if (mp3pcf_status s = run_far(ctx, a, fp, b_lo, b_hi)) return s;
+            if (fp.b_far < b_hi) return run_far(ctx, all, fp, b_lo, b_hi);
         }
-    }
+        return MP3PCF_OK;
+    };
+    // tables to be made first: the other forms' kernels run meanwhile
+    if (!make_tables)
+        if (mp3pcf_status s = sectors()) return s;
     if (b_near > b_lo) {
         NearArgs<T> na;
         na.m = a;
@@ -1120,6 +1124,10 @@ static mp3pcf_status accumulate_t(mp3pcf_ctx* ctx, int64_t n, const int32_t* xq,
         else
             e = launch_moments_f32(a, ctx->n_sm, st);
         MP3_CK(e);
+    }
+    if (make_tables && fp.b_far < b_hi) {
+        if (mp3pcf_status s = make_far_tables(ctx)) return s;
+        return sectors();
     }
     return MP3PCF_OK;
 }
@@ -1668,8 +1676,7 @@ mp3pcf_status mp3pcf_run_batch(mp3pcf_ctx* ctx, const mp3pcf_catalog_view* h_cat
     };
     cudaError_t e;
     if (!ctx->fp64) {  // before any capture
-        bool ready = false;
-        if (mp3pcf_status s = ensure_far_tables(ctx, &ready)) return restore(s);
+        if (mp3pcf_status s = make_far_tables(ctx)) return restore(s);
     }
     if ((e = ctx->bups.ensure(sizeof(double) * 2 * z3 * 4 * (c.n_max + 1) * nbb)) != cudaSuccess ||
         (e = ctx->bnorm.ensure(sizeof(double) * 2 * z3 * D * nbb)) != cudaSuccess ||
